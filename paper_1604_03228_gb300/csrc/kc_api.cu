@@ -645,6 +645,7 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
         // CTAs' lower bounds too
         uint64_t *slots = cv.take<uint64_t>(res_grid ? (size_t)keff * grid * res_sw
                                                       : (size_t)slot_words(keff, grid, lp != 0));
+        uint64_t *bc = cv.take<uint64_t>((size_t)bc_words(d));
         int *tail = use_tail ? cv.take<int>((size_t)keff) : nullptr;
         unsigned *flag_words = c.o.dtype == KC_F32 ? cv.take<unsigned>(2) : nullptr;   // flagged count, done
         *zero_bytes = cv.off;
@@ -662,6 +663,7 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
         gon_single(g, pk, c.o.dtype, n, d, keff, first, mind, slots, *cen_dev, *kout_dev,
                    (uint64_t *)key32, range2, grid);
         g.single.tail = tail;
+        g.single.bc = bc;
         if (lp) {
             attach_lp(g.single, LB, lp, cenT, keff, ecmax);
             g.lp_kind = lp;
@@ -1000,7 +1002,7 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
     struct L {
         int32_t *range2;
         unsigned long long *key32, *max64, *arg64;
-        uint64_t *slots1, *slots2, *fk2;
+        uint64_t *slots1, *slots2, *fk2, *bc1, *bc2;
         int64_t *nU;
         int *counter;
         void *staging, *pk, *pkU, *cen;
@@ -1027,6 +1029,8 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
         Lo.counter = cv.take<int>(1);
         Lo.slots1 = cv.take<uint64_t>((size_t)std::max<int64_t>(1, slot_off[m]));
         Lo.slots2 = cv.take<uint64_t>((size_t)slot_words(k, G2, false));
+        Lo.bc1 = cv.take<uint64_t>((size_t)bc_words(d) * m);
+        Lo.bc2 = cv.take<uint64_t>((size_t)bc_words(d));
         Lo.zero_bytes = cv.off;
         Lo.staging = (dev_pts || pin_pts) ? nullptr : cv.take<char>((size_t)n * d * esz);
         Lo.pk = cv.take<char>((size_t)nb * BLK * d * esz);
@@ -1076,6 +1080,7 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
             I.pk = Lo.pk;
             I.mind = Lo.mind;
             I.slots = Lo.slots1 + slot_off[i];
+            I.bc = Lo.bc1 + bc_words(d) * i;
             I.centers = Lo.c1 + (int64_t)i * k;
             I.k_out = Lo.k1 + i;
             I.final_key = Lo.fk1 + i;
@@ -1100,6 +1105,7 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
     proto.pk = Lo.pkU;
     proto.mind = Lo.mindU;
     proto.slots = Lo.slots2;
+    proto.bc = Lo.bc2;
     proto.centers = Lo.cen_dev;
     proto.k_out = Lo.kout_dev;
     proto.final_key = Lo.fk2;
@@ -1344,7 +1350,7 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         int32_t *range2;
         unsigned long long *key32, *max64, *arg64;
         uint32_t *thr, *v;
-        uint64_t *fk, *slots;
+        uint64_t *fk, *slots, *bc;
         uint8_t *mask;
         PruneBufs pb;
         void *staging, *pk, *Sc, *Hc, *pkC, *cen;
@@ -1370,6 +1376,7 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         Lo.v = cv.take<uint32_t>(1);
         Lo.fk = cv.take<uint64_t>(1);
         Lo.slots = cv.take<uint64_t>((size_t)slot_words(keff_max, grid, lp != 0));
+        Lo.bc = cv.take<uint64_t>((size_t)bc_words(d));
         Lo.mask = cv.take<uint8_t>((size_t)n);
         Lo.zero_bytes = cv.off;
         Lo.staging = dev_pts ? nullptr : cv.take<char>((size_t)n * d * esz);
@@ -1532,6 +1539,7 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         gon_single(g, Lo.pkC, c.o.dtype, nC, d, kC, 0, Lo.mindC, Lo.slots, Lo.cen_dev, Lo.kout_dev, Lo.fk,
                    Lo.range2, std::min(grid, choose_gon_grid(c.o.dtype, d, nC, lp)));
         g.single.map = Lo.C;
+        g.single.bc = Lo.bc;
         if (lp) {
             attach_lp(g.single, LB, lp, cenT, kC, ecmax);
             g.lp_kind = lp;
@@ -1707,7 +1715,7 @@ struct BatchBufs {
         uint32_t *lpw;
         float *ept, *eblk, *cenT, *ecmax;
         uint32_t *m32, *stamp;
-        uint64_t *slots;
+        uint64_t *slots, *bc;
     };
     std::vector<Per> per;
     int *counter = nullptr;
@@ -1738,6 +1746,7 @@ void batch_layout(Carve &cv, const BatchShape &b, BatchBufs &B, const int64_t *n
     for (int q = 0; q < b.nheavy; ++q) {
         const int i = b.order[q];
         B.per[i].slots = cv.take<uint64_t>((size_t)slot_words(std::min<int64_t>(k[i], n[i]), b.G[q], b.lp != 0));
+        B.per[i].bc = cv.take<uint64_t>((size_t)bc_words(d[i]));
     }
     B.zero_bytes = cv.off;
     B.kout_dev = dev_kout ? k_out : cv.take<int32_t>((size_t)count);
@@ -1806,6 +1815,7 @@ std::vector<char> batch_descriptors(const BatchShape &b, BatchBufs &B, const voi
         I.pk = P.pk;
         I.mind = P.mind;
         I.slots = q < b.nheavy ? P.slots : nullptr;
+        I.bc = q < b.nheavy ? P.bc : nullptr;
         I.centers = P.cen;
         I.k_out = B.kout_dev + i;
         I.final_key = B.fkeys + i;

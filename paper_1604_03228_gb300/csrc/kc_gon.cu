@@ -18,7 +18,9 @@
 //   3. warp 0 publishes the CTA's key in its slot for this step, polls the
 //      group's slots of this step (relaxed loads, all of a lane's slots in
 //      flight at once, bounded by a cycle budget), reduces them to the group
-//      key, and loads the winner's coordinates for the next step;
+//      key, and loads the winner's coordinates for the next step; in large
+//      groups only the first CTA does so, and passes key and coordinates on
+//      (kc_gon.cuh);
 //   4. one more barrier hands the key and the new center to the CTA.
 // Slots are per step and zeroed before the launch, so a non-zero slot always
 // belongs to the current step; the key itself is the payload, so relaxed
@@ -30,7 +32,7 @@
 #include <cstdlib>
 #include <type_traits>
 
-#include "kc_internal.cuh"
+#include "kc_gon.cuh"
 
 namespace kc {
 
@@ -64,87 +66,6 @@ __device__ __forceinline__ void pc_publish(const long long *c) {
 }
 
 namespace {
-
-constexpr int GROUP_NT = 1024;   // group mode: one CTA per SM
-constexpr int QUEUE_NT = 256;    // queue mode: several CTAs per SM
-
-template <typename T> struct Vec4;
-template <> struct Vec4<float> { using type = float4; };
-template <> struct Vec4<int32_t> { using type = int4; };
-
-__device__ __forceinline__ uint64_t ld_relaxed_u64(const uint64_t *p) {
-    uint64_t v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_relaxed_u64(uint64_t *p, uint64_t v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-template <typename T, int DC>
-__device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T *cs, int lane,
-                                      typename AccOf<T>::type acc[4]) {
-    using V4 = typename Vec4<T>::type;
-    using A = typename AccOf<T>::type;
-    const V4 *src = reinterpret_cast<const V4 *>(blk) + lane;
-    A a0 = A(0), a1 = A(0), a2 = A(0), a3 = A(0);
-    if constexpr (DC > 0) {
-#pragma unroll
-        for (int j = 0; j < DC; ++j) {
-            const V4 v = __ldg(src + j * (BLK / 4));
-            const T c = cs[j];
-            a0 = sq_step(a0, v.x, c);
-            a1 = sq_step(a1, v.y, c);
-            a2 = sq_step(a2, v.z, c);
-            a3 = sq_step(a3, v.w, c);
-        }
-    } else {
-#pragma unroll 4
-        for (int j = 0; j < d; ++j) {
-            const V4 v = __ldg(src + j * (BLK / 4));
-            const T c = cs[j];
-            a0 = sq_step(a0, v.x, c);
-            a1 = sq_step(a1, v.y, c);
-            a2 = sq_step(a2, v.z, c);
-            a3 = sq_step(a3, v.w, c);
-        }
-    }
-    acc[0] = a0;
-    acc[1] = a1;
-    acc[2] = a2;
-    acc[3] = a3;
-}
-
-// The blocks of CTA r (of G, W warps each) over [b0, b1] are
-// b(i) = b0 + r W + i % W + (i / W) G W for i = 0, 1, ... (increasing in i).
-// Within a step the CTA's warps take i from a counter in shared memory (ctr;
-// the next index is claimed while the current block is processed), so a warp
-// whose loads came back sooner takes more blocks and the CTA's share is done
-// when its blocks are, not when its slowest warp's fixed list is.  A block's
-// minima stay with the CTA, which orders every step's accesses with its
-// barriers.  ctr null: the fixed assignment i = warp + j W.
-__device__ __forceinline__ int64_t cta_block(int64_t b0, int r, int G, int W, int i) {
-    return b0 + (int64_t)r * W + (i % W) + (int64_t)(i / W) * G * W;
-}
-__device__ __forceinline__ int claim_block(int *ctr, int lane) {
-    int v = 0;
-    if (lane == 0) v = atomicAdd(ctr, 1);
-    return __shfl_sync(0xFFFFFFFFu, v, 0);
-}
-
-// First block of the group's shared tail: with a tail counter, the CTAs own
-// the blocks below it (7/8 of the range, whole rounds of G W blocks) and any
-// warp of the group claims the rest, two blocks at a time, from a per-step
-// counter in global memory, so the group's step ends when its blocks are done
-// rather than when the CTA that got the least bandwidth is.  Blocks of the
-// tail change CTA from step to step: their minima are read past L1 and every
-// step's writes are fenced before the step's slot is published (gon_solve).
-__device__ __forceinline__ int64_t tail_start(int64_t b0, int64_t b1, int G, int W, bool tail) {
-    if (!tail) return b1 + 1;
-    const int64_t GW = (int64_t)G * W;
-    const int64_t rounds = (b1 - b0 + 1) * 7 / 8 / GW;
-    return rounds >= 2 ? b0 + rounds * GW : b1 + 1;
-}
 
 // One step's sweep of this CTA's share (rank r of G) of [lo, lo + n).
 template <typename T, int DC, int NT>
@@ -228,44 +149,6 @@ __device__ __forceinline__ uint64_t sweep(const T *__restrict__ pk, uint32_t *__
     return best;
 }
 
-// Warp 0: wait for all G slots of this step and return their maximum.
-__device__ uint64_t poll_slots(const uint64_t *slots, int G, long long timeout, DevStatus *st,
-                               int step, bool *abort_out) {
-    const int lane = threadIdx.x & 31;
-    uint64_t g = 0;
-    bool ab = false;
-    for (int s0 = 0; s0 < G && !ab; s0 += 128) {
-        uint64_t v[4];
-        unsigned pend = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (s0 + q * 32 + lane < G) pend |= 1u << q;
-        const long long t0 = clock64();
-        while (pend) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (pend >> q & 1u) v[q] = ld_relaxed_u64(slots + s0 + q * 32 + lane);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if ((pend >> q & 1u) && v[q] != 0) {
-                    g = umax64(g, v[q]);
-                    pend &= ~(1u << q);
-                }
-            if (pend && (clock64() - t0 > timeout || ld_volatile_i32(&st->code) != 0)) {
-                set_status(st, KC_ERR_TIMEOUT, 3, step);
-                ab = true;
-                break;
-            }
-        }
-    }
-    *abort_out = __any_sync(0xFFFFFFFFu, ab);
-    return warp_max_u64(g);
-}
-
-__device__ __forceinline__ int64_t out_index(const GonInst &I, int64_t local) {
-    return I.map ? I.map[local] : I.base + local;
-}
-
 struct Shared {
     uint64_t red[32];
     uint64_t key;
@@ -283,21 +166,28 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int d = DC > 0 ? DC : I.d;
     const T *pk = (const T *)I.pk;
+    int64_t first = I.first;
+    if (I.it0 > 0) {   // continue behind an earlier launch, from its last winner
+        const uint64_t K0 = __ldcg(I.final_key);
+        if (key_val(K0) == 0) return;   // which stopped early
+        first = key_idx(K0);
+        if (!KC_IN_RANGE(st, first, I.n, KC_AT_CENTER_LOAD)) return;
+    }
     if (warp == 0) {
-        for (int j = lane; j < d; j += 32) cs[j] = pk[pk_index(I.lo + I.first, j, d)];
+        for (int j = lane; j < d; j += 32) cs[j] = pk[pk_index(I.lo + first, j, d)];
         if (lane == 0) {
             sh.abort = 0;
             sh.ctr[0] = sh.ctr[1] = 0;
         }
     }
-    if (r == 0 && tid == 0) I.centers[0] = out_index(I, I.first);
+    if (r == 0 && tid == 0) I.centers[I.it0] = out_index(I, first);
     __syncthreads();
     const bool claim = DYN && NT == GROUP_NT && (I.lo + I.n - 1) / BLK - I.lo / BLK + 1 >= 4 * (int64_t)G * W;
     const bool tail = DYN && G > 1 && I.tail != nullptr;
 
     int it;
     uint64_t K = 0;
-    for (it = 0; it < I.k; ++it) {
+    for (it = I.it0; it < I.it1; ++it) {
         // claimed blocks in the 1024-thread group CTAs when every warp has
         // several (measured: GON on 8M x 64, k = 1024, 313 -> 308 ms); the
         // fixed assignment in the 256-thread queue CTAs (MRG round 1 on
@@ -313,19 +203,34 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
             v = warp_max_u64(v);
             uint64_t g = v;
             bool ab = false;
+            const bool more = it + 1 < I.it1;
+            // (queue CTAs share their SM with other groups; there the leader
+            // gained nothing and the sweep's code grew: MRG round 1 on 10M x 16
+            // 20.2 -> 20.7 ms)
+            const bool lead = NT == GROUP_NT && G > LEADER_MIN && I.bc != nullptr;
+            const uint64_t tagw = (uint64_t)(it + 1) << 32;
             if (G > 1) {
-                const int64_t row = (int64_t)it * slot_stride(G);
+                uint64_t *row = I.slots + (int64_t)it * slot_stride(G);
                 const bool held = withhold == it + 1 && r == G - 1;
                 // with a shared tail, the step's minima (written by this
                 // CTA's threads before the barrier) are made visible to the
                 // group before the slot is, and the other CTAs' after it is
                 // seen (the release / acquire pattern of a grid barrier)
                 if (tail) __threadfence();
-                if (lane == 0 && !held) st_relaxed_u64(&I.slots[row + r], v ? v : 1);
-                g = poll_slots(I.slots + row, G, timeout, st, it, &ab);
+                if (lane == 0 && !held && !(lead && r == 0)) st_relaxed_u64(row + r, v ? v : 1);
+                if (!lead || r == 0) {
+                    g = lead ? poll_slots<1>(row, G, timeout, st, it, &ab, v) : poll_slots(row, G, timeout, st, it, &ab);
+                } else {
+                    uint32_t kw = 0;
+                    ab = follow_leader(I.bc, (uint32_t)it + 1, more ? d + 2 : 2, timeout, st, it, [&](int w, uint32_t b) {
+                        if (w < 2) kw = b;
+                        else cs[w - 2] = *reinterpret_cast<const T *>(&b);
+                    });
+                    g = ((uint64_t)__shfl_sync(0xFFFFFFFFu, kw, 0) << 32) | __shfl_sync(0xFFFFFFFFu, kw, 1);
+                }
                 if (tail) __threadfence();
             }
-            if (!ab && key_val(g) != 0 && it + 1 < I.k) {
+            if (!ab && more && (!lead || r == 0)) {
 #ifdef KC_CHECKS
                 // testing hook of the checked build: a winner index one past
                 // the instance, which the check below must catch
@@ -333,13 +238,18 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
 #else
                 const int64_t c = key_idx(g);
 #endif
-                if (KC_IN_RANGE(st, c, I.n, KC_AT_CENTER_LOAD)) {
-                    for (int j = lane; j < d; j += 32) cs[j] = pk[pk_index(I.lo + c, j, d)];
-                    if (r == 0 && lane == 0) I.centers[it + 1] = out_index(I, c);
+                if (key_val(g) == 0 || KC_IN_RANGE(st, c, I.n, KC_AT_CENTER_LOAD)) {
+                    for (int j = lane; j < d; j += 32) {
+                        const T x = key_val(g) != 0 ? pk[pk_index(I.lo + c, j, d)] : T(0);
+                        cs[j] = x;
+                        if (lead) st_relaxed_u64(I.bc + 2 + j, tagw | *reinterpret_cast<const uint32_t *>(&x));
+                    }
+                    if (r == 0 && lane == 0 && key_val(g) != 0) I.centers[it + 1] = out_index(I, c);
                 } else {
                     ab = true;
                 }
             }
+            if (lead && r == 0 && !ab && lane < 2) st_relaxed_u64(I.bc + lane, tagw | (lane == 0 ? g >> 32 : g & 0xFFFFFFFFu));
             if (lane == 0) {
                 sh.key = g;
                 sh.abort = ab;
@@ -643,23 +553,32 @@ __device__ void gon_solve_lp(const GonInst &I, int r, int G, float *smem, ShLP &
     // counter, as the FP32 sweep does, measured slower here: 183 -> 188 ms
     // per solve on 8M x 64, k = 1024)
     const int64_t b0 = lo / BLK;
+    int64_t first = I.first;
+    float ec0 = 0.f;
+    if (I.it0 > 0) {   // continue behind an earlier launch, from its last winner
+        const uint64_t K0 = __ldcg(I.final_key);
+        if (key_val(K0) == 0) return;   // which stopped early
+        first = key_idx(K0);
+        if (!KC_IN_RANGE(st, first, I.n, KC_AT_CENTER_LOAD)) return;
+        ec0 = __ldcg(I.ecmax_out);
+    }
     if (warp == 0) {
         float ec;
-        lp_load_center<KIND>(I, I.first, d, ng, cl, scs, 0, lane, &ec);
+        lp_load_center<KIND>(I, first, d, ng, cl, scs, I.it0, lane, &ec);
         if (lane == 0) {
-            sh.ecmax = ec;
+            sh.ecmax = fmaxf(ec, ec0);
             sh.abort = 0;
             sh.Lcta = 0u;
         }
     }
-    if (r == 0 && tid == 0) I.centers[0] = out_index(I, I.first);
+    if (r == 0 && tid == 0) I.centers[I.it0] = out_index(I, first);
     __syncthreads();
 
     int it;
     uint64_t K = 0;
     if (clk && tid == 0) pc_start(sh.pc);
     volatile unsigned *Lcta = &sh.Lcta;
-    for (it = 0; it < I.k; ++it) {
+    for (it = I.it0; it < I.it1; ++it) {
         const float ecmax = sh.ecmax;
         float Lrun = -INFINITY;
         int cnt = 0;
@@ -875,7 +794,7 @@ __device__ void gon_solve_lp(const GonInst &I, int r, int G, float *smem, ShLP &
                 g = poll_slots(I.slots + row, G, timeout, st, it, &ab);
             }
             if (lane == 0) sh.Lcta = 0u;   // next step's admission bound starts over
-            if (!ab && key_val(g) != 0 && it + 1 < I.k) {
+            if (!ab && key_val(g) != 0 && it + 1 < I.it1) {
                 const int64_t c = key_idx(g);
                 if (KC_IN_RANGE(st, c, I.n, KC_AT_CENTER_LOAD) && KC_IN_RANGE(st, it + 1, I.kcap, KC_AT_CENTER_COPY)) {
                     float ec;
@@ -909,42 +828,17 @@ __device__ void gon_solve_lp(const GonInst &I, int r, int G, float *smem, ShLP &
     }
 }
 
-template <typename T>
-__device__ bool instance_ok(const GonInst &I, DevStatus *st) {
-    if constexpr (std::is_same<T, int32_t>::value) {
-        if (!int_range_ok(I.range2, I.d)) {
-            set_status(st, KC_ERR_RANGE, 2, 0);
-            return false;
-        }
-    }
-    return true;
-}
-
-// Last instance of insts[0, m) whose CTA group starts at or before this CTA.
-__device__ __forceinline__ void find_group(const GonInst *insts, int m, GonInst &I) {
-    int lo = 0, hi = m - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (insts[mid].cta0 <= (int)blockIdx.x) lo = mid;
-        else hi = mid - 1;
-    }
-    I = insts[lo];
-}
-
 template <typename T, int DC, bool DYN>
 __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_kernel(GonArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *cs = reinterpret_cast<T *>(smem_raw);
     __shared__ GonInst I;
     __shared__ Shared sh;
-    if (threadIdx.x == 0) {
-        if (a.insts) find_group(a.insts, a.ninst, I);
-        else I = a.single;
-    }
-    __syncthreads();
+    copy_instance(I, a.insts ? find_group(a.insts, a.ninst) : &a.single);
     const int r = (int)blockIdx.x - I.cta0;
     if (r < 0 || r >= I.G) return;
     if (ld_volatile_i32(&a.st->code) != 0) return;
+    if (a.route && ld_volatile_i32(a.route) != 0) return;   // the skip kernel runs the rest
     if (!instance_ok<T>(I, a.st)) return;
     gon_solve<T, DC, GROUP_NT, DYN>(I, r, I.G, cs, sh, a.st, a.timeout_cycles, a.withhold, a.bad_index != 0);
 }
@@ -961,29 +855,21 @@ __global__ void __launch_bounds__(QUEUE_NT) gon_queue_kernel(GonArgs a) {
     __shared__ Shared sh;
     __shared__ int s_i;
     if ((int)blockIdx.x < a.gheavy) {
-        if (threadIdx.x == 0) find_group(a.insts, a.nheavy, I);
-        __syncthreads();
+        copy_instance(I, find_group(a.insts, a.nheavy));
         const int r = (int)blockIdx.x - I.cta0;
         if (r >= 0 && r < I.G && ld_volatile_i32(&a.st->code) == 0 && instance_ok<T>(I, a.st))
             gon_solve<T, DC, QUEUE_NT>(I, r, I.G, cs, sh, a.st, a.timeout_cycles);
         __syncthreads();
     }
     for (;;) {
-        if (threadIdx.x == 0) {
-            s_i = a.nheavy + atomicAdd(a.counter, 1);
-            if (s_i < a.ninst) I = a.insts[s_i];
-        }
+        if (threadIdx.x == 0) s_i = a.nheavy + atomicAdd(a.counter, 1);
         __syncthreads();
         if (s_i >= a.ninst) return;
+        copy_instance(I, a.insts + s_i);
         if (ld_volatile_i32(&a.st->code) != 0) return;
         if (instance_ok<T>(I, a.st)) gon_solve<T, DC, QUEUE_NT>(I, 0, 1, cs, sh, a.st, a.timeout_cycles);
         __syncthreads();
     }
-}
-
-__device__ __forceinline__ void find_instance(const GonArgs &a, GonInst &I) {
-    if (a.insts) find_group(a.insts, a.ninst, I);
-    else I = a.single;
 }
 
 template <int KIND, int DC>
@@ -991,11 +877,11 @@ __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_lp_kernel(GonArgs a) {
     extern __shared__ __align__(16) float smem_f[];
     __shared__ GonInst I;
     __shared__ ShLP sh;
-    if (threadIdx.x == 0) find_instance(a, I);
-    __syncthreads();
+    copy_instance(I, a.insts ? find_group(a.insts, a.ninst) : &a.single);
     const int r = (int)blockIdx.x - I.cta0;
     if (r < 0 || r >= I.G) return;
     if (ld_volatile_i32(&a.st->code) != 0) return;
+    if (a.route && ld_volatile_i32(a.route) != 0) return;   // the skip kernel runs the rest
     gon_solve_lp<KIND, DC, GROUP_NT>(I, r, I.G, smem_f, sh, a.st, a.timeout_cycles, a.withhold, a.lp_local_t != 0);
 }
 
@@ -1006,20 +892,17 @@ __global__ void __launch_bounds__(QUEUE_NT, 4) gon_queue_lp_kernel(GonArgs a) {
     __shared__ ShLP sh;
     __shared__ int s_i;
     if ((int)blockIdx.x < a.gheavy) {
-        if (threadIdx.x == 0) find_group(a.insts, a.nheavy, I);
-        __syncthreads();
+        copy_instance(I, find_group(a.insts, a.nheavy));
         const int r = (int)blockIdx.x - I.cta0;
         if (r >= 0 && r < I.G && ld_volatile_i32(&a.st->code) == 0)
             gon_solve_lp<KIND, DC, QUEUE_NT>(I, r, I.G, smem_f, sh, a.st, a.timeout_cycles, 0, a.lp_local_t != 0);
         __syncthreads();
     }
     for (;;) {
-        if (threadIdx.x == 0) {
-            s_i = a.nheavy + atomicAdd(a.counter, 1);
-            if (s_i < a.ninst) I = a.insts[s_i];
-        }
+        if (threadIdx.x == 0) s_i = a.nheavy + atomicAdd(a.counter, 1);
         __syncthreads();
         if (s_i >= a.ninst) return;
+        copy_instance(I, a.insts + s_i);
         if (ld_volatile_i32(&a.st->code) != 0) return;
         gon_solve_lp<KIND, DC, QUEUE_NT>(I, 0, 1, smem_f, sh, a.st, a.timeout_cycles);
         __syncthreads();
@@ -1074,6 +957,65 @@ __device__ __forceinline__ void res_check(T v, bool &bad, bool &nonfin, uint32_t
         lo = max(lo, 0xFFFFFFFFu - bv);
         hi = max(hi, bv);
     }
+}
+
+// Wait for a word whose high half is tag.
+__device__ __forceinline__ uint64_t poll_word(const uint64_t *p, uint32_t tag, long long timeout, DevStatus *st, int step,
+                                              bool *ab) {
+    uint64_t w = ld_relaxed_u64(p);
+    if ((uint32_t)(w >> 32) == tag) return w;
+    const long long t0 = clock64();
+    for (int n = 1;; ++n) {
+        w = ld_relaxed_u64(p);
+        if ((uint32_t)(w >> 32) == tag) return w;
+        if ((n & 31) == 0 && (clock64() - t0 > timeout || ld_volatile_i32(&st->code) != 0)) {
+            set_status(st, KC_ERR_TIMEOUT, 3, step);
+            *ab = true;
+            return 0;
+        }
+    }
+}
+
+// Warp 0: the largest key of a step's G slots (SW words each) and the slot
+// that holds it.
+template <int SW>
+__device__ __forceinline__ uint64_t poll_keys(const uint64_t *row, int G, long long timeout, DevStatus *st, int step,
+                                              int *win, bool *abort_out) {
+    const int lane = threadIdx.x & 31;
+    uint64_t kv[5] = {0, 0, 0, 0, 0};
+    unsigned pend = 0;
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+        if (lane + 32 * q < G) pend |= 1u << q;
+    bool ab = false;
+    const long long t0 = clock64();
+    int n = 0;
+    while (pend) {
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+            if (pend >> q & 1u) kv[q] = ld_relaxed_u64(row + (int64_t)(lane + 32 * q) * SW);
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+            if ((pend >> q & 1u) && kv[q] != 0) pend &= ~(1u << q);
+        if (pend && (++n & 31) == 0 && (clock64() - t0 > timeout || ld_volatile_i32(&st->code) != 0)) {
+            set_status(st, KC_ERR_TIMEOUT, 3, step);
+            ab = true;
+            break;
+        }
+    }
+    *abort_out = __any_sync(0xFFFFFFFFu, ab);
+    uint64_t lk = 0;
+    int ls = 0;
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+        if (kv[q] > lk) {
+            lk = kv[q];
+            ls = lane + 32 * q;
+        }
+    const uint64_t gg = warp_max_u64(lk);
+    const unsigned wl = __ballot_sync(0xFFFFFFFFu, gg != 0 && lk == gg);
+    *win = __shfl_sync(0xFFFFFFFFu, ls, wl ? __ffs(wl) - 1 : 0);
+    return gg;
 }
 
 template <typename T, int DC>
@@ -1175,60 +1117,22 @@ __global__ void __launch_bounds__(GROUP_NT, 1) gon_resident_kernel(GonArgs a) {
             const int wsrc = ow ? __ffs(ow) - 1 : 0;
             if (G > 1) {
                 // publish the CTA's candidate: coordinates (tagged) and key
-                uint64_t *mine = I.slots + ((int64_t)it * G + r) * SW;
+                uint64_t *row = I.slots + (int64_t)it * G * SW, *mine = row + (int64_t)r * SW;
                 if (!(a.withhold == it + 1 && r == G - 1)) {
                     if (lane < DC) st_relaxed_u64(mine + 1 + lane, (1ull << 32) | sh.cand[wsrc][lane]);
                     if (lane == 0) st_relaxed_u64(mine, g ? g : 1);
                 }
-                // poll the keys of the step's slots (lane: slots lane + 32 q)
-                const uint64_t *row = I.slots + (int64_t)it * G * SW;
-                uint64_t kv[5] = {0, 0, 0, 0, 0};
-                unsigned pend = 0;
-#pragma unroll
-                for (int q = 0; q < 5; ++q)
-                    if (lane + 32 * q < G) pend |= 1u << q;
+                // the keys of the step's slots, then the winner's coordinates
+                // from its slot (each tag set once written); a leader that
+                // passes them on was slower here (1M points: 4.9 us a step
+                // against 3.6), the coordinates being in the slots already
+                int win = 0;
                 bool ab = false;
-                const long long t0 = clock64();
-                while (pend) {
-#pragma unroll
-                    for (int q = 0; q < 5; ++q)
-                        if (pend >> q & 1u) kv[q] = ld_relaxed_u64(row + (int64_t)(lane + 32 * q) * SW);
-#pragma unroll
-                    for (int q = 0; q < 5; ++q)
-                        if ((pend >> q & 1u) && kv[q] != 0) pend &= ~(1u << q);
-                    if (pend && (clock64() - t0 > a.timeout_cycles || ld_volatile_i32(&a.st->code) != 0)) {
-                        set_status(a.st, KC_ERR_TIMEOUT, 3, it);
-                        ab = true;
-                        break;
-                    }
-                }
-                ab = __any_sync(0xFFFFFFFFu, ab);
-                uint64_t lk = 0;
-                int ls = 0;
-#pragma unroll
-                for (int q = 0; q < 5; ++q)
-                    if (kv[q] > lk) {
-                        lk = kv[q];
-                        ls = lane + 32 * q;
-                    }
-                const uint64_t gg = warp_max_u64(lk);
-                const unsigned wl = __ballot_sync(0xFFFFFFFFu, gg != 0 && lk == gg);
-                const int win = __shfl_sync(0xFFFFFFFFu, ls, wl ? __ffs(wl) - 1 : 0);
-                // the winner's coordinates from its slot (each tag set once written)
+                const uint64_t gg = poll_keys<SW>(row, G, a.timeout_cycles, a.st, it, &win, &ab);
                 if (!ab && !KC_IN_RANGE(a.st, win, G, KC_AT_SLOT)) ab = true;
-                if (!ab && lane < DC) {
-                    const uint64_t *wp = row + (int64_t)win * SW + 1 + lane;
-                    uint64_t w = ld_relaxed_u64(wp);
-                    while ((w >> 32) == 0) {
-                        if (clock64() - t0 > a.timeout_cycles || ld_volatile_i32(&a.st->code) != 0) {
-                            set_status(a.st, KC_ERR_TIMEOUT, 3, it);
-                            ab = true;
-                            break;
-                        }
-                        w = ld_relaxed_u64(wp);
-                    }
-                    sh.pc[0][lane] = (uint32_t)w;
-                }
+                if (!ab && lane < DC)
+                    sh.pc[0][lane] =
+                        (uint32_t)poll_word(row + (int64_t)win * SW + 1 + lane, 1u, a.timeout_cycles, a.st, it, &ab);
                 ab = __any_sync(0xFFFFFFFFu, ab);
                 if (lane == 0) {
                     sh.pkey[0] = gg;

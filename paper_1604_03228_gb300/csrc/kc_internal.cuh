@@ -97,9 +97,11 @@ __device__ __forceinline__ uint32_t key_val(uint64_t k) { return (uint32_t)(k >>
 __device__ __forceinline__ uint64_t umax64(uint64_t a, uint64_t b) { return a > b ? a : b; }
 
 __device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v = umax64(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    return v;
+    // two warp reductions of 32 bits: the high words, then the low words of
+    // the lanes that hold the largest
+    const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(v >> 32));
+    const uint32_t lo = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
+    return ((uint64_t)hi << 32) | lo;
 }
 
 __device__ __forceinline__ uint64_t ld_acquire_u64(const uint64_t *p) {
@@ -221,6 +223,7 @@ struct GonInst {
     const float *rm;
     uint32_t *mind;          // [nblocks(n) * BLK] running minimum (value bits)
     uint64_t *slots;         // [k * G] per-step, per-CTA argmax keys (zeroed)
+    uint64_t *bc;            // [bc_words(d)] the leader's words of a step (zeroed), or nullptr: every CTA polls the slots
     int64_t *centers;        // [k] out
     int32_t *k_out;          // out
     uint64_t *final_key;     // out: key of the largest final minimum
@@ -242,6 +245,21 @@ struct GonInst {
     // low-precision pack), so a recheck evaluates only the newer centers
     uint32_t *m32;
     uint32_t *stamp;
+    // skip kernel (kc_gonskip.cu): per point of the packed array the center
+    // (its position in the selection) that gave the running minimum, and the
+    // row of rm that holds local point i (nullptr: row i); cenT as above
+    uint16_t *asg;
+    const int64_t *rmap;
+    // its regrouped states (two in turn), skip_positions(n) entries each (asg
+    // and pk have as many): the point of a position, minima, assignments (the
+    // second state's in asg); the regrouping's bin counts
+    uint32_t *skip_perm[2], *skip_mind[2];
+    uint16_t *skip_asg;
+    unsigned *skip_hist;
+    // this launch runs steps [it0, it1) of the k (it1 = 0: to the end); from
+    // it0 > 0 on, the state of the steps before it is in place and the first
+    // center is the one *final_key names
+    int32_t it0, it1;
     int32_t lp_kind;
     int32_t kcap;
     int64_t lo;              // first point of the range in the packed array
@@ -287,8 +305,27 @@ struct GonArgs {
     // resident form (single instance, gon_resident_kernel): points per
     // coordinate held in each CTA's shared memory; 0 = the streaming kernels
     int res_cap;
+    // single instances that may change over to the skip kernel: a device word,
+    // 0 while the streaming kernels run, else the step at which it took over
+    // (streaming launches then return at once); nullptr: never
+    int *route;
+    int skip_units;          // skip kernel: units of 32 points a CTA has room for
+    float skip_g2, skip_f;   // its slack factors for this d (kc_gonskip.cu)
 };
 cudaError_t launch_gon(GonArgs &a, cudaStream_t s);
+// Single large float instances with row-major rows in device memory: the
+// ends of the streaming segments after which a probe decides whether the rest
+// of the k steps leaves out evaluations by the triangle inequality (0: never
+// for these sizes).  launch_gon_probe follows the segment that ended at it0
+// (words: zeroed); launch_gon_skip runs the steps from *route
+// on, if any (last: the largest step it can be).
+int64_t skip_positions(int64_t n);   // positions of the regrouped arrays, at most
+int64_t skip_hist_words(int G);
+int64_t skip_route_words();          // the route word, the probe's counter and its sample
+int64_t skip_slot_rows();            // slot rows behind the k exchange rows
+int gon_skip_segments(int dtype, int d, int64_t n, int k, int grid, int *ends, int cap);
+cudaError_t launch_gon_probe(const GonInst &I, int it0, int *route, unsigned *words, DevStatus *st, cudaStream_t s);
+cudaError_t launch_gon_skip(GonArgs &a, int last, cudaStream_t s);
 // Resident form for one instance of n points (row-major rows in device
 // memory): the grid (0 when the instance does not fit on chip or d has no
 // specialisation), with the shared-memory columns per coordinate in *cap and
@@ -307,6 +344,9 @@ int device_clock_khz(int dev);
 // then the CTAs' lower bounds).
 __host__ __device__ inline int64_t slot_stride(int G) { return (int64_t)G; }
 inline int64_t slot_words(int64_t k, int G, bool lp) { return k * slot_stride(G) * (lp ? 2 : 1); }
+// Words the first CTA of a large group publishes a step's result in
+// (group_exchange): the key's halves and the d coordinates.
+inline int64_t bc_words(int d) { return (d + 2 + 15) / 16 * 16; }
 int gon_queue_warps();
 int gon_warps_per_cta();
 
@@ -321,6 +361,7 @@ inline void gon_single(GonArgs &g, const void *pk, int dtype, int64_t n, int d, 
     I.rm = nullptr;
     I.mind = mind;
     I.slots = slots;
+    I.bc = nullptr;
     I.centers = centers;
     I.k_out = k_out;
     I.final_key = final_key;
@@ -335,6 +376,12 @@ inline void gon_single(GonArgs &g, const void *pk, int dtype, int64_t n, int d, 
     I.ecmax_out = nullptr;
     I.m32 = nullptr;
     I.stamp = nullptr;
+    I.asg = nullptr;
+    I.rmap = nullptr;
+    I.skip_perm[0] = I.skip_perm[1] = I.skip_mind[0] = I.skip_mind[1] = nullptr;
+    I.skip_asg = nullptr;
+    I.skip_hist = nullptr;
+    I.it0 = I.it1 = 0;
     I.lp_kind = 0;
     I.kcap = k;
     I.lo = 0;
@@ -468,6 +515,9 @@ struct RadiusArgs {
     // fp16 sweep: the device word holding its power-of-two scale (the
     // bounds above are in the scaled units); nullptr = 1
     const float *lpscale;
+    // device word: non-zero when mind holds canonical minima after all (the
+    // solve changed over to the skip kernel) and the three above do not apply
+    const int *route;
     // tensor-core filter scratch (float points, d <= 128); tc_at null: CUDA cores
     void *tc_at, *tc_bt;
     float *tc_an, *tc_ae, *tc_cn, *tc_ce, *tc_mlo, *tc_mhi;
