@@ -68,6 +68,11 @@
  *                            they fit, d = 8 or 10)
  *  KC_GON_RESIDENT_PTS=P     points per CTA the resident form aims for
  *                            (default 4096)
+ *  KC_GON_SKIP=0|1           single float Gonzalez solves never change over to
+ *                            the kernel that leaves out distances by the
+ *                            triangle inequality / change over at the first
+ *                            probe whatever the sizes (default: on large sets,
+ *                            where a probe expects it to be faster)
  *  KC_GON_TAIL=0             no shared tail of blocks in large streaming FP32
  *                            Gonzalez launches
  *  KC_LP_LOCAL_T=1           mixed-precision sweeps recheck against each CTA's

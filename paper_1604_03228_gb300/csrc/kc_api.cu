@@ -431,6 +431,49 @@ void attach_lp(GonInst &I, const LPBufs &L, int lp, float *cenT, int kcap, float
     I.lp_kind = lp;
 }
 
+// Scratch of the skip kernel (kc_gonskip.cu) for n points.
+struct SkipBufs {
+    uint16_t *asg[2];
+    uint32_t *perm[2], *mind[2];
+    unsigned *hist;
+};
+
+void take_skip(Carve &cv, SkipBufs &B, int64_t n, int grid) {
+    const size_t np = (size_t)skip_positions(n);
+    for (int i = 0; i < 2; ++i) {
+        B.asg[i] = cv.take<uint16_t>(np);
+        B.perm[i] = cv.take<uint32_t>(np);
+        B.mind[i] = cv.take<uint32_t>(np);
+    }
+    B.hist = cv.take<unsigned>((size_t)skip_hist_words(grid));
+}
+
+void attach_skip(GonInst &I, const SkipBufs &B) {
+    I.asg = B.asg[0];
+    I.skip_asg = B.asg[1];
+    for (int i = 0; i < 2; ++i) {
+        I.skip_perm[i] = B.perm[i];
+        I.skip_mind[i] = B.mind[i];
+    }
+    I.skip_hist = B.hist;
+}
+
+// A single instance: the streaming kernel to the end, or (nseg > 0) in
+// segments with a probe behind each, and the skip kernel for the steps after
+// the one at which a probe changed over.
+cudaError_t launch_gon_segments(GonArgs &g, const int *ends, int nseg, int *route, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i <= nseg && e == cudaSuccess; ++i) {
+        g.single.it0 = i > 0 ? ends[i - 1] : 0;
+        g.single.it1 = i < nseg ? ends[i] : 0;
+        e = launch_gon(g, s);
+        if (i < nseg && e == cudaSuccess)
+            e = launch_gon_probe(g.single, ends[i], route, (unsigned *)route + 4, g.st, s);
+    }
+    if (nseg && e == cudaSuccess) e = launch_gon_skip(g, ends[nseg - 1], s);
+    return e;
+}
+
 int choose_gon_grid(int dtype, int d, int64_t n, int lp = 0) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -629,10 +672,17 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
                      nblocks(n) >= 4 * (int64_t)grid * gon_warps_per_cta();   // claimed blocks pay off
     bool use_tail = dyn && grid > 1 && nblocks(n) * 7 / 8 / ((int64_t)grid * gon_warps_per_cta()) >= 2;
     if (const char *env = getenv("KC_GON_TAIL")) use_tail = use_tail && atoi(env) != 0;
+    // large float sets whose rows are in device memory may change over to the
+    // skip kernel after one of these steps
+    int seg_end[8];
+    const int nseg = !res_grid && !pin_pts && !bad_index
+                         ? gon_skip_segments(c.o.dtype, d, n, keff, grid, seg_end, 8) : 0;
     const int64_t nb = nblocks(n);
     const size_t esz = 4;
     LPBufs LB;
     float *cenT = nullptr, *ecmax = nullptr;
+    SkipBufs SB;
+    unsigned *route = nullptr;   // the route word and the probe's words
 
     auto layout = [&](Carve &cv, GonArgs &g, RadiusArgs &ra, void **staging, int64_t **cen_dev,
                       int32_t **kout_dev, double **rad_dev, size_t *zero_bytes) {
@@ -644,13 +694,15 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
         // per (step, CTA): argmax keys, and for the mixed-precision sweep the
         // CTAs' lower bounds too
         uint64_t *slots = cv.take<uint64_t>(res_grid ? (size_t)keff * grid * res_sw
-                                                      : (size_t)slot_words(keff, grid, lp != 0));
+                                                      : (size_t)slot_words(keff, grid, lp != 0) +
+                                                            (nseg ? (size_t)skip_slot_rows() * grid : 0));
         uint64_t *bc = cv.take<uint64_t>((size_t)bc_words(d));
         int *tail = use_tail ? cv.take<int>((size_t)keff) : nullptr;
         unsigned *flag_words = c.o.dtype == KC_F32 ? cv.take<unsigned>(2) : nullptr;   // flagged count, done
+        route = nseg ? cv.take<unsigned>((size_t)skip_route_words()) : nullptr;
         *zero_bytes = cv.off;
         *staging = (dev_pts || pin_pts) ? nullptr : cv.take<char>((size_t)n * d * esz);
-        void *pk = res_grid ? nullptr : cv.take<char>((size_t)nb * BLK * d * esz);
+        void *pk = res_grid ? nullptr : cv.take<char>((size_t)(nseg ? skip_positions(n) : nb * BLK) * d * esz);
         uint32_t *mind = cv.take<uint32_t>((size_t)nb * BLK);
         void *cen = cv.take<char>((size_t)keff * d * esz);
         double *m64 = cv.take<double>(c.o.dtype == KC_F32 ? (size_t)n : 1);
@@ -658,8 +710,9 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
         *kout_dev = dev_kout ? k_out : cv.take<int32_t>(1);
         *rad_dev = dev_rad ? radius : cv.take<double>(1);
         take_lp(cv, LB, lp, n, d);
-        cenT = lp ? cv.take<float>((size_t)keff * d) : nullptr;
+        cenT = lp || nseg ? cv.take<float>((size_t)keff * d) : nullptr;
         ecmax = lp ? cv.take<float>(1) : nullptr;
+        if (nseg) take_skip(cv, SB, n, grid);
         gon_single(g, pk, c.o.dtype, n, d, keff, first, mind, slots, *cen_dev, *kout_dev,
                    (uint64_t *)key32, range2, grid);
         g.single.tail = tail;
@@ -688,6 +741,7 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
         ra.radius_out = *rad_dev;
         ra.argmax_out = nullptr;
         ra.have_mind = true;
+        ra.route = (const int *)route;
         if (flag_words) {
             ra.flagged = cv.take<uint32_t>((size_t)n);
             ra.flagged_n = flag_words;
@@ -724,7 +778,14 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
     r = stage_points(c, pts, (size_t)n * d * esz, dev_pts, staging, &src, pin_pts);
     if (r != KC_OK) return r;
     // exact rechecks read the FP32 rows where they are in device memory
-    if (lp && !pin_pts) g.single.rm = (const float *)src;
+    if ((lp && !pin_pts) || nseg) g.single.rm = (const float *)src;
+    if (nseg) {
+        attach_skip(g.single, SB);
+        ra.pk = nullptr;   // the skip kernel packs the points anew, in its own order
+        ra.rm = (const float *)src;
+        g.single.cenT = cenT;
+        g.route = (int *)route;
+    }
     if (res_grid) {
         // the resident kernel reads (and checks) the rows itself: no pack
         g.single.pk = src;
@@ -743,7 +804,7 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
     }
     {
         TraceStep t("gonzalez", c.s);
-        KC_CUDA(launch_gon(g, c.s), "gonzalez launch");
+        KC_CUDA(launch_gon_segments(g, seg_end, nseg, (int *)route, c.s), "gonzalez launch");
         if (res_grid && c.o.dtype == KC_I32)
             KC_CUDA(launch_range_check(g.single.range2, d, c.arena->status, c.s), "range check");
     }

@@ -310,11 +310,15 @@ __global__ void __launch_bounds__(256) recheck_kernel(
     const int32_t *kc_dev, int kc_max, const uint32_t *__restrict__ mind, const unsigned long long *key32,
     unsigned long long *max64, double *m64, DevStatus *st, const float *eblk, const float *ecmax,
     const float *lpscale, const uint32_t *__restrict__ list, const unsigned long long *lcount, uint32_t *flagged,
-    unsigned *flagged_n, unsigned *done, double *radius_out, int64_t *argmax_out) {
+    unsigned *flagged_n, unsigned *done, double *radius_out, int64_t *argmax_out, const int *route) {
     __shared__ int s_last;
     __shared__ unsigned long long s_arg[8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool run = ld_volatile_i32(&st->code) == 0 && key_val(*key32) != 0;
+    if (route && *route != 0) {   // canonical minima after all
+        eblk = nullptr;
+        lpscale = nullptr;
+    }
     if (run) {
         const double sc = lpscale ? (double)*lpscale : 1.0;
         const int kc = (int)dev_count(kc_dev, kc_max);
@@ -473,7 +477,7 @@ cudaError_t launch_radius(RadiusArgs &a, cudaStream_t s) {
         recheck_kernel<<<grid, 256, 0, s>>>((const float *)a.pk, a.rm, a.n, a.d, (const float *)a.cen, a.kc_dev,
                                             a.kc_max, a.mind, a.key32, a.max64, a.m64, a.st, a.eblk, a.ecmax,
                                             a.lpscale, tcl ? a.tc_flist : nullptr, tcl ? a.tc_fcount : nullptr,
-                                            a.flagged, a.flagged_n, a.done, a.radius_out, a.argmax_out);
+                                            a.flagged, a.flagged_n, a.done, a.radius_out, a.argmax_out, a.route);
         const bool tc = tcl;
         note_launches(2 + (a.have_mind || tc ? 0 : 1));
         return cudaGetLastError();

@@ -1,0 +1,75 @@
+"""The Gonzalez steps that leave out distances by the triangle inequality
+(KC_GON_SKIP=1 changes over at the first probe, after 16 steps) against the
+oracle: sizes around units of 32 and blocks of 128 points, several regroupings,
+coordinate counts around the loads' batches, unaligned rows, ties, duplicate
+points and an early stop, and behind the low-precision sweeps.
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1604_03228_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+def _dev(x):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+def _check(kc, pts, k, first=0, **kw):
+    x = kw.pop("x", None)
+    r = kc.kc_gonzalez(_dev(pts) if x is None else x, k, first=first, **kw)
+    ref = O.gonzalez(pts, k, first=first, mode="f32")
+    assert r.centers.cpu().numpy().tolist() == ref.centers.tolist()
+    assert r.k_out == len(ref.centers)
+    assert r.radius == O.radius(pts, ref.centers, mode="f64")[0]
+
+
+@pytest.fixture(autouse=True)
+def _forced(monkeypatch):
+    monkeypatch.setenv("KC_GON_SKIP", "1")
+    monkeypatch.setenv("KC_GON_RESIDENT", "0")
+
+
+@pytest.mark.parametrize("n,d,k", [(31, 3, 30), (129, 5, 60), (4097, 1, 40), (20_000, 16, 200), (33_333, 37, 100),
+                                   (60_000, 64, 300), (9_000, 65, 40), (5_000, 130, 30), (50_000, 2, 600)])
+@pytest.mark.parametrize("shape", ["gau", "unif"])
+def test_skip_equals_oracle(kc, n, d, k, shape):
+    pts = (I.gauss_mixture(n, d, 700 + d, 20, 0.5, -10.0, 10.0) if shape == "gau" else I.unif_points(n, d, 700 + d))
+    _check(kc, pts, k, first=n // 3)
+
+
+@pytest.mark.parametrize("sweep", ["bf16", "fp16", "fp8"])
+def test_skip_behind_a_low_precision_sweep(kc, sweep):
+    _check(kc, I.gauss_mixture(40_000, 24, 710, 30, 0.5, -10.0, 10.0), 120, sweep=sweep)
+
+
+def test_skip_unaligned_rows(kc):
+    import torch
+    pts = I.gauss_mixture(20_000, 12, 711, 10, 0.5, -10.0, 10.0)
+    buf = torch.empty(pts.size + 1, dtype=torch.float32, device="cuda")
+    x = buf[1:].view(pts.shape)
+    x.copy_(torch.from_numpy(pts))
+    _check(kc, pts, 90, x=x)
+
+
+def test_skip_ties_duplicates_and_early_stop(kc):
+    grid = I.int_points(30_000, 3, 712, 0, 4).astype(np.float32)   # 125 distinct points
+    _check(kc, grid, 100)
+    r = kc.kc_gonzalez(_dev(grid), 300)
+    assert r.k_out == len(O.gonzalez(grid, 300, mode="f32").centers) < 300 and r.radius == 0.0
+
+
+@pytest.mark.parametrize("scale", [1e-22, 2e-20, 1e-15, 1e16])
+def test_skip_tiny_and_huge_coordinates(kc, monkeypatch, scale):
+    # squared distances that underflow, and near the largest accepted
+    # magnitude: the same as the streaming kernel
+    pts = (I.gauss_mixture(20_000, 4, 713, 8, 0.01, -1.0, 1.0) * np.float32(scale)).astype(np.float32)
+    x = _dev(pts)
+    a = kc.kc_gonzalez(x, 60)
+    monkeypatch.setenv("KC_GON_SKIP", "0")
+    b = kc.kc_gonzalez(x, 60)
+    assert a.centers.cpu().tolist() == b.centers.cpu().tolist() == O.gonzalez(pts, 60, mode="f32").centers.tolist()
+    assert (a.k_out, a.radius) == (b.k_out, b.radius)
