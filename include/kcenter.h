@@ -53,6 +53,9 @@
  *  KC_PRUNE_TC=0|1           EIM prune on CUDA cores / tensor cores (default:
  *                            tensor cores for float points, 16 <= d <= 128,
  *                            |S| >= 256)
+ *  KC_EIM_CELLS=0|1          EIM's prune never / wherever S has 1024 points by
+ *                            Voronoi cells of pivots (default: float points,
+ *                            when the block |R| x |S| is large)
  *  KC_TC_STREAM_CENTERS=1    tensor-core blocks stream the center tiles through
  *                            a two-stage ring even when all of them fit in
  *                            shared memory

@@ -474,6 +474,9 @@ cudaError_t launch_gon_segments(GonArgs &g, const int *ends, int nseg, int *rout
     return e;
 }
 
+// Pivots of EIM's prune on the tensor cores.
+constexpr int EIM_PIVOTS_TC = 128;
+
 int choose_gon_grid(int dtype, int d, int64_t n, int lp = 0) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -1401,6 +1404,19 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
     const int keff_max = (int)std::min<int64_t>(k, n);
     const int lp = lp_of(c.o);
     const int grid = choose_gon_grid(c.o.dtype, d, n, lp);
+    // the prune by cells: float points on the CUDA cores for d < 16, on the
+    // tensor cores above; pivots (cells) at most
+    const char *cenv = getenv("KC_EIM_CELLS");
+    const bool cells_ok = c.o.dtype == KC_F32 && !(cenv && atoi(cenv) == 0);
+    const int Pmax = !cells_ok ? 0 : (d < 16 ? CELLS_MAX : EIM_PIVOTS_TC);
+    const int64_t npad = n + (int64_t)Pmax * (TC_CELL_UNIT - 1);   // a list sorted by cell
+    constexpr int64_t PSAMPLE = 8192;                              // rows of S the pivots are chosen from (d >= 16)
+    CellBufs CB;
+    CellSort CR, CS;
+    int *ctiles = nullptr, *cntile = nullptr;
+    bool assigned = false;
+    SkipBufs SB{};
+    const bool skip_ok = !lp && gon_skip_possible(c.o.dtype, d, n, keff_max, grid);
     LPBufs LB;
     float *cenT = nullptr, *ecmax = nullptr;
     RadiusArgs Rtc{}, Ptc{};
@@ -1411,7 +1427,13 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         int32_t *range2;
         unsigned long long *key32, *max64, *arg64;
         uint32_t *thr, *v;
-        uint64_t *fk, *slots, *bc;
+        uint64_t *fk, *slots, *bc, *pslots, *pfk;
+        unsigned *route;
+        void *ppk;
+        uint32_t *pmind;
+        int64_t *pcen;
+        int32_t *pk_out;
+        float *Ss, *cenT;
         uint8_t *mask;
         PruneBufs pb;
         void *staging, *pk, *Sc, *Hc, *pkC, *cen;
@@ -1436,7 +1458,11 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         Lo.thr = cv.take<uint32_t>(1);
         Lo.v = cv.take<uint32_t>(1);
         Lo.fk = cv.take<uint64_t>(1);
-        Lo.slots = cv.take<uint64_t>((size_t)slot_words(keff_max, grid, lp != 0));
+        Lo.slots = cv.take<uint64_t>((size_t)slot_words(keff_max, grid, lp != 0) +
+                                     (skip_ok ? (size_t)skip_slot_rows() * grid : 0));
+        Lo.route = skip_ok ? cv.take<unsigned>((size_t)skip_route_words()) : nullptr;
+        Lo.pfk = cv.take<uint64_t>(1);
+        Lo.pslots = Pmax ? cv.take<uint64_t>((size_t)slot_words(EIM_PIVOTS_TC, 8, false)) : nullptr;
         Lo.bc = cv.take<uint64_t>((size_t)bc_words(d));
         Lo.mask = cv.take<uint8_t>((size_t)n);
         Lo.zero_bytes = cv.off;
@@ -1453,9 +1479,34 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         Lo.counts = cv.take<int>((size_t)nchunks);
         Lo.offs = cv.take<int64_t>((size_t)nchunks);
         Lo.C = cv.take<int64_t>((size_t)n);
-        Lo.pkC = cv.take<char>((size_t)nb * BLK * d * esz);
+        Lo.pkC = cv.take<char>((size_t)(skip_ok ? skip_positions(n) : nb * BLK) * d * esz);
+        if (skip_ok) take_skip(cv, SB, n, grid);
+        if (Pmax) {
+            CB.piv = cv.take<float>((size_t)Pmax * d);
+            CB.cell = cv.take<uint16_t>((size_t)nb * BLK);
+            CB.dist = cv.take<uint32_t>((size_t)nb * BLK);
+            CB.near = cv.take<uint16_t>((size_t)Pmax * Pmax);
+            CB.nnear = cv.take<int>((size_t)Pmax);
+            for (CellSort *o : {&CR, &CS}) {
+                o->idx = cv.take<uint32_t>((size_t)npad);
+                o->count = cv.take<unsigned>(2 * (size_t)Pmax);
+                o->start = cv.take<unsigned>((size_t)Pmax + 1);
+                o->cursor = cv.take<unsigned>((size_t)Pmax);
+            }
+            if (d < 16) {
+                Lo.Ss = cv.take<float>((size_t)n * d);
+            } else {
+                ctiles = cv.take<int>((size_t)Pmax * tc_center_tiles(npad));
+                cntile = cv.take<int>((size_t)Pmax);
+                Lo.ppk = cv.take<char>((size_t)PSAMPLE * d * esz);
+                Lo.pmind = cv.take<uint32_t>((size_t)PSAMPLE);
+                Lo.pcen = cv.take<int64_t>((size_t)Pmax);
+                Lo.pk_out = cv.take<int32_t>(1);
+            }
+        }
         Lo.mindC = cv.take<uint32_t>((size_t)nb * BLK);
         Lo.cen = cv.take<char>((size_t)keff_max * d * esz);
+        Lo.cenT = skip_ok ? cv.take<float>((size_t)keff_max * d) : nullptr;
         Lo.m64 = cv.take<double>(c.o.dtype == KC_F32 ? (size_t)n : 1);
         Lo.cen_dev = dev_cen ? centers : cv.take<int64_t>((size_t)keff_max);
         Lo.kout_dev = dev_kout ? k_out : cv.take<int32_t>(1);
@@ -1471,14 +1522,14 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         const char *ptc = getenv("KC_PRUNE_TC");
         const bool tcp = c.o.dtype == KC_F32 && tc_supported(d) && (ptc ? atoi(ptc) != 0 : d >= 16);
         Ptc.tc_at = nullptr;
-        if (tcp) {   // tiles for up to n points of R and n centers of S
-            Ptc.tc_at = cv.take<char>(tc_point_bytes(n, d));
-            Ptc.tc_an = cv.take<float>((size_t)tc_point_rows(n));
-            Ptc.tc_ae = cv.take<float>((size_t)tc_point_rows(n));
-            Ptc.tc_rin = cv.take<uint8_t>((size_t)tc_point_rows(n));
-            Ptc.tc_bt = cv.take<char>(tc_center_bytes(n, d));
-            Ptc.tc_cn = cv.take<float>((size_t)tc_center_tiles(n) * 256);
-            Ptc.tc_ce = cv.take<float>((size_t)tc_center_tiles(n) * 256);
+        if (tcp) {   // tiles for up to n points of R and n centers of S, sorted by cell
+            Ptc.tc_at = cv.take<char>(tc_point_bytes(npad, d));
+            Ptc.tc_an = cv.take<float>((size_t)tc_point_rows(npad));
+            Ptc.tc_ae = cv.take<float>((size_t)tc_point_rows(npad));
+            Ptc.tc_rin = cv.take<uint8_t>((size_t)tc_point_rows(npad));
+            Ptc.tc_bt = cv.take<char>(tc_center_bytes(npad, d));
+            Ptc.tc_cn = cv.take<float>((size_t)tc_center_tiles(npad) * 256);
+            Ptc.tc_ce = cv.take<float>((size_t)tc_center_tiles(npad) * 256);
             Ptc.tc_maxes = cv.take<unsigned>(3);
             Ptc.tc_absmax = cv.take<unsigned>(3);
         }
@@ -1487,9 +1538,9 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
             Lo.pb.pcap = std::max<int64_t>(2 * n, 1 << 16);
             if (const char *e = getenv("KC_PRUNE_PAIR_CAP")) Lo.pb.pcap = std::max<int64_t>(1, atoll(e));
             Lo.pb.pairs = cv.take<uint2>((size_t)Lo.pb.pcap);
-            Lo.pb.flag = cv.take<uint8_t>((size_t)n);
-            Lo.pb.hit = cv.take<uint8_t>((size_t)n);
-            Lo.pb.pend = cv.take<uint32_t>((size_t)n);
+            Lo.pb.flag = cv.take<uint8_t>((size_t)npad);
+            Lo.pb.hit = cv.take<uint8_t>((size_t)npad);
+            Lo.pb.pend = cv.take<uint32_t>((size_t)npad);
             Lo.pb.npairs = cv.take<unsigned long long>(1);
             Lo.pb.npend = cv.take<unsigned long long>(1);
         }
@@ -1559,7 +1610,53 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
             }
             TraceStep t("eim_prune", c.s);
             g_prune_pairs += (unsigned long long)rn * (unsigned long long)sn;
-            if (Ptc.tc_at && sn >= 256) {
+            const bool tcp = Ptc.tc_at && sn >= 256;
+            // by cells when the whole block costs more than assigning and sorting
+            bool cells = Pmax > 0 && (assigned || sn >= 1024) && (tcp ? d >= 16 && tc_prune_pairs(d, sn) : d < 16) &&
+                         (cenv || (double)rn * (double)sn * d >= (tcp ? 2e12 : 4e9));
+            if (cells && !assigned) {
+                if (d < 16) {
+                    // pivots: the first rows of S (a random sample of the points)
+                    CB.P = (int)std::min<int64_t>(CELLS_MAX, std::max<int64_t>(64, sn / 16));
+                    KC_CUDA(cudaMemcpyAsync(CB.piv, Lo.Sc, (size_t)CB.P * d * esz, cudaMemcpyDeviceToDevice, c.s),
+                            "pivots");
+                } else {
+                    // pivots: Gonzalez centers of a part of S, so that every
+                    // cluster gets one
+                    CB.P = EIM_PIVOTS_TC;
+                    const int64_t M = std::min<int64_t>(sn, PSAMPLE);
+                    KC_CUDA(launch_pack(Lo.Sc, c.o.dtype, M, d, Lo.ppk, Lo.range2, st, c.s), "pivot pack");
+                    GonArgs g{};
+                    gon_single(g, Lo.ppk, c.o.dtype, M, d, CB.P, 0, Lo.pmind, Lo.pslots, Lo.pcen, Lo.pk_out, Lo.pfk,
+                               Lo.range2, std::min(8, choose_gon_grid(c.o.dtype, d, M)));
+                    g.st = st;
+                    g.timeout_cycles = timeout_cycles(c.o);
+                    KC_CUDA(launch_gon(g, c.s), "pivot selection");
+                    KC_CUDA(launch_pivot_rows((const float *)Lo.Sc, M, d, Lo.pcen, Lo.pk_out, CB.P, CB.piv, c.s),
+                            "pivot rows");
+                }
+                KC_CUDA(launch_cells_assign((const float *)Lo.pk, n, d, CB, c.s), "cell assignment");
+                assigned = true;
+            }
+            if (cells) {
+                const int ru = tcp ? TC_CELL_UNIT : cells_prune_unit(), su = tcp ? TC_CELL_UNIT : 1;
+                KC_CUDA(launch_cells_sort(Rc, rn, ru, CB, CR, c.s), "sort R");
+                KC_CUDA(launch_cells_sort(Lo.S, sn, su, CB, CS, c.s), "sort S");
+                KC_CUDA(launch_cells_near(d, CB, CR, CS, Lo.thr, c.s), "near cells");
+            }
+            if (cells && tcp) {
+                const int64_t rp = rn + (int64_t)CB.P * (TC_CELL_UNIT - 1), sp = sn + (int64_t)CB.P * (TC_CELL_UNIT - 1);
+                const int cap = tc_center_tiles(sp);
+                KC_CUDA(launch_cells_tiles(CB, CS, TC_CELL_UNIT, cap, ctiles, cntile, c.s), "center tiles");
+                const TcCells tcc{&CR, &CS, CB.P, ctiles, cntile, cap};
+                KC_CUDA(launch_tc_prune((const float *)src, d, nullptr, rp, Lo.mask, nullptr, sp, tc_bufs(Ptc), Lo.pb,
+                                        Lo.thr, Rx, Lo.rnn, st, c.s, &tcc),
+                        "prune");
+            } else if (cells) {
+                KC_CUDA(launch_eim_gather_rows(src, c.o.dtype, d, CS.idx, 0, sn, Lo.Ss, c.s), "sorted S");
+                KC_CUDA(launch_cells_prune((const float *)src, d, rn, Lo.mask, Lo.Ss, CB, CR, CS, Lo.thr, Rx, Lo.rnn, c.s),
+                        "prune");
+            } else if (tcp) {
                 // tensor-core R x S block with exact rechecks of undecided pairs
                 KC_CUDA(launch_tc_prune((const float *)src, d, Rc, rn, Lo.mask, (const float *)Lo.Sc, sn, tc_bufs(Ptc),
                                         Lo.pb, Lo.thr, Rx, Lo.rnn, st, c.s),
@@ -1608,7 +1705,16 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         }
         g.st = st;
         g.timeout_cycles = timeout_cycles(c.o);
-        KC_CUDA(launch_gon(g, c.s), "gonzalez launch");
+        int seg_end[8];
+        const int nseg = skip_ok ? gon_skip_segments(c.o.dtype, d, nC, kC, g.grid, seg_end, 8) : 0;
+        if (nseg) {   // the rows of the sample are found through its index
+            attach_skip(g.single, SB);
+            g.single.rm = (const float *)src;
+            g.single.rmap = Lo.C;
+            g.single.cenT = Lo.cenT;
+            g.route = (int *)Lo.route;
+        }
+        KC_CUDA(launch_gon_segments(g, seg_end, nseg, (int *)Lo.route, c.s), "gonzalez launch");
     }
     {
         TraceStep t("radius", c.s);

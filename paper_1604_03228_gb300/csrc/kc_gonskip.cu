@@ -782,6 +782,11 @@ int gon_skip_segments(int dtype, int d, int64_t n, int k, int grid, int *ends, i
     return m;
 }
 
+bool gon_skip_possible(int dtype, int d, int64_t n, int k, int grid) {
+    int ends[8];
+    return gon_skip_segments(dtype, d, n, k, grid, ends, 8) > 0;
+}
+
 cudaError_t launch_gon_probe(const GonInst &I, int it0, int *route, unsigned *words, DevStatus *st, cudaStream_t s) {
     // microseconds: a whole sweep at the HBM rate (half the bytes in mixed
     // precision), the assignment at the FP32 rate and two regroupings

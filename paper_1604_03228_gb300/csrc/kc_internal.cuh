@@ -323,6 +323,7 @@ int64_t skip_positions(int64_t n);   // positions of the regrouped arrays, at mo
 int64_t skip_hist_words(int G);
 int64_t skip_route_words();          // the route word, the probe's counter and its sample
 int64_t skip_slot_rows();            // slot rows behind the k exchange rows
+bool gon_skip_possible(int dtype, int d, int64_t n, int k, int grid);   // for n points at most
 int gon_skip_segments(int dtype, int d, int64_t n, int k, int grid, int *ends, int cap);
 cudaError_t launch_gon_probe(const GonInst &I, int it0, int *route, unsigned *words, DevStatus *st, cudaStream_t s);
 cudaError_t launch_gon_skip(GonArgs &a, int last, cudaStream_t s);
@@ -486,6 +487,41 @@ cudaError_t launch_eim_mark(const uint32_t *R, int64_t rn, uint8_t *mask, cudaSt
 cudaError_t launch_compact(const uint8_t *mask, int64_t n, int *counts, int64_t *offs, int64_t *out, int64_t *total,
                            cudaStream_t s);
 
+// --------------------------------------------------- EIM's prune by cells
+// Pivots (rows), every point's cell and canonical distance to its pivot, and
+// the near lists of a round (kc_cells.cu).
+constexpr int CELLS_MAX = 1024;
+struct CellBufs {
+    int P = 0;
+    float *piv = nullptr;      // [P][d]
+    uint16_t *cell = nullptr;  // [nblocks(n) * BLK]
+    uint32_t *dist = nullptr;  // [nblocks(n) * BLK] value bits
+    uint16_t *near = nullptr;  // [P][P] cells of S near a cell of R
+    int *nnear = nullptr;      // [P]
+};
+// A list of points sorted by cell: cell p's points are idx[start[p] ..), each
+// start a multiple of the unit, gaps 0xFFFFFFFF.
+struct CellSort {
+    uint32_t *idx = nullptr;    // [cnt + P (unit - 1)]
+    unsigned *count = nullptr;  // [2 P]: points, largest distance (value bits)
+    unsigned *start = nullptr;  // [P + 1]
+    unsigned *cursor = nullptr; // [P]
+};
+cudaError_t launch_pivot_rows(const float *rows, int64_t n, int d, const int64_t *centers, const int32_t *k_out, int P,
+                              float *piv, cudaStream_t s);
+cudaError_t launch_cells_assign(const float *pk, int64_t n, int d, const CellBufs &C, cudaStream_t s);
+cudaError_t launch_cells_sort(const uint32_t *list, int64_t cnt, int unit, const CellBufs &C, CellSort &O,
+                              cudaStream_t s);
+cudaError_t launch_cells_near(int d, const CellBufs &C, const CellSort &R, const CellSort &S, const uint32_t *thr,
+                              cudaStream_t s);
+cudaError_t launch_cells_tiles(const CellBufs &C, const CellSort &S, int tile, int cap, int *tiles, int *ntile,
+                               cudaStream_t s);
+int cells_prune_unit();
+// Float points, d <= 16; R sorted with that unit, S with unit 1, Ss its rows.
+cudaError_t launch_cells_prune(const float *src, int d, int64_t rn, const uint8_t *inS, const float *Ss,
+                               const CellBufs &C, const CellSort &R, const CellSort &S, const uint32_t *thr, uint32_t *Rn,
+                               unsigned long long *rnn, cudaStream_t s);
+
 struct RadiusArgs {
     const void *pk;
     // float points may come row-major instead ([n][d], pk null): on the
@@ -576,9 +612,21 @@ struct PruneBufs {
     unsigned long long *npairs, *npend;
 };
 // B.absmax must already hold the coordinate maximum over a superset of R and S.
+// cells (optional): R and S come sorted by cell instead, both with unit
+// TC_CELL_UNIT (rn and sn then count the positions, gaps included), Scen is not
+// read, and a point pair of tiles meets the near cells' center tiles only
+// (tiles [P][tcap], ntile [P]).
+constexpr int TC_CELL_UNIT = 256;   // a pair of point tiles, or one center tile
+struct TcCells {
+    const CellSort *R, *S;
+    int P;
+    const int *tiles, *ntile;
+    int tcap;
+};
 cudaError_t launch_tc_prune(const float *src, int d, const uint32_t *R, int64_t rn, const uint8_t *inS, const float *Scen,
                             int64_t sn, const TcBufs &B, const PruneBufs &P, const uint32_t *thr, uint32_t *Rn,
-                            unsigned long long *rnn, DevStatus *st, cudaStream_t s);
+                            unsigned long long *rnn, DevStatus *st, cudaStream_t s, const TcCells *cells = nullptr);
+bool tc_prune_pairs(int d, int64_t sn);   // streamed centers, two point tiles per center tile (cells need it)
 cudaError_t launch_radius(RadiusArgs &a, cudaStream_t s);
 
 }  // namespace kc

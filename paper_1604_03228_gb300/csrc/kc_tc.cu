@@ -464,7 +464,7 @@ __global__ void tc_rows_kernel(const float *__restrict__ pk, const float *__rest
         const int64_t t = i / R;
         const int r = (int)(i % R);
         __half *tile = tiles + t * (int64_t)R * kp;
-        const bool valid = i < cnt;
+        const bool valid = i < cnt && (!idx || idx[i] != 0xFFFFFFFFu);   // sorted lists have gaps
         int64_t g = 0;
         if (valid) g = pk ? i : (idx ? (int64_t)idx[i] : i);
         // coordinates first: norm and rounding bound
@@ -561,7 +561,31 @@ struct TcArgs {
     uint8_t *pflag;             // per row: bit 0 pairs deferred, bit 1 pair buffer overflowed
     uint32_t *pend;             // rows decided by the pair check
     unsigned long long *npend;
+    // prune by cells (tc_dmin2_kernel): the starts of the cells of the sorted
+    // rows, and per cell the center tiles it meets; null: all of them
+    const unsigned *rstart;
+    int P, tcap;
+    const int *tiles, *ntile;
     DevStatus *st;
+};
+
+// The center tiles of point-tile pair pp: how many, and the i-th.
+struct PairTiles {
+    const int *list;
+    int count;
+    __device__ __forceinline__ PairTiles(const TcArgs &a, int64_t pp) : list(nullptr), count(a.ntiles) {
+        if (!a.tiles) return;
+        const int64_t r0 = pp * TC_CELL_UNIT;
+        int lo = 0, hi = a.P;   // the last cell that starts at or before row r0 (P: past the last row)
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if ((int64_t)__ldg(a.rstart + mid) <= r0) lo = mid;
+            else hi = mid - 1;
+        }
+        count = lo < a.P ? __ldg(a.ntile + lo) : 0;
+        list = a.tiles + (int64_t)lo * a.tcap;
+    }
+    __device__ __forceinline__ int operator[](int i) const { return list ? __ldg(list + i) : i; }
 };
 
 __device__ __forceinline__ float tc_eta(int d, int kp) {
@@ -764,6 +788,20 @@ __global__ void __launch_bounds__(384, 1) tc_dmin_kernel(TcArgs a) {
             bool emitted = false, ovf = false;
             volatile int *s_gone_v = s_gone;
             int cbase = 0;
+            auto emit = [&](uint32_t und, int col) {
+                while (und && !ovf) {
+                    const int64_t ci = (int64_t)col + __ffs(und) - 1;
+                    und &= und - 1;
+                    if (ci >= a.kc) break;
+                    const unsigned long long slot = atomicAdd(a.npairs, 1ull);
+                    if (slot < (unsigned long long)a.pcap)
+                        a.pairs[slot] = make_uint2((uint32_t)pi, (uint32_t)ci);
+                    else
+                        ovf = true;
+                    emitted = true;
+                    ++namb;
+                }
+            };
             // One 32-column chunk of accumulators v (columns cbase + c0 ..),
             // folded into running maxima three values at a time.
             auto chunk = [&](const uint32_t(&r)[32], int c0) {
@@ -784,29 +822,19 @@ __global__ void __launch_bounds__(384, 1) tc_dmin_kernel(TcArgs a) {
                         m0 = max3f(m0, __uint_as_float(r[j]), __uint_as_float(r[j + 1]));
                         m1 = max3f(m1, __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
                     }
-                    if (fmaxf(m0, m1) >= vhi) {
+                    const float mx = fmaxf(m0, m1);
+                    if (mx >= vlo) {
+                        removed = true;
+                        s_gone_v[row] = 1;
+                    } else if (mx >= vhi) {
+                        // undecided: the columns as a mask, deferred to the exact
+                        // pair check one by one (an unrolled check and atomic per
+                        // column was so much code that the warps waited for
+                        // instructions: nine tenths of the prune by cells)
+                        uint32_t und = 0;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float v = __uint_as_float(r[j]);
-                            if (v >= vhi && !removed) {
-                                if (v >= vlo) {
-                                    removed = true;
-                                } else if (!ovf) {
-                                    // undecided: deferred to the exact pair check
-                                    const int64_t ci = (int64_t)cbase + c0 + j;
-                                    if (ci < a.kc) {
-                                        const unsigned long long slot = atomicAdd(a.npairs, 1ull);
-                                        if (slot < (unsigned long long)a.pcap)
-                                            a.pairs[slot] = make_uint2((uint32_t)pi, (uint32_t)ci);
-                                        else
-                                            ovf = true;
-                                        emitted = true;
-                                        ++namb;
-                                    }
-                                }
-                            }
-                        }
-                        if (removed) s_gone_v[row] = 1;
+                        for (int j = 0; j < 32; ++j) und |= __uint_as_float(r[j]) >= vhi ? 1u << j : 0u;
+                        emit(und, cbase + c0);
                     }
                 }
             };
@@ -982,7 +1010,9 @@ __global__ void __launch_bounds__(384, 1) tc_dmin2_kernel(TcArgs a) {
                 if (has2)
                     bulk_g2s(sAb + (2 * sa + 1) * a_bytes, a.at + (t0 + 1) * (int64_t)TC_M * kp, a_bytes, &a_full[sa]);
                 afill ^= 1u << sa;
-                for (int t = 0; t < a.ntiles; ++t, ++u) {
+                const PairTiles pt(a, pp);
+                for (int li = 0; li < pt.count; ++li, ++u) {
+                    const int t = pt[li];
                     const int s = (int)(u & 1);
                     if (!mbar_wait(&b_empty[s], ((bfill >> s) & 1u) ^ 1u, abort)) {
                         *abort = 1;
@@ -1016,7 +1046,8 @@ __global__ void __launch_bounds__(384, 1) tc_dmin2_kernel(TcArgs a) {
                     break;
                 }
                 clk.wa += clock64() - c0;
-                for (int t = 0; t < a.ntiles && !*abort; ++t, ++u) {
+                const int ntl = PairTiles(a, pp).count;
+                for (int t = 0; t < ntl && !*abort; ++t, ++u) {
                     const int s = (int)(u & 1);
                     c0 = clock64();
                     if (!mbar_wait(&b_full[s], (buse >> s) & 1u, abort)) {
@@ -1069,7 +1100,7 @@ __global__ void __launch_bounds__(384, 1) tc_dmin2_kernel(TcArgs a) {
             const int64_t pt = 2 * pp + j;
             if (pt >= ntile_pts) continue;   // the last pair has one tile (uniform over the warp)
             const int64_t pi = pt * TC_M + row;
-            const bool valid = pi < a.npts;
+            const bool valid = pi < a.npts && !(MODE == 1 && a.R[pi] == 0xFFFFFFFFu);   // sorted rows have gaps
             const float xn = valid ? a.an[pi] : 0.f;
             const float sl = __fadd_ru(valid ? a.ae[pi] : 0.f, E);
             const float eps = __fadd_ru(__fmul_ru(eta, __fadd_ru(xn, cnmax2)), rmax);
@@ -1095,6 +1126,20 @@ __global__ void __launch_bounds__(384, 1) tc_dmin2_kernel(TcArgs a) {
             unsigned long long namb = 0;
             bool emitted = false, ovf = false;
             int cbase = 0;
+            auto emit = [&](uint32_t und, int col) {
+                while (und && !ovf) {
+                    const int64_t ci = (int64_t)col + __ffs(und) - 1;
+                    und &= und - 1;
+                    if (ci >= a.kc) break;
+                    const unsigned long long slot = atomicAdd(a.npairs, 1ull);
+                    if (slot < (unsigned long long)a.pcap)
+                        a.pairs[slot] = make_uint2((uint32_t)pi, (uint32_t)ci);
+                    else
+                        ovf = true;
+                    emitted = true;
+                    ++namb;
+                }
+            };
             auto chunk = [&](const uint32_t(&r)[32], int c0) {
                 if (MODE == 0) {
 #pragma unroll
@@ -1111,31 +1156,20 @@ __global__ void __launch_bounds__(384, 1) tc_dmin2_kernel(TcArgs a) {
                         m0 = max3f(m0, __uint_as_float(r[q]), __uint_as_float(r[q + 1]));
                         m1 = max3f(m1, __uint_as_float(r[q + 2]), __uint_as_float(r[q + 3]));
                     }
-                    if (fmaxf(m0, m1) >= vhi) {
+                    const float mx = fmaxf(m0, m1);
+                    if (mx >= vlo) {
+                        removed = true;
+                    } else if (mx >= vhi) {   // undecided columns, as in tc_dmin_kernel
+                        uint32_t und = 0;
 #pragma unroll
-                        for (int q = 0; q < 32; ++q) {
-                            const float v = __uint_as_float(r[q]);
-                            if (v >= vhi && !removed) {
-                                if (v >= vlo) {
-                                    removed = true;
-                                } else if (!ovf) {
-                                    const int64_t ci = (int64_t)cbase + c0 + q;
-                                    if (ci < a.kc) {
-                                        const unsigned long long slot = atomicAdd(a.npairs, 1ull);
-                                        if (slot < (unsigned long long)a.pcap)
-                                            a.pairs[slot] = make_uint2((uint32_t)pi, (uint32_t)ci);
-                                        else
-                                            ovf = true;
-                                        emitted = true;
-                                        ++namb;
-                                    }
-                                }
-                            }
-                        }
+                        for (int q = 0; q < 32; ++q) und |= __uint_as_float(r[q]) >= vhi ? 1u << q : 0u;
+                        emit(und, cbase + c0);
                     }
                 }
             };
-            for (int t = 0; t < a.ntiles; ++t) {
+            const PairTiles ptl(a, pp);
+            for (int li = 0; li < ptl.count; ++li) {
+                const int t = ptl[li];
                 if (!__all_sync(0xFFFFFFFFu, mbar_wait(&t_full[j], tuse & 1u, abort))) {
                     set_status(a.st, KC_ERR_TIMEOUT, 10, t);
                     *abort = 1;
@@ -1347,14 +1381,16 @@ __device__ __forceinline__ float row_dist(const float *__restrict__ x, const flo
 // Exact check of the deferred pairs: hit[row] once a pair is within the
 // threshold (canonical FP32 distance, the same test as the CUDA-core prune).
 __global__ void tc_pair_kernel(const float *__restrict__ src, int d, bool v4, const uint32_t *__restrict__ R,
-                               const float *__restrict__ cen, const uint2 *__restrict__ pairs,
-                               const unsigned long long *npairs, int64_t pcap, const uint32_t *thr, uint8_t *hit) {
+                               const float *__restrict__ cen, const uint32_t *__restrict__ cidx,
+                               const uint2 *__restrict__ pairs, const unsigned long long *npairs, int64_t pcap,
+                               const uint32_t *thr, uint8_t *hit) {
     const int64_t np = (int64_t)min(*npairs, (unsigned long long)pcap);
     const uint32_t T = *thr;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
         const uint2 p = pairs[i];
         if (hit[p.x]) continue;
-        const float acc = row_dist(src + (int64_t)R[p.x] * d, cen + (int64_t)p.y * d, d, v4);
+        const float acc = row_dist(src + (int64_t)R[p.x] * d, cidx ? src + (int64_t)cidx[p.y] * d : cen + (int64_t)p.y * d,
+                                   d, v4);
         if (__float_as_uint(acc) <= T) hit[p.x] = 1;
     }
 }
@@ -1363,7 +1399,8 @@ __global__ void tc_pair_kernel(const float *__restrict__ src, int d, bool v4, co
 // scanned against every center (one warp, lanes over centers); the rest are
 // kept.
 __global__ void tc_resolve_kernel(const float *__restrict__ src, int d, bool v4, const uint32_t *__restrict__ R,
-                                  const float *__restrict__ cen, int64_t sn, const uint32_t *__restrict__ pend,
+                                  const float *__restrict__ cen, const uint32_t *__restrict__ cidx, int64_t sn,
+                                  const uint32_t *__restrict__ pend,
                                   const unsigned long long *npend, const uint8_t *__restrict__ flag,
                                   const uint8_t *__restrict__ hit, const uint32_t *thr, uint32_t *Rn,
                                   unsigned long long *rnn) {
@@ -1378,7 +1415,9 @@ __global__ void tc_resolve_kernel(const float *__restrict__ src, int d, bool v4,
         if (!rm && (flag[pi] & 2)) {
             for (int64_t cb = 0; cb < sn && !rm; cb += 32) {
                 const int64_t ci = cb + lane;
-                const bool h = ci < sn && __float_as_uint(row_dist(src + gx * d, cen + ci * d, d, v4)) <= T;
+                const bool in = ci < sn && (!cidx || cidx[ci] != 0xFFFFFFFFu);
+                const float *c = in && cidx ? src + (int64_t)cidx[ci] * d : cen + ci * d;
+                const bool h = in && __float_as_uint(row_dist(src + gx * d, c, d, v4)) <= T;
                 rm = __any_sync(0xFFFFFFFFu, h);
             }
         }
@@ -1480,9 +1519,10 @@ cudaError_t launch_tc_absmax(const float *pk, int64_t n, int d, unsigned *absmax
 }
 
 cudaError_t launch_tc_centers(const float *cen_rows, const int32_t *kc_dev, int64_t kc, int d, const unsigned *absmax,
-                              void *bt, float *cn, float *ce, unsigned *maxes, cudaStream_t s) {
+                              void *bt, float *cn, float *ce, unsigned *maxes, cudaStream_t s,
+                              const uint32_t *idx = nullptr) {
     cudaMemsetAsync(maxes, 0, 3 * sizeof(unsigned), s);
-    return rows<TC_N>(nullptr, cen_rows, nullptr, kc_dev, kc, d, absmax, bt, cn, ce, maxes, s);
+    return rows<TC_N>(nullptr, cen_rows, idx, kc_dev, kc, d, absmax, bt, cn, ce, maxes, s);
 }
 
 cudaError_t launch_tc_points(const float *pk, const float *rm, const uint32_t *idx, int64_t n, int d,
@@ -1568,13 +1608,25 @@ cudaError_t launch_tc_radius(const float *pk, const float *rm, int64_t n, int d,
     return cudaGetLastError();
 }
 
+bool tc_prune_pairs(int d, int64_t sn) {
+    TcArgs a{};
+    a.kp = kpad(d);
+    a.ntiles = tc_center_tiles(sn);
+    tc_smem_for(a);
+    return !a.resident && tc_pair_smem(a.kp) != 0;
+}
+
 cudaError_t launch_tc_prune(const float *src, int d, const uint32_t *R, int64_t rn, const uint8_t *inS, const float *Scen,
                             int64_t sn, const TcBufs &B, const PruneBufs &P, const uint32_t *thr, uint32_t *Rn,
-                            unsigned long long *rnn, DevStatus *st, cudaStream_t s) {
+                            unsigned long long *rnn, DevStatus *st, cudaStream_t s, const TcCells *cells) {
     cudaError_t e;
+    if (cells) R = cells->R->idx;
+    const uint32_t *cidx = cells ? cells->S->idx : nullptr;
     if ((e = launch_tc_points(nullptr, src, R, rn, d, B.absmax, B.at, B.an, B.ae, s, inS, B.rin)) != cudaSuccess)
         return e;
-    if ((e = launch_tc_centers(Scen, nullptr, sn, d, B.absmax, B.bt, B.cn, B.ce, B.maxes, s)) != cudaSuccess) return e;
+    if ((e = launch_tc_centers(cells ? src : Scen, nullptr, sn, d, B.absmax, B.bt, B.cn, B.ce, B.maxes, s, cidx)) !=
+        cudaSuccess)
+        return e;
     cudaMemsetAsync(P.npairs, 0, sizeof(unsigned long long), s);
     cudaMemsetAsync(P.npend, 0, sizeof(unsigned long long), s);
     cudaMemsetAsync(P.hit, 0, (size_t)rn, s);
@@ -1604,11 +1656,19 @@ cudaError_t launch_tc_prune(const float *src, int d, const uint32_t *R, int64_t 
     a.pflag = P.flag;
     a.pend = P.pend;
     a.npend = P.npend;
+    if (cells) {
+        a.rstart = cells->R->start;
+        a.P = cells->P;
+        a.tiles = cells->tiles;
+        a.ntile = cells->ntile;
+        a.tcap = cells->tcap;
+    }
     a.st = st;
     const size_t smem = tc_smem_for(a);
     const int64_t tiles = (rn + TC_M - 1) / TC_M;
     if (tiles == 0) return cudaGetLastError();
     const size_t smem2 = a.resident ? 0 : tc_pair_smem(a.kp);
+    if (cells && !smem2) return cudaErrorInvalidValue;
     if (smem2) {
         // streamed centers: two point tiles per center tile
         if ((e = launch_dmin2<1>(a, smem2, s)) != cudaSuccess) return e;
@@ -1619,10 +1679,10 @@ cudaError_t launch_tc_prune(const float *src, int d, const uint32_t *R, int64_t 
         const int grid = (int)std::min<int64_t>(tiles, (int64_t)sms());
         tc_dmin_kernel<1><<<grid, TC_THREADS, smem, s>>>(a);
     }
-    const bool v4 = (d & 3) == 0 && ((uintptr_t)src & 15) == 0 && ((uintptr_t)Scen & 15) == 0;
+    const bool v4 = (d & 3) == 0 && ((uintptr_t)src & 15) == 0 && (cells || ((uintptr_t)Scen & 15) == 0);
     const int g2 = sms() * 8;
-    tc_pair_kernel<<<g2, 256, 0, s>>>(src, d, v4, R, Scen, P.pairs, P.npairs, P.pcap, thr, P.hit);
-    tc_resolve_kernel<<<g2, 256, 0, s>>>(src, d, v4, R, Scen, sn, P.pend, P.npend, P.flag, P.hit, thr, Rn, rnn);
+    tc_pair_kernel<<<g2, 256, 0, s>>>(src, d, v4, R, Scen, cidx, P.pairs, P.npairs, P.pcap, thr, P.hit);
+    tc_resolve_kernel<<<g2, 256, 0, s>>>(src, d, v4, R, Scen, cidx, sn, P.pend, P.npend, P.flag, P.hit, thr, Rn, rnn);
     note_launches(3);
     return cudaGetLastError();
 }
