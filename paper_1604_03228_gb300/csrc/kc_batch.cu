@@ -127,7 +127,7 @@ __global__ void batch_radius_kernel(const GonInst *__restrict__ insts, int ninst
         const int d = I.d;
         const int kc = *I.k_out;
         const T *pk = (const T *)I.pk;
-        const double thr = (double)__uint_as_float(key_val(K)) * (1.0 - 3.0 * f32_gamma(d));
+        const float thr = reach_threshold(__uint_as_float(key_val(K)), d);
         const float opg = __fadd_ru(1.f, lp_slack(d));
         const float ecmax = I.lp_kind ? *I.ecmax_out : 0.f;
         double best = -1.0;
@@ -138,9 +138,9 @@ __global__ void batch_radius_kernel(const GonInst *__restrict__ insts, int ninst
                 if (I.lp_kind) {
                     const uint32_t hi = ((uint32_t)reinterpret_cast<const uint16_t *>(I.mind)[I.lo + x] + 1u) << 16;
                     const float U = lp_upper(hi, __fadd_ru(I.eblk[(I.lo + x) / BLK], ecmax), opg);
-                    flag = (double)U * (double)U >= thr;
+                    flag = __fmul_ru(U, U) >= thr;
                 } else {
-                    flag = (double)__uint_as_float(I.mind[I.lo + x]) >= thr;
+                    flag = __uint_as_float(I.mind[I.lo + x]) >= thr;
                 }
             }
             unsigned todo = __ballot_sync(0xFFFFFFFFu, flag);
@@ -148,9 +148,23 @@ __global__ void batch_radius_kernel(const GonInst *__restrict__ insts, int ninst
                 const int src = __ffs(todo) - 1;
                 todo &= todo - 1;
                 const int64_t xs = base + src;
+                // canonical FP32 distances first: FP64 only for the centers that
+                // can be the FP64 minimum
+                auto d32 = [&](int64_t c) {
+                    float acc = 0.f;
+#pragma unroll 8
+                    for (int j = 0; j < d; ++j)
+                        acc = sq_step(acc, pk[pk_index(I.lo + xs, j, d)], pk[pk_index(I.lo + c, j, d)]);
+                    return acc;
+                };
+                uint32_t m32 = 0xFFFFFFFFu;
+                for (int ci = lane; ci < kc; ci += 32) m32 = min(m32, __float_as_uint(d32(I.centers[ci] - I.base)));
+                m32 = __reduce_min_sync(0xFFFFFFFFu, m32);
+                const float lim = min64_limit(__uint_as_float(m32), d);
                 double mm = INFINITY;
                 for (int ci = lane; ci < kc; ci += 32) {
                     const int64_t c = I.centers[ci] - I.base;
+                    if (d32(c) > lim) continue;
                     double s = 0.0;
                     for (int j = 0; j < d; ++j)
                         s = sq_step64(s, pk[pk_index(I.lo + xs, j, d)], pk[pk_index(I.lo + c, j, d)]);

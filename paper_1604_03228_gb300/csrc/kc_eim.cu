@@ -11,6 +11,7 @@
 //   prune     x stays in R only if d(x, S) > thr (equal is removed, Section
 //             4.1); the scan over S stops at the first center within thr
 // and at the end C = S u R is compacted in ascending index order.
+#include <cmath>
 #include <type_traits>
 
 #include "kc_internal.cuh"
@@ -28,13 +29,13 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     return z ^ (z >> 31);
 }
 
-// U(seed, it, x, stream) in [0, 1): splitmix64 output number (counter + 1) of
-// the stream with state `seed`, counter = it << 33 | x << 1 | stream, top 53
-// bits scaled by 2^-53 (exact in double).
-__device__ __forceinline__ double eim_uniform(uint64_t seed, uint64_t it, uint64_t x, uint64_t stream) {
+// U(seed, it, x, stream) in [0, 1) is the top 53 bits of splitmix64 output
+// number (counter + 1) of the stream with state `seed`, counter = it << 33 |
+// x << 1 | stream, scaled by 2^-53.  U < p is decided on the 53 bits as an
+// integer below ceil(p 2^53) (exact, and no FP64, which is slow here).
+__device__ __forceinline__ uint64_t eim_bits(uint64_t seed, uint64_t it, uint64_t x, uint64_t stream) {
     const uint64_t ctr = (it << 33) | (x << 1) | stream;
-    const uint64_t h = mix64(seed + (ctr + 1ull) * 0x9E3779B97F4A7C15ull);
-    return (double)(h >> 11) * 0x1p-53;
+    return mix64(seed + (ctr + 1ull) * 0x9E3779B97F4A7C15ull) >> 11;
 }
 
 __global__ void iota_kernel(uint32_t *R, int64_t n) {
@@ -42,17 +43,17 @@ __global__ void iota_kernel(uint32_t *R, int64_t n) {
         R[i] = (uint32_t)i;
 }
 
-__global__ void sample_kernel(const uint32_t *__restrict__ R, int64_t rn, uint64_t seed, int it, double pS,
-                              double pH, uint8_t *__restrict__ inS, uint32_t *__restrict__ S,
+__global__ void sample_kernel(const uint32_t *__restrict__ R, int64_t rn, uint64_t seed, int it, uint64_t tS,
+                              uint64_t tH, uint8_t *__restrict__ inS, uint32_t *__restrict__ S,
                               unsigned long long *sn, uint32_t *__restrict__ H, unsigned long long *hn,
                               int64_t hcap, DevStatus *st) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rn; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t x = R[i];
-        if (eim_uniform(seed, (uint64_t)it, x, 0) < pS) {
+        if (eim_bits(seed, (uint64_t)it, x, 0) < tS) {
             inS[x] = 1;
             S[atomicAdd(sn, 1ull)] = x;
         }
-        if (eim_uniform(seed, (uint64_t)it, x, 1) < pH) {
+        if (eim_bits(seed, (uint64_t)it, x, 1) < tH) {
             const unsigned long long pos = atomicAdd(hn, 1ull);
             if ((int64_t)pos < hcap) H[pos] = x;
             else set_status(st, KC_ERR_OOM, 5, (int64_t)pos);
@@ -309,7 +310,7 @@ cudaError_t launch_eim_iota(uint32_t *R, int64_t n, cudaStream_t s) {
 cudaError_t launch_eim_sample(const uint32_t *R, int64_t rn, uint64_t seed, int it, double pS, double pH,
                               uint8_t *inS, uint32_t *S, unsigned long long *sn, uint32_t *H, unsigned long long *hn,
                               int64_t hcap, DevStatus *st, cudaStream_t s) {
-    sample_kernel<<<grid_for(rn, 256), 256, 0, s>>>(R, rn, seed, it, pS, pH, inS, S, sn, H, hn, hcap, st);
+    sample_kernel<<<grid_for(rn, 256), 256, 0, s>>>(R, rn, seed, it, (uint64_t)ceil(pS * 0x1p53), (uint64_t)ceil(pH * 0x1p53), inS, S, sn, H, hn, hcap, st);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -196,6 +196,26 @@ __host__ __device__ inline double f32_gamma(int d) {
     return m / (1.0 - m);
 }
 
+// The same bound and what is derived from it in FP32, rounded to the safe side:
+// FP64 is slow on this part (its 40-odd instructions per thread, a division
+// among them, were half of a recheck launch on 1M points).
+__host__ __device__ inline float f32_gamma_up(int d) {   // >= f32_gamma(d)
+    const float m = (float)(d + 2) * 5.9604644775390625e-08f;
+    return m * (1.f + 4.f * m) * 1.000001f;   // m / (1 - m) <= m (1 + 4 m) for m <= 3/4
+}
+// Lower end of the canonical minima that can reach the FP64 maximum behind a
+// largest canonical minimum M32: M32 (1 - 3 gamma).
+__device__ __forceinline__ float reach_threshold(float M32, int d) {
+    return __fmul_rd(M32, fmaxf(__fsub_rd(1.f, __fmul_ru(3.f, f32_gamma_up(d))), 0.f));
+}
+// Canonical distances above this cannot be the FP64 minimum of a point whose
+// canonical minimum is m32: m32 (1 + gamma) / (1 - gamma), and FP64's own
+// rounding, far below the factor's 2^-22.
+__device__ __forceinline__ float min64_limit(float m32, int d) {
+    const float g = f32_gamma_up(d);
+    return __fmul_ru(m32, __fadd_ru(__fdiv_ru(__fadd_ru(1.f, g), __fsub_rd(1.f, g)), 0x1p-22f));
+}
+
 // --------------------------------------------------------- launchers
 // Every launcher reports the number of kernels it launched (tracing and the
 // process-wide launch counter).
@@ -416,7 +436,7 @@ __device__ __forceinline__ float lp_lower(uint32_t mbits, float delta, float omg
     const float r = __fsqrt_rd(__uint_as_float(mbits));
     return __fmul_rd(omg, __fsub_rd(__fmul_rd(r, omg), delta));
 }
-__host__ __device__ inline float lp_slack(int d) { return (float)(f32_gamma(d) + 0x1p-20); }
+__host__ __device__ inline float lp_slack(int d) { return f32_gamma_up(d) + 0x1.00001p-20f; }
 
 // --------------------------------------------- low-precision sweep data
 // Coordinates per 32-bit word of the low-precision copy (bf16, fp16: 2;

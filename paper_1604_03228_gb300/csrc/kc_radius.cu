@@ -185,23 +185,22 @@ __global__ void __launch_bounds__(RAD_NT) radius_min_generic_kernel(
     if ((threadIdx.x & 31) == 0 && best) atomicMax(key32, (unsigned long long)best);
 }
 
-__device__ __forceinline__ double flag_threshold(const unsigned long long *key32, int d) {
-    const float M32 = __uint_as_float(key_val(*key32));
-    return (double)M32 * (1.0 - 3.0 * f32_gamma(d));
+__device__ __forceinline__ float flag_threshold(const unsigned long long *key32, int d) {
+    return reach_threshold(__uint_as_float(key_val(*key32)), d);
 }
 
 // Can point x reach the FP64 maximum?  FP32 minima: m32(x) >= thr.  After a
 // mixed-precision sweep mind holds approximate minima m~; then U(x)^2 >= thr
 // with U(x) >= sqrt of the exact minimum (kc_gon.cu), which also bounds the
 // FP64 value within the same (1 - 3 gamma) margin.
-__device__ __forceinline__ bool can_reach(const uint32_t *mind, int64_t x, double thr, const float *eblk,
-                                          const float *ecmax, float opg, double sc) {
-    if (!eblk) return (double)__uint_as_float(mind[x]) >= thr;
+__device__ __forceinline__ bool can_reach(const uint32_t *mind, int64_t x, float thr, const float *eblk,
+                                          const float *ecmax, float opg, float sc) {
+    if (!eblk) return __uint_as_float(mind[x]) >= thr;
     // mixed precision: 16-bit truncated codes, upper end of the code's
-    // interval; sc: the fp16 sweep's power-of-two unit (exact in double)
+    // interval; sc: the fp16 sweep's power-of-two unit
     const uint32_t hi = ((uint32_t)reinterpret_cast<const uint16_t *>(mind)[x] + 1u) << 16;
-    const double U = (double)lp_upper(hi, __fadd_ru(eblk[x / BLK], *ecmax), opg) * sc;
-    return U * U >= thr;
+    const float U = __fmul_ru(lp_upper(hi, __fadd_ru(eblk[x / BLK], *ecmax), opg), sc);
+    return __fmul_ru(U, U) >= thr;
 }
 
 // FP64 minimum over all centers of point x, computed by the whole warp (lane
@@ -222,12 +221,11 @@ __device__ double min64_warp(const float *__restrict__ pk, const float *__restri
 #pragma unroll
         for (int o = 16; o; o >>= 1) m32 = min(m32, __shfl_xor_sync(0xFFFFFFFFu, m32, o));
     }
-    const double g = f32_gamma(d);
-    const double lim = (double)__uint_as_float(m32) * ((1.0 + g) / (1.0 - g)) * (1.0 + 4.0 * (d + 2) * 0x1p-53);
+    const float lim = min64_limit(__uint_as_float(m32), d);
     double m = INFINITY;
     for (int ci = lane; ci < kc; ci += 32) {
         const float s = point_row_dist(pk, rm, x, d, cen + (int64_t)ci * d, v4);
-        if ((double)s > lim) continue;
+        if (s > lim) continue;
         double s64 = 0.0;
         for (int j = 0; j < d; ++j) s64 = sq_step64(s64, point_at(pk, rm, x, j, d), cen[(int64_t)ci * d + j]);
         m = fmin(m, s64);
@@ -249,9 +247,9 @@ __global__ void recheck_max_kernel(const float *__restrict__ pk, const float *__
                                    const uint32_t *__restrict__ list, const unsigned long long *lcount) {
     if (ld_volatile_i32(&st->code) != 0) return;
     if (key_val(*key32) == 0) return;   // every minimum is exactly 0
-    const double sc = lpscale ? (double)*lpscale : 1.0;
+    const float sc = lpscale ? *lpscale : 1.f;
     const int kc = (int)dev_count(kc_dev, kc_max);
-    const double thr = flag_threshold(key32, d);
+    const float thr = flag_threshold(key32, d);
     const float opg = __fadd_ru(1.f, lp_slack(d));
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -285,8 +283,8 @@ __global__ void recheck_arg_kernel(int64_t n, int d, const uint32_t *__restrict_
                                    const unsigned long long *lcount) {
     if (ld_volatile_i32(&st->code) != 0) return;
     if (key_val(*key32) == 0) return;
-    const double sc = lpscale ? (double)*lpscale : 1.0;
-    const double thr = flag_threshold(key32, d);
+    const float sc = lpscale ? *lpscale : 1.f;
+    const float thr = flag_threshold(key32, d);
     const float opg = __fadd_ru(1.f, lp_slack(d));
     const double M = __longlong_as_double((long long)*max64);
     const int64_t cnt = list ? (int64_t)*lcount : n;
@@ -320,9 +318,9 @@ __global__ void __launch_bounds__(256) recheck_kernel(
         lpscale = nullptr;
     }
     if (run) {
-        const double sc = lpscale ? (double)*lpscale : 1.0;
+        const float sc = lpscale ? *lpscale : 1.f;
         const int kc = (int)dev_count(kc_dev, kc_max);
-        const double thr = flag_threshold(key32, d);
+        const float thr = flag_threshold(key32, d);
         const float opg = __fadd_ru(1.f, lp_slack(d));
         const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
         const int64_t cnt = list ? (int64_t)*lcount : n;

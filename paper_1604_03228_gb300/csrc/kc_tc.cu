@@ -589,7 +589,7 @@ struct PairTiles {
 };
 
 __device__ __forceinline__ float tc_eta(int d, int kp) {
-    return (float)(f32_gamma(d) + (double)(kp + 16) * 0x1p-21 + 0x1p-21);
+    return __fmul_ru(__fadd_ru(f32_gamma_up(d), (float)(kp + 17) * 0x1p-21f), 1.000001f);
 }
 
 // Launch bounds of 384 threads for a 320-thread launch: they cap the
@@ -1264,7 +1264,7 @@ __global__ void tc_flag_kernel(int64_t n, int d, const float *__restrict__ mhi, 
                                uint32_t *__restrict__ mind, uint32_t *__restrict__ flist,
                                unsigned long long *fcount, const DevStatus *st) {
     if (ld_volatile_i32(&st->code) != 0) return;
-    const double T = (double)__uint_as_float(*mlo_max) * (1.0 - 3.0 * f32_gamma(d));
+    const float T = reach_threshold(__uint_as_float(*mlo_max), d);
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     // a warp takes 128 consecutive points per pass, four loads in flight
@@ -1279,7 +1279,7 @@ __global__ void tc_flag_kernel(int64_t n, int d, const float *__restrict__ mhi, 
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int64_t x = base + 32 * q + lane;
-            const bool flag = x < n && (double)h[q] >= T;
+            const bool flag = x < n && h[q] >= T;
             if (x < n) mind[x] = flag ? 0xFFFFFFFFu : 0u;
             const unsigned b = __ballot_sync(0xFFFFFFFFu, flag);
             if (!b) continue;
