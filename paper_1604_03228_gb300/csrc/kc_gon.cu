@@ -184,6 +184,14 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
     __syncthreads();
     const bool claim = DYN && NT == GROUP_NT && (I.lo + I.n - 1) / BLK - I.lo / BLK + 1 >= 4 * (int64_t)G * W;
     const bool tail = DYN && G > 1 && I.tail != nullptr;
+    // Through the leader while a step's sweep is short, fewer than four blocks
+    // a warp: behind longer ones the CTAs arrive apart, do not slow each other's
+    // polling, and the leader's second hop is what shows (int32 6.4M x 55,
+    // 230 us a step: 1% slower; float 8M x 64: 0.7%).  Not between queue CTAs,
+    // which share their SM with other groups: nothing gained, and the sweep's
+    // code grew (MRG round 1 on 10M x 16 20.2 -> 20.7 ms).
+    const bool lead = NT == GROUP_NT && !DYN && G > LEADER_MIN && I.bc != nullptr &&
+                      (I.lo + I.n - 1) / BLK - I.lo / BLK + 1 < 4 * (int64_t)G * W;
 
     int it;
     uint64_t K = 0;
@@ -204,10 +212,6 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
             uint64_t g = v;
             bool ab = false;
             const bool more = it + 1 < I.it1;
-            // (queue CTAs share their SM with other groups; there the leader
-            // gained nothing and the sweep's code grew: MRG round 1 on 10M x 16
-            // 20.2 -> 20.7 ms)
-            const bool lead = NT == GROUP_NT && G > LEADER_MIN && I.bc != nullptr;
             const uint64_t tagw = (uint64_t)(it + 1) << 32;
             if (G > 1) {
                 uint64_t *row = I.slots + (int64_t)it * slot_stride(G);
