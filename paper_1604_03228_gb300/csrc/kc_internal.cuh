@@ -476,6 +476,17 @@ struct PackSeg {
     int32_t d;
     int32_t pad;
 };
+// Segment of block gb: the last of segs[0, nseg) with blk0 <= gb.
+template <typename Seg>
+__device__ __forceinline__ int find_seg(const Seg *segs, int nseg, int64_t gb) {
+    int lo = 0, hi = nseg - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (segs[mid].blk0 <= gb) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
 cudaError_t launch_pack_many(const PackSeg *segs, int nseg, int64_t total_blocks, int dtype, DevStatus *st,
                              cudaStream_t s);
 cudaError_t launch_mrg_union(const int64_t *c1, const int32_t *k1, int m, int k, int64_t *U, int64_t *nU,

@@ -164,22 +164,24 @@ __global__ void __launch_bounds__(BLK) lp_pack_kernel(const float *__restrict__ 
 }
 
 // bf16 copies of many packed arrays in one launch (segment s owns blocks
-// [blk0, blk0 + nblocks(n)) of the launch).
+// [blk0, blk0 + nblocks(n)) of the launch); a CTA takes a contiguous run of
+// blocks and looks for its segment once, as pack_many_kernel does (154M points
+// of d 3, 8 and 32 in 4096 arrays, both packs: 11.6 -> 7.7 ms).
 __global__ void __launch_bounds__(BLK) lp_pack_many_kernel(const LpSeg *__restrict__ segs, int nseg,
                                                            int64_t total_blocks) {
     __shared__ LpSeg S;
-    for (int64_t gb = blockIdx.x; gb < total_blocks; gb += gridDim.x) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int lo = 0, hi = nseg - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (segs[mid].blk0 <= gb) lo = mid;
-                else hi = mid - 1;
-            }
-            S = segs[lo];
+    const int64_t per = (total_blocks + gridDim.x - 1) / gridDim.x;
+    const int64_t g0 = per * blockIdx.x, g1 = min(total_blocks, g0 + per);
+    int seg = 0;
+    int64_t send = g0;   // first block past the current segment
+    for (int64_t gb = g0; gb < g1; ++gb) {
+        if (gb >= send) {
+            __syncthreads();
+            seg = gb == g0 ? find_seg(segs, nseg, gb) : seg + 1;
+            if (threadIdx.x == 0) S = segs[seg];
+            __syncthreads();
+            send = S.blk0 + nblocks(S.n);
         }
-        __syncthreads();
         lp_pack_block<KC_SWEEP_BF16>(S.pk, S.n, S.d, nullptr, S.lp, S.ept, S.eblk, S.stamp, gb - S.blk0);
     }
 }
@@ -190,7 +192,7 @@ cudaError_t launch_lp_pack_many(const LpSeg *segs, int nseg, int64_t total_block
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = (int)(total_blocks < (int64_t)sms * 16 ? total_blocks : (int64_t)sms * 16);
+    const int grid = (int)(total_blocks < (int64_t)sms * 64 ? total_blocks : (int64_t)sms * 64);
     lp_pack_many_kernel<<<grid, BLK, 0, s>>>(segs, nseg, total_blocks);
     note_launches(1);
     return cudaGetLastError();
