@@ -266,9 +266,12 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
  * are [count] arrays in host or device memory.
  * Launch shape: instances are ordered longest-first by modelled work
  * n k (d b + 8) bytes (b = 4 for FP32, 2 for the bf16 sweep).  An instance
- * whose work exceeds theta times the fair share of one resident CTA is solved
- * by a group of CTAs sized to its work (cooperative launch); the others go
- * through a queue, one CTA each, longest first.  theta is 1 by default; with
+ * whose work exceeds the fair share of one resident CTA (FP32: or whose points
+ * exceed its part of the L2 cache) is solved by a group of CTAs (cooperative
+ * launch), and groups solve further instances one after another; the others go
+ * through a queue, one CTA each, longest first.  With KC_BATCH_THETA or
+ * KC_AUTOTUNE each group solves one instance: those whose work exceeds theta
+ * times the fair share, as long as half of the CTAs suffice.  With
  * KC_AUTOTUNE in opts->flags the first call for a batch shape (count, dtype,
  * sweep and every (n, d, k)) solves the batch once per candidate theta
  * (plain queue, 4, 2, 1, 0.5), keeps the fastest for later calls in the
@@ -300,8 +303,9 @@ kc_status kc_gonzalez_batch(int32_t count, const void *const *pts, const int64_t
  * must not overlap (they share scratch): order them on one stream.
  * kc_batch_plan_wait waits for the last run and returns its device status
  * (KC_ERR_RANGE, KC_ERR_NONFINITE, KC_ERR_TIMEOUT as kc_gonzalez).
- * kc_batch_plan_info reports the chosen theta, the number of group-solved
- * instances, their CTAs, and the grid size.
+ * kc_batch_plan_info reports the chosen theta (1 if none was set or timed),
+ * the number of group-solved instances, the CTAs of their groups (the first
+ * ones of the grid), and the grid size.
  * kc_batch_plan_destroy waits for the last run and frees the plan (NULL is
  * accepted).
  */

@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <queue>
 #include <mutex>
 #include <string>
 #include <utility>
@@ -1164,7 +1165,7 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
             cta += I.G;
         }
     }
-    GonInst proto;
+    GonInst proto{};
     memset(&proto, 0, sizeof proto);
     proto.pk = Lo.pkU;
     proto.mind = Lo.mindU;
@@ -1755,14 +1756,34 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
 //
 // Launch policy.  Instances are ordered longest-first by modelled work
 // w = n k (d b + 8) bytes (b bytes per streamed coordinate, the running
-// minimum read and written).  With S resident queue-mode CTAs and the fair
-// share W / S of the total work W, an instance with w > theta W / S is heavy:
-// it is solved by a CTA group of G = ceil(w / (W / S)) CTAs (at most one per
-// warp's worth of 128-point blocks) at the front of a cooperative grid, while
-// the groups take at most half of the CTAs.  The other instances go through
-// the queue longest-first, and group CTAs join the queue when their instance
-// is done.  theta = +inf is the plain queue.  KC_AUTOTUNE times every theta
-// of kThetas on the batch itself and keeps the fastest per batch shape.
+// minimum read and written); W is the total, S the resident queue-mode CTAs.
+//
+// By default an instance whose work exceeds the fair share W / S is solved by
+// a CTA group of the power of two above w / (W / S), and with the FP32 sweep
+// also one that exceeds a CTA's part of L2: its group is then the power of two
+// whose parts hold it, so the instances in flight stay in L2 from step to
+// step (at most one CTA per warp's worth of 128-point blocks).  The groups'
+// lists are laid out on the host; the rest goes through the queue
+// longest-first, which the CTAs join when their list is done.  If groups of
+// any size fit side by side they are not rounded and all start at once.  Batches
+// whose slots would take much scratch use the one-level split below, theta 1.
+// Before, instances above the share took groups of the first half of the CTAs
+// once, and what did not fit there was left to single CTAs.  Measured on
+// mixed batches (d 3, 8, 32; k 8 to 128; GON launch alone, before / now, ms):
+//   instances x points         FP32           bf16
+//   4096 x 1k..200k          87.6 / 60.6    62.4 / 62.5
+//    512 x 1k..200k          17.8 /  8.2    25.4 / 13.4
+//     69 x 1k..200k           6.2 /  1.9    13.9 /  2.8
+//    905 x 1k..20k            2.6 /  1.9     3.9 /  3.2
+// bf16 does not group by L2: it is issue-bound, with two exchanges a step
+// (4096: 62.5 -> 83 ms).
+//
+// KC_BATCH_THETA and KC_AUTOTUNE take the one-level split instead: an instance
+// with w > theta W / S is heavy and solved by a CTA group of
+// G = ceil(w / (W / S)) CTAs at the front of a cooperative grid, while the
+// groups take at most half of the CTAs; the others go through the queue.
+// theta = +inf is the plain queue.  KC_AUTOTUNE times every theta of kThetas
+// on the batch itself and keeps the fastest per batch shape.
 namespace {
 
 constexpr double kThetaQueue = 1e300;
@@ -1773,11 +1794,105 @@ struct BatchShape {
     int count = 0, dtype = 0, lp = 0, dc = 0, dmax = 0;
     std::vector<int> order;   // descriptor position -> instance
     std::vector<int> G;       // CTAs per descriptor position (1: queue)
+    std::vector<int> cta0;    // first CTA of each descriptor position's group
+    bool teams = false;       // groups solve several instances, one after another
     int nheavy = 0, gheavy = 0, grid = 0;
     double theta = kThetaQueue;
 };
 
-void batch_policy(BatchShape &b, const int64_t *n, const int32_t *d, const int32_t *k, double theta) {
+int pow2_floor(int64_t v) {
+    int64_t p = 1;
+    while (2 * p <= v) p *= 2;
+    return (int)p;
+}
+
+void batch_teams(BatchShape &b, const int64_t *n, const int32_t *k, const std::vector<double> &w,
+                 const std::vector<int> &lpt, int slots, double share) {
+    int dev = 0, l2 = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+    const double part = b.lp ? 0.0 : (double)l2 / slots;   // a CTA's part of L2 (0: not a criterion)
+    std::vector<int> size((size_t)b.count);
+    auto fit = [&](int64_t g, int i) {   // at most a block per warp
+        const int64_t W = gon_queue_warps(), gmax = std::min<int64_t>((nblocks(n[i]) + W - 1) / W, slots);
+        return (int)std::max<int64_t>(1, std::min(g, gmax));
+    };
+    auto l2_parts = [&](int i) {
+        return part > 0 ? (int64_t)std::ceil(w[i] / (double)std::min<int64_t>(k[i], n[i]) / part) : (int64_t)1;
+    };
+    auto place = [&](int i, int g, int c) {
+        b.order.push_back(i);
+        b.G.push_back(g);
+        b.cta0.push_back(c);
+        b.gheavy = std::max(b.gheavy, c + g);
+        ++b.nheavy;
+    };
+    // all instances at once, with the largest groups that fit
+    int64_t sum = slots + 1;
+    for (double f = 4.0; f >= 1.0 && sum > slots; f *= 0.5) {
+        sum = 0;
+        for (int i = 0; i < b.count; ++i)
+            sum += size[i] = fit(std::max<int64_t>(l2_parts(i), (int64_t)std::ceil(f * w[i] / share)), i);
+    }
+    if (sum <= slots) {
+        for (int i : lpt)
+            if (size[i] > 1) place(i, size[i], b.gheavy);
+    } else {
+        const int gcap = pow2_floor(slots);
+        for (int i = 0; i < b.count; ++i) {
+            const int64_t parts = l2_parts(i);
+            int64_t g = 1;
+            while (g < gcap && (g < parts || g * share <= w[i])) g *= 2;
+            size[i] = pow2_floor(fit(std::min<int64_t>(g, gcap), i));
+        }
+        // From the largest size down, each instance to the team that is free
+        // first (times in bytes a CTA; a step's exchange as 75 KB).  A team of
+        // one size is the two of half the size side by side, so no CTA waits
+        // for another one between them.
+        using Team = std::pair<double, int>;   // (time its CTAs are free, first CTA)
+        std::vector<double> load((size_t)slots, 0.0);
+        for (int g = gcap; g >= 2; g /= 2) {
+            std::priority_queue<Team, std::vector<Team>, std::greater<Team>> q;
+            for (int c = 0; c + g <= slots; c += g)
+                q.push({*std::max_element(load.begin() + c, load.begin() + c + g), c});
+            bool any = false;
+            for (int i : lpt) {
+                if (size[i] != g) continue;
+                any = true;
+                Team t = q.top();
+                q.pop();
+                place(i, g, t.second);
+                t.first += w[i] / g + 75e3 * (double)std::min<int64_t>(k[i], n[i]);
+                q.push(t);
+            }
+            for (; any && !q.empty(); q.pop())
+                std::fill(load.begin() + q.top().second, load.begin() + q.top().second + g, q.top().first);
+        }
+    }
+    for (int i : lpt)
+        if (size[i] == 1) {
+            b.order.push_back(i);
+            b.G.push_back(1);
+            b.cta0.push_back(0);
+        }
+    const int nlight = b.count - b.nheavy;
+    b.grid = b.nheavy ? std::max(b.gheavy, std::min(slots, b.gheavy + nlight)) : std::min(slots, b.count);
+}
+
+// Whether the groups' exchange slots (8 bytes a step and CTA) stay within a
+// sixteenth of the packed points and 16 MB; with more (k near n) the one-level
+// split, whose groups share half of the CTAs once, keeps to the scratch it took.
+bool slot_room(const BatchShape &b, const int64_t *n, const int32_t *d, const int32_t *k) {
+    double slots = 0, packed = 0;
+    for (int q = 0; q < b.nheavy; ++q) {
+        const int i = b.order[q];
+        slots += 8.0 * (double)slot_words(std::min<int64_t>(k[i], n[i]), b.G[q], b.lp != 0);
+    }
+    for (int i = 0; i < b.count; ++i) packed += 4.0 * (double)n[i] * d[i];
+    return slots <= packed / 16 + 16.0 * 1048576;
+}
+
+void batch_policy(BatchShape &b, const int64_t *n, const int32_t *d, const int32_t *k, double theta, bool teams) {
     const int count = b.count;
     const double bpc = b.lp == KC_SWEEP_BF16 ? 2.0 : 4.0;
     std::vector<double> w((size_t)count);
@@ -1789,12 +1904,23 @@ void batch_policy(BatchShape &b, const int64_t *n, const int32_t *d, const int32
     std::vector<int> lpt((size_t)count);
     for (int i = 0; i < count; ++i) lpt[i] = i;
     std::stable_sort(lpt.begin(), lpt.end(), [&](int a, int c) { return w[a] > w[c]; });
-    const int slots = gon_queue_grid(b.dtype, b.dc, b.lp);
+    const int slots = gon_queue_grid(b.dtype, b.dc, b.lp, b.dmax);
     const double share = W / std::max(1, slots);
     b.order.clear();
     b.G.clear();
+    b.cta0.clear();
     b.nheavy = b.gheavy = 0;
     b.theta = theta;
+    b.teams = teams;
+    if (teams) {
+        batch_teams(b, n, k, w, lpt, slots, share);
+        if (slot_room(b, n, d, k)) return;
+        b.order.clear();
+        b.G.clear();
+        b.cta0.clear();
+        b.nheavy = b.gheavy = 0;
+        b.teams = false;
+    }
     std::vector<char> heavy((size_t)count, 0);
     for (int q = 0; q < count && theta < kThetaQueue; ++q) {
         const int i = lpt[q];
@@ -1806,6 +1932,7 @@ void batch_policy(BatchShape &b, const int64_t *n, const int32_t *d, const int32
         heavy[i] = 1;
         b.order.push_back(i);
         b.G.push_back(g);
+        b.cta0.push_back(b.gheavy);
         b.gheavy += g;
         ++b.nheavy;
     }
@@ -1813,6 +1940,7 @@ void batch_policy(BatchShape &b, const int64_t *n, const int32_t *d, const int32
         if (!heavy[lpt[q]]) {
             b.order.push_back(lpt[q]);
             b.G.push_back(1);
+            b.cta0.push_back(0);
         }
     const int nlight = count - b.nheavy;
     b.grid = b.nheavy ? std::max(b.gheavy, std::min(slots, b.gheavy + nlight)) : std::min(slots, count);
@@ -1860,7 +1988,8 @@ void remember_theta(uint64_t sig, double theta) {
 // The theta for a batch: KC_BATCH_THETA if set ("inf": the plain queue;
 // it also skips tuning), else the tuned one for this shape, else the
 // default.  Returns whether the choice is settled (no tuning needed).
-bool pick_theta(uint64_t sig, double *theta) {
+bool pick_theta(uint64_t sig, double *theta, bool *teams) {
+    *teams = false;
     const char *e = getenv("KC_BATCH_THETA");
     if (e && *e) {
         const double v = strcmp(e, "inf") == 0 ? kThetaQueue : atof(e);
@@ -1868,7 +1997,9 @@ bool pick_theta(uint64_t sig, double *theta) {
         return true;
     }
     *theta = kThetaDefault;
-    return tuned_theta(sig, theta);
+    const bool tuned = tuned_theta(sig, theta);
+    *teams = !tuned;
+    return tuned;
 }
 
 // Device buffers of one batch, carved from one allocation.  The zero region
@@ -1882,7 +2013,8 @@ struct BatchBufs {
         uint32_t *lpw;
         float *ept, *eblk, *cenT, *ecmax;
         uint32_t *m32, *stamp;
-        uint64_t *slots, *bc;
+        uint64_t *slots;
+        int *join;
     };
     std::vector<Per> per;
     int *counter = nullptr;
@@ -1913,7 +2045,7 @@ void batch_layout(Carve &cv, const BatchShape &b, BatchBufs &B, const int64_t *n
     for (int q = 0; q < b.nheavy; ++q) {
         const int i = b.order[q];
         B.per[i].slots = cv.take<uint64_t>((size_t)slot_words(std::min<int64_t>(k[i], n[i]), b.G[q], b.lp != 0));
-        B.per[i].bc = cv.take<uint64_t>((size_t)bc_words(d[i]));
+        B.per[i].join = b.teams ? cv.take<int>(1) : nullptr;
     }
     B.zero_bytes = cv.off;
     B.kout_dev = dev_kout ? k_out : cv.take<int32_t>((size_t)count);
@@ -1955,7 +2087,6 @@ std::vector<char> batch_descriptors(const BatchShape &b, BatchBufs &B, const voi
     GonInst *hg = reinterpret_cast<GonInst *>(host.data() + gi_off);
     LpSeg *hl = reinterpret_cast<LpSeg *>(host.data() + ls_off);
     int64_t blk0 = 0;
-    int cta0 = 0;
     for (int q = 0; q < count; ++q) {
         const int i = b.order[q];
         const BatchBufs::Per &P = B.per[i];
@@ -1982,7 +2113,7 @@ std::vector<char> batch_descriptors(const BatchShape &b, BatchBufs &B, const voi
         I.pk = P.pk;
         I.mind = P.mind;
         I.slots = q < b.nheavy ? P.slots : nullptr;
-        I.bc = q < b.nheavy ? P.bc : nullptr;
+        I.join = q < b.nheavy ? P.join : nullptr;
         I.centers = P.cen;
         I.k_out = B.kout_dev + i;
         I.final_key = B.fkeys + i;
@@ -1995,9 +2126,8 @@ std::vector<char> batch_descriptors(const BatchShape &b, BatchBufs &B, const voi
         I.first = 0;
         I.d = d[i];
         I.k = (int)std::min<int64_t>(k[i], n[i]);
-        I.cta0 = q < b.nheavy ? cta0 : 0;
-        I.G = q < b.nheavy ? b.G[q] : 1;
-        if (q < b.nheavy) cta0 += b.G[q];
+        I.cta0 = b.cta0[q];
+        I.G = b.G[q];
         I.kcap = I.k;
         if (b.lp) {
             I.lp = P.lpw;
@@ -2105,12 +2235,13 @@ kc_status kc_gonzalez_batch(int32_t count, const void *const *pts, const int64_t
     if (tune && c.async) return fail(KC_ERR_ARG, "KC_AUTOTUNE times the batch and does not take KC_ASYNC");
     const uint64_t sig = batch_signature(b, n, d, k);
     double theta = kThetaDefault;
-    const bool known = pick_theta(sig, &theta);
+    bool teams = false;
+    const bool known = pick_theta(sig, &theta, &teams);
 
     BatchBufs B;
     // One solve with the given theta: layout, inputs, descriptors, launches.
-    auto solve = [&](double th, float *ms) -> kc_status {
-        batch_policy(b, n, d, k, th);
+    auto solve = [&](double th, bool teams, float *ms) -> kc_status {
+        batch_policy(b, n, d, k, th, teams);
         Carve sizing(nullptr);
         batch_layout(sizing, b, B, n, d, k, centers, k_out, radii, dev_pts.data(), dev_cen.data(), dev_kout, dev_rad);
         kc_status rr = arena_reserve(c.arena, sizing.off, c.s);
@@ -2151,7 +2282,7 @@ kc_status kc_gonzalez_batch(int32_t count, const void *const *pts, const int64_t
         float best_ms = 0.f;
         for (double th : kThetas) {
             float ms = 0.f;
-            if ((r = solve(th, &ms)) != KC_OK) return r;
+            if ((r = solve(th, false, &ms)) != KC_OK) return r;
             if ((r = finish(c.arena, c.s)) != KC_OK) return r;
             if (th == kThetas[0] || ms < best_ms) {
                 best_ms = ms;
@@ -2159,8 +2290,9 @@ kc_status kc_gonzalez_batch(int32_t count, const void *const *pts, const int64_t
             }
         }
         remember_theta(sig, theta);
+        teams = false;
     }
-    if ((r = solve(theta, nullptr)) != KC_OK) return r;
+    if ((r = solve(theta, teams, nullptr)) != KC_OK) return r;
     for (int i = 0; i < count; ++i)
         if (!dev_cen[i])
             KC_CUDA(cudaMemcpyAsync(centers[i], B.per[i].cen, (size_t)std::min<int64_t>(k[i], n[i]) * sizeof(int64_t),
@@ -2204,10 +2336,10 @@ void plan_free(kc_batch_plan *p) {
 // Build one plan: its own device allocation (outside the per-stream arena,
 // so later calls cannot move it), descriptors uploaded once, and the solve
 // captured into a CUDA graph.
-kc_status plan_build(BatchShape &b, double theta, int32_t count, const void *const *pts, const int64_t *n,
+kc_status plan_build(BatchShape &b, double theta, bool teams, int32_t count, const void *const *pts, const int64_t *n,
                      const int32_t *d, const int32_t *k, int64_t *const *centers, int32_t *k_out, double *radii,
                      const kc_opts &o, kc_batch_plan **out) {
-    batch_policy(b, n, d, k, theta);
+    batch_policy(b, n, d, k, theta, teams);
     std::vector<char> dev_pts((size_t)count, 1), dev_cen((size_t)count, 1);
     BatchBufs B;
     Carve sizing(nullptr);
@@ -2296,7 +2428,8 @@ kc_status kc_batch_plan_create(int32_t count, const void *const *pts, const int6
             return fail(KC_ERR_ARG, "instance %d: a plan needs device memory for points and centers", i);
     const uint64_t sig = batch_signature(b, n, d, k);
     double theta = kThetaDefault;
-    const bool known = pick_theta(sig, &theta);
+    bool teams = false;
+    const bool known = pick_theta(sig, &theta, &teams);
     if ((c.o.flags & KC_AUTOTUNE) && !known) {
         // Time each candidate's graph (one warm-up replay, then the fastest of
         // five replays timed one by one: a mean of a few replays let one slow
@@ -2308,7 +2441,7 @@ kc_status kc_batch_plan_create(int32_t count, const void *const *pts, const int6
         KC_CUDA(cudaEventCreate(&e1), "cudaEventCreate");
         for (double th : kThetas) {
             kc_batch_plan *p = nullptr;
-            if ((r = plan_build(b, th, count, pts, n, d, k, centers, k_out, radii, c.o, &p)) != KC_OK) break;
+            if ((r = plan_build(b, th, false, count, pts, n, d, k, centers, k_out, radii, c.o, &p)) != KC_OK) break;
             float ms = 0.f;
             cudaError_t e = cudaGraphLaunch(p->exec, c.s);
             for (int rep = 0; rep < 5 && e == cudaSuccess; ++rep) {
@@ -2347,7 +2480,7 @@ kc_status kc_batch_plan_create(int32_t count, const void *const *pts, const int6
         *plan = best;
         return KC_OK;
     }
-    return plan_build(b, theta, count, pts, n, d, k, centers, k_out, radii, c.o, plan);
+    return plan_build(b, theta, teams, count, pts, n, d, k, centers, k_out, radii, c.o, plan);
 }
 
 kc_status kc_batch_plan_run(kc_batch_plan *plan, void *stream) {

@@ -848,10 +848,82 @@ __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_kernel(GonArgs a) {
     gon_solve<T, DC, GROUP_NT, DYN>(I, r, I.G, cs, sh, a.st, a.timeout_cycles, a.withhold, a.bad_index != 0);
 }
 
-// Queue mode, optionally with heavy instances in front: insts[0, nheavy)
-// are solved by CTA groups [cta0, cta0 + G) of the first gheavy CTAs (the
-// launch is then cooperative, so the groups are co-resident); every CTA then
-// takes the remaining instances insts[nheavy, ninst) one at a time, in order.
+// A launch of mixed d solves each instance with the sweep made for its d, as
+// launches of one d do; out of line, so that each has the registers it needs
+// (inlined side by side they spilled: 4096 mixed FP32 instances 95 -> 114 ms).
+// With CTA groups that hold their instances in L2 the generic sweep's dependent
+// loads are what was left: 89 ms at the best group size, 60 with these.  The mixed-precision kernel keeps its
+// generic loop: out of line its sweeps gained less than its longer recheck
+// path lost (62 -> 70 ms).
+template <typename T, int DC>
+__device__ __noinline__ void queue_solve_d(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
+                                           long long timeout) {
+    gon_solve<T, DC, QUEUE_NT>(I, r, G, cs, sh, st, timeout);
+}
+template <typename T, int DC>
+__device__ __forceinline__ void queue_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
+                                            long long timeout) {
+    if constexpr (DC == 0 && std::is_same<T, float>::value) {
+        switch (I.d) {
+            case 3: queue_solve_d<T, 3>(I, r, G, cs, sh, st, timeout); return;
+            case 8: queue_solve_d<T, 8>(I, r, G, cs, sh, st, timeout); return;
+            case 16: queue_solve_d<T, 16>(I, r, G, cs, sh, st, timeout); return;
+            case 32: queue_solve_d<T, 32>(I, r, G, cs, sh, st, timeout); return;
+            default: queue_solve_d<T, 0>(I, r, G, cs, sh, st, timeout); return;
+        }
+    } else {
+        gon_solve<T, DC, QUEUE_NT>(I, r, G, cs, sh, st, timeout);
+    }
+}
+
+// Queue mode: position of the first of insts[from, m) that this CTA's group
+// solves, -1 if there is none (256 descriptors a round, a thread each).
+__device__ __forceinline__ int next_group(const GonInst *insts, int from, int m, int *s_i) {
+    for (int base = from; base < m; base += QUEUE_NT) {
+        const int i = base + (int)threadIdx.x;
+        const int r = i < m ? (int)blockIdx.x - insts[i].cta0 : -1;
+        const bool mine = r >= 0 && r < insts[i].G;
+        if (threadIdx.x == 0) *s_i = m;
+        if (__syncthreads_or(mine)) {
+            if (mine) atomicMin(s_i, i);
+            __syncthreads();
+            const int q = *s_i;
+            __syncthreads();
+            return q;
+        }
+    }
+    return -1;
+}
+
+// Wait until every CTA of the instance's group has come from its earlier
+// instances (I.join, zeroed, counts them; nullptr: the group has only this
+// instance and starts with the launch).  Each of the mates' own waits is
+// bounded by the budget, so this one takes several budgets before it gives up.
+__device__ __forceinline__ bool join_group(const GonInst &I, long long timeout, DevStatus *st) {
+    int stop = 0;
+    if (threadIdx.x == 0) {
+        stop = ld_volatile_i32(&st->code) != 0;
+        if (I.join) {
+            atomicAdd(I.join, 1);
+            const long long t0 = clock64();
+            for (int n = 1; !stop && ld_volatile_i32(I.join) < I.G; ++n)
+                if ((n & 31) == 0) {
+                    if (ld_volatile_i32(&st->code) != 0) stop = 1;
+                    else if ((clock64() - t0) / JOIN_BUDGETS > timeout) {
+                        set_status(st, KC_ERR_TIMEOUT, 3, 0);
+                        stop = 1;
+                    }
+                }
+        }
+    }
+    return !__syncthreads_or(stop);
+}
+
+// Queue mode, optionally with instances solved by CTA groups in front:
+// insts[0, nheavy) belong to the groups [cta0, cta0 + G) of the first gheavy
+// CTAs (the launch is then cooperative, so the groups are co-resident); a CTA
+// solves those whose group it is in, in order; every CTA then takes the
+// remaining instances insts[nheavy, ninst) one at a time, in order.
 template <typename T, int DC>
 __global__ void __launch_bounds__(QUEUE_NT) gon_queue_kernel(GonArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -860,11 +932,13 @@ __global__ void __launch_bounds__(QUEUE_NT) gon_queue_kernel(GonArgs a) {
     __shared__ Shared sh;
     __shared__ int s_i;
     if ((int)blockIdx.x < a.gheavy) {
-        copy_instance(I, find_group(a.insts, a.nheavy));
-        const int r = (int)blockIdx.x - I.cta0;
-        if (r >= 0 && r < I.G && ld_volatile_i32(&a.st->code) == 0 && instance_ok<T>(I, a.st))
-            gon_solve<T, DC, QUEUE_NT>(I, r, I.G, cs, sh, a.st, a.timeout_cycles);
-        __syncthreads();
+        for (int q = 0; (q = next_group(a.insts, q, a.nheavy, &s_i)) >= 0; ++q) {
+            copy_instance(I, a.insts + q);
+            if (!join_group(I, a.timeout_cycles, a.st)) return;
+            if (instance_ok<T>(I, a.st))
+                queue_solve<T, DC>(I, (int)blockIdx.x - I.cta0, I.G, cs, sh, a.st, a.timeout_cycles);
+            __syncthreads();
+        }
     }
     for (;;) {
         if (threadIdx.x == 0) s_i = a.nheavy + atomicAdd(a.counter, 1);
@@ -872,7 +946,7 @@ __global__ void __launch_bounds__(QUEUE_NT) gon_queue_kernel(GonArgs a) {
         if (s_i >= a.ninst) return;
         copy_instance(I, a.insts + s_i);
         if (ld_volatile_i32(&a.st->code) != 0) return;
-        if (instance_ok<T>(I, a.st)) gon_solve<T, DC, QUEUE_NT>(I, 0, 1, cs, sh, a.st, a.timeout_cycles);
+        if (instance_ok<T>(I, a.st)) queue_solve<T, DC>(I, 0, 1, cs, sh, a.st, a.timeout_cycles);
         __syncthreads();
     }
 }
@@ -897,11 +971,13 @@ __global__ void __launch_bounds__(QUEUE_NT, 4) gon_queue_lp_kernel(GonArgs a) {
     __shared__ ShLP sh;
     __shared__ int s_i;
     if ((int)blockIdx.x < a.gheavy) {
-        copy_instance(I, find_group(a.insts, a.nheavy));
-        const int r = (int)blockIdx.x - I.cta0;
-        if (r >= 0 && r < I.G && ld_volatile_i32(&a.st->code) == 0)
-            gon_solve_lp<KIND, DC, QUEUE_NT>(I, r, I.G, smem_f, sh, a.st, a.timeout_cycles, 0, a.lp_local_t != 0);
-        __syncthreads();
+        for (int q = 0; (q = next_group(a.insts, q, a.nheavy, &s_i)) >= 0; ++q) {
+            copy_instance(I, a.insts + q);
+            if (!join_group(I, a.timeout_cycles, a.st)) return;
+            gon_solve_lp<KIND, DC, QUEUE_NT>(I, (int)blockIdx.x - I.cta0, I.G, smem_f, sh, a.st, a.timeout_cycles, 0,
+                                             a.lp_local_t != 0);
+            __syncthreads();
+        }
     }
     for (;;) {
         if (threadIdx.x == 0) s_i = a.nheavy + atomicAdd(a.counter, 1);
@@ -1322,11 +1398,11 @@ int gon_max_grid(int dtype, int d, int lp) {
     return gon_occupancy(pick_fn(dtype, lp, d, false), GROUP_NT, smem_for(dtype, lp, d, false)) * sms;
 }
 
-int gon_queue_grid(int dtype, int d, int lp) {
+int gon_queue_grid(int dtype, int d, int lp, int dmax) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return gon_occupancy(pick_fn(dtype, lp, d, true), QUEUE_NT, smem_for(dtype, lp, d, true)) * sms;
+    return gon_occupancy(pick_fn(dtype, lp, d, true), QUEUE_NT, smem_for(dtype, lp, std::max(d, dmax), true)) * sms;
 }
 
 int gon_resident_plan(int dtype, int d, int64_t n, int *cap, int *slot_words) {

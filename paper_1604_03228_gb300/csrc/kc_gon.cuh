@@ -12,6 +12,7 @@ namespace {
 
 constexpr int GROUP_NT = 1024;   // group mode: one CTA per SM
 constexpr int QUEUE_NT = 256;    // queue mode: several CTAs per SM
+constexpr int JOIN_BUDGETS = 16; // wait for a group's CTAs to leave their earlier instances, in spin-wait budgets
 
 template <typename T> struct Vec4;
 template <> struct Vec4<float> { using type = float4; };

@@ -243,6 +243,7 @@ struct GonInst {
     const float *rm;
     uint32_t *mind;          // [nblocks(n) * BLK] running minimum (value bits)
     uint64_t *slots;         // [k * G] per-step, per-CTA argmax keys (zeroed)
+    int *join;               // queue kernels: CTAs of the group that have come to this instance (zeroed), or nullptr
     uint64_t *bc;            // [bc_words(d)] the leader's words of a step (zeroed), or nullptr: every CTA polls the slots
     int64_t *centers;        // [k] out
     int32_t *k_out;          // out
@@ -355,7 +356,7 @@ int gon_resident_plan(int dtype, int d, int64_t n, int *cap, int *slot_words);
 // Mixed-precision diagnostics (synchronous): exact rechecks, overflows.
 cudaError_t read_counters(unsigned long long out[8], bool reset);
 int gon_max_grid(int dtype, int d, int lp = 0);
-int gon_queue_grid(int dtype, int d, int lp = 0);
+int gon_queue_grid(int dtype, int d, int lp = 0, int dmax = 0);
 int gon_threads();
 // SM clock rate of a device in kHz (queried once per device: the query
 // costs a few hundred microseconds on some hosts).
@@ -383,6 +384,7 @@ inline void gon_single(GonArgs &g, const void *pk, int dtype, int64_t n, int d, 
     I.mind = mind;
     I.slots = slots;
     I.bc = nullptr;
+    I.join = nullptr;
     I.centers = centers;
     I.k_out = k_out;
     I.final_key = final_key;
