@@ -158,8 +158,10 @@ struct Shared {
 
 // All k steps of one instance by this CTA (rank r of a group of G).  DYN:
 // the instance is large enough for claimed blocks and the shared tail (a
-// separate instantiation, so that small instances run the plain loop).
-template <typename T, int DC, int NT, bool DYN = false>
+// separate instantiation, so that small instances run the plain loop).  LEAD:
+// the exchange may go through the leader (its own instantiation as well: one
+// CTA on 3608 x 16 takes 2.35 us a step without its code, 2.73 with it).
+template <typename T, int DC, int NT, bool DYN = false, bool LEAD = false>
 __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
                           long long timeout, int withhold = 0, bool bad_index = false) {
     constexpr int W = NT / 32;
@@ -190,12 +192,13 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
     // 230 us a step: 1% slower; float 8M x 64: 0.7%).  Not between queue CTAs,
     // which share their SM with other groups: nothing gained, and the sweep's
     // code grew (MRG round 1 on 10M x 16 20.2 -> 20.7 ms).
-    const bool lead = NT == GROUP_NT && !DYN && G > LEADER_MIN && I.bc != nullptr &&
+    const bool lead = LEAD && G > LEADER_MIN && I.bc != nullptr &&
                       (I.lo + I.n - 1) / BLK - I.lo / BLK + 1 < 4 * (int64_t)G * W;
 
+    const int it1 = I.it1;
     int it;
     uint64_t K = 0;
-    for (it = I.it0; it < I.it1; ++it) {
+    for (it = I.it0; it < it1; ++it) {
         // claimed blocks in the 1024-thread group CTAs when every warp has
         // several (measured: GON on 8M x 64, k = 1024, 313 -> 308 ms); the
         // fixed assignment in the 256-thread queue CTAs (MRG round 1 on
@@ -211,7 +214,7 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
             v = warp_max_u64(v);
             uint64_t g = v;
             bool ab = false;
-            const bool more = it + 1 < I.it1;
+            const bool more = it + 1 < it1;
             const uint64_t tagw = (uint64_t)(it + 1) << 32;
             if (G > 1) {
                 uint64_t *row = I.slots + (int64_t)it * slot_stride(G);
@@ -234,7 +237,7 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
                 }
                 if (tail) __threadfence();
             }
-            if (!ab && more && (!lead || r == 0)) {
+            if (!ab && more && (lead ? r == 0 : key_val(g) != 0)) {
 #ifdef KC_CHECKS
                 // testing hook of the checked build: a winner index one past
                 // the instance, which the check below must catch
@@ -242,13 +245,13 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
 #else
                 const int64_t c = key_idx(g);
 #endif
-                if (key_val(g) == 0 || KC_IN_RANGE(st, c, I.n, KC_AT_CENTER_LOAD)) {
+                if ((lead && key_val(g) == 0) || KC_IN_RANGE(st, c, I.n, KC_AT_CENTER_LOAD)) {
                     for (int j = lane; j < d; j += 32) {
-                        const T x = key_val(g) != 0 ? pk[pk_index(I.lo + c, j, d)] : T(0);
+                        const T x = !lead || key_val(g) != 0 ? pk[pk_index(I.lo + c, j, d)] : T(0);
                         cs[j] = x;
                         if (lead) st_relaxed_u64(I.bc + 2 + j, tagw | *reinterpret_cast<const uint32_t *>(&x));
                     }
-                    if (r == 0 && lane == 0 && key_val(g) != 0) I.centers[it + 1] = out_index(I, c);
+                    if (r == 0 && lane == 0 && (!lead || key_val(g) != 0)) I.centers[it + 1] = out_index(I, c);
                 } else {
                     ab = true;
                 }
@@ -833,7 +836,7 @@ __device__ void gon_solve_lp(const GonInst &I, int r, int G, float *smem, ShLP &
     }
 }
 
-template <typename T, int DC, bool DYN>
+template <typename T, int DC, bool DYN, bool LEAD>
 __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_kernel(GonArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *cs = reinterpret_cast<T *>(smem_raw);
@@ -845,7 +848,7 @@ __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_kernel(GonArgs a) {
     if (ld_volatile_i32(&a.st->code) != 0) return;
     if (a.route && ld_volatile_i32(a.route) != 0) return;   // the skip kernel runs the rest
     if (!instance_ok<T>(I, a.st)) return;
-    gon_solve<T, DC, GROUP_NT, DYN>(I, r, I.G, cs, sh, a.st, a.timeout_cycles, a.withhold, a.bad_index != 0);
+    gon_solve<T, DC, GROUP_NT, DYN, LEAD>(I, r, I.G, cs, sh, a.st, a.timeout_cycles, a.withhold, a.bad_index != 0);
 }
 
 // A launch of mixed d solves each instance with the sweep made for its d, as
@@ -1265,7 +1268,7 @@ void *pick_resident(int dtype, int d) {
     return d == 10 ? resident_fn<int32_t, 10>() : nullptr;
 }
 
-template <typename T, int DC, bool DYN = false> void *group_fn() { return (void *)gon_group_kernel<T, DC, DYN>; }
+template <typename T, int DC, bool DYN, bool LEAD> void *group_fn() { return (void *)gon_group_kernel<T, DC, DYN, LEAD>; }
 template <typename T, int DC> void *queue_fn() { return (void *)gon_queue_kernel<T, DC>; }
 template <int KIND, int DC> void *group_lp_fn() { return (void *)gon_group_lp_kernel<KIND, DC>; }
 template <int KIND, int DC> void *queue_lp_fn() { return (void *)gon_queue_lp_kernel<KIND, DC>; }
@@ -1309,36 +1312,29 @@ size_t lp_smem_bytes(int kind, int dmax, int nt) {
     return (size_t)2 * ((dp + 1) & ~1) * sizeof(float) + (size_t)(nt / 32) * LP_CAP * sizeof(Cand);
 }
 
-void *pick_group(int dtype, int dc, bool dyn = false) {
-    if (dtype == KC_F32 && dyn) {
-        switch (dc) {
-            case 2: return group_fn<float, 2, true>();
-            case 3: return group_fn<float, 3, true>();
-            case 8: return group_fn<float, 8, true>();
-            case 10: return group_fn<float, 10, true>();
-            case 16: return group_fn<float, 16, true>();
-            case 32: return group_fn<float, 32, true>();
-            case 64: return group_fn<float, 64, true>();
-            default: return group_fn<float, 0, true>();
-        }
-    }
-    if (dtype == KC_F32) {
-        switch (dc) {
-            case 2: return group_fn<float, 2>();
-            case 3: return group_fn<float, 3>();
-            case 8: return group_fn<float, 8>();
-            case 10: return group_fn<float, 10>();
-            case 16: return group_fn<float, 16>();
-            case 32: return group_fn<float, 32>();
-            case 64: return group_fn<float, 64>();
-            default: return group_fn<float, 0>();
-        }
-    }
+template <bool DYN, bool LEAD> void *pick_group_f32(int dc) {
     switch (dc) {
-        case 2: return group_fn<int32_t, 2>();
-        case 10: return group_fn<int32_t, 10>();
-        default: return group_fn<int32_t, 0>();
+        case 2: return group_fn<float, 2, DYN, LEAD>();
+        case 3: return group_fn<float, 3, DYN, LEAD>();
+        case 8: return group_fn<float, 8, DYN, LEAD>();
+        case 10: return group_fn<float, 10, DYN, LEAD>();
+        case 16: return group_fn<float, 16, DYN, LEAD>();
+        case 32: return group_fn<float, 32, DYN, LEAD>();
+        case 64: return group_fn<float, 64, DYN, LEAD>();
+        default: return group_fn<float, 0, DYN, LEAD>();
     }
+}
+template <bool LEAD> void *pick_group_i32(int dc) {
+    switch (dc) {
+        case 2: return group_fn<int32_t, 2, false, LEAD>();
+        case 10: return group_fn<int32_t, 10, false, LEAD>();
+        default: return group_fn<int32_t, 0, false, LEAD>();
+    }
+}
+void *pick_group(int dtype, int dc, bool dyn, bool lead) {
+    if (dtype != KC_F32) return lead ? pick_group_i32<true>(dc) : pick_group_i32<false>(dc);
+    if (dyn) return pick_group_f32<true, false>(dc);
+    return lead ? pick_group_f32<false, true>(dc) : pick_group_f32<false, false>(dc);
 }
 
 void *pick_queue(int dtype, int dc) {
@@ -1369,9 +1365,9 @@ int gon_threads() { return GROUP_NT; }
 int gon_queue_warps() { return QUEUE_NT / 32; }
 int gon_warps_per_cta() { return GROUP_NT / 32; }
 
-static void *pick_fn(int dtype, int lp, int dc, bool queue, bool dyn = false) {
+static void *pick_fn(int dtype, int lp, int dc, bool queue, bool dyn = false, bool lead = false) {
     if (dtype == KC_F32 && lp) return queue ? pick_queue_lp(lp, dc) : pick_group_lp(lp, dc);
-    return queue ? pick_queue(dtype, dc) : pick_group(dtype, dc, dyn);
+    return queue ? pick_queue(dtype, dc) : pick_group(dtype, dc, dyn, lead);
 }
 
 static size_t smem_for(int dtype, int lp, int dmax, bool queue) {
@@ -1471,7 +1467,7 @@ cudaError_t launch_gon(GonArgs &a, cudaStream_t s) {
         return cudaLaunchKernelExC(&cfg, fn, args);
     }
     const size_t smem = smem_for(a.dtype, a.lp_kind, a.dmax, a.queue != 0);
-    void *fn = pick_fn(a.dtype, a.lp_kind, a.dc, a.queue != 0, a.dyn != 0);
+    void *fn = pick_fn(a.dtype, a.lp_kind, a.dc, a.queue != 0, a.dyn != 0, a.grid > LEADER_MIN);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
