@@ -485,8 +485,14 @@ int choose_gon_grid(int dtype, int d, int64_t n, int lp = 0) {
     const int maxg = gon_max_grid(dtype, d, lp);
     const int W = gon_warps_per_cta();
     const int64_t nb = nblocks(n);
-    // Aim for about two 128-point blocks per warp; whole waves of SMs.
-    int64_t want = (nb + 2 * W - 1) / (2 * W);
+    // One 128-point block per warp while that needs no more than one CTA per
+    // SM, so that a step's sweep is one round of loads (at two per warp, us a
+    // step, FP32 / bf16: 10k x 64 12.0 / 15.9 against 7.6 / 12.1, 100k x 20
+    // 7.0 / 11.3 against 4.8 / 9.4, 300k x 37 12.2 / 16.6 against 7.6 / 12.9);
+    // beyond, two per warp (777k x 37 on 95 CTAs 26.6 / 17.8, on 152, some
+    // warps with two blocks and some with one, 28.0 / 18.9); whole waves of SMs.
+    int64_t want = (nb + W - 1) / W;
+    if (want > sms) want = (nb + 2 * W - 1) / (2 * W);
     int g;
     if (want >= sms) {
         int64_t per = (want + sms - 1) / sms;
