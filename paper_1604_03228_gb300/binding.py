@@ -256,6 +256,13 @@ def _item(x):
     return x[0].item()
 
 
+def _host_scalars(*types):
+    """Host memory for a waiting call's scalar results (they come back with
+    its status) and their addresses."""
+    v = [t() for t in types]
+    return v, [ct.addressof(x) for x in v]
+
+
 @dataclass
 class GonResult:
     centers: object        # int64 [k_out] (tensor or ndarray, same place as the input)
@@ -277,13 +284,18 @@ def kc_gonzalez(points, k: int, first: int = 0, *, stream=None, flags: int = 0,
     raw device outputs (centers[k], k_out[1], radius[1]) without waiting."""
     L = load()
     p, n, d, code = _points(points)
+    o = _opts(code, p, stream, flags, timeout_ms, sweep=sweep)
+    if out is None and not flags & KC_ASYNC:
+        centers = _empty_like_place(p, k, np.int64)
+        (k_out, radius), at = _host_scalars(ct.c_int32, ct.c_double)
+        _check(L, L.kc_gonzalez(_ptr(p), n, d, k, first, _ptr(centers), *at, ct.byref(o)))
+        return GonResult(centers[:k_out.value], k_out.value, radius.value)
     if out is None:
         centers = _empty_like_place(p, k, np.int64)
         k_out = _empty_like_place(p, 1, np.int32)
         radius = _empty_like_place(p, 1, np.float64)
     else:
         centers, k_out, radius = out
-    o = _opts(code, p, stream, flags, timeout_ms, sweep=sweep)
     st = L.kc_gonzalez(_ptr(p), n, d, k, first, _ptr(centers), _ptr(k_out), _ptr(radius), ct.byref(o))
     _check(L, st)
     if flags & KC_ASYNC:
@@ -325,12 +337,16 @@ def kc_radius(points, centers, *, stream=None, flags: int = 0, timeout_ms: int =
     else:
         c = np.ascontiguousarray(centers, dtype=np.int64)
     kc = int(c.shape[0])
+    o = _opts(code, p, stream, flags, timeout_ms)
+    if out is None and not flags & KC_ASYNC:
+        (radius, argmax), at = _host_scalars(ct.c_double, ct.c_int64)
+        _check(L, L.kc_radius(_ptr(p), n, d, _ptr(c), kc, *at, ct.byref(o)))
+        return RadiusResult(radius.value, argmax.value)
     if out is None:
         radius = _empty_like_place(p, 1, np.float64)
         argmax = _empty_like_place(p, 1, np.int64)
     else:
         radius, argmax = out
-    o = _opts(code, p, stream, flags, timeout_ms)
     st = L.kc_radius(_ptr(p), n, d, _ptr(c), kc, _ptr(radius), _ptr(argmax), ct.byref(o))
     _check(L, st)
     if flags & KC_ASYNC:
@@ -352,13 +368,18 @@ def kc_mrg(points, k: int, m: int, offsets=None, *, stream=None, flags: int = 0,
             off = np.ascontiguousarray(offsets, dtype=np.int64)
         if int(off.shape[0]) != m + 1:
             raise ValueError("offsets must have m+1 entries")
+    o = _opts(code, p, stream, flags, timeout_ms, sweep=sweep)
+    if out is None and not flags & KC_ASYNC:
+        centers = _empty_like_place(p, k, np.int64)
+        (k_out, radius), at = _host_scalars(ct.c_int32, ct.c_double)
+        _check(L, L.kc_mrg(_ptr(p), n, d, k, m, _ptr(off), _ptr(centers), *at, ct.byref(o)))
+        return GonResult(centers[:k_out.value], k_out.value, radius.value)
     if out is None:
         centers = _empty_like_place(p, k, np.int64)
         k_out = _empty_like_place(p, 1, np.int32)
         radius = _empty_like_place(p, 1, np.float64)
     else:
         centers, k_out, radius = out
-    o = _opts(code, p, stream, flags, timeout_ms, sweep=sweep)
     st = L.kc_mrg(_ptr(p), n, d, k, m, _ptr(off), _ptr(centers), _ptr(k_out), _ptr(radius), ct.byref(o))
     _check(L, st)
     if flags & KC_ASYNC:
@@ -379,15 +400,13 @@ def kc_mrg_rounds(points, k: int, m: int, capacity: int, offsets=None, *, stream
         if int(off.shape[0]) != m + 1:
             raise ValueError("offsets must have m+1 entries")
     centers = _empty_like_place(p, k, np.int64)
-    k_out = _empty_like_place(p, 1, np.int32)
-    radius = _empty_like_place(p, 1, np.float64)
+    (k_out, radius), at = _host_scalars(ct.c_int32, ct.c_double)
     rounds = ct.c_int32(0)
     o = _opts(code, p, stream, 0, timeout_ms, sweep=sweep)
-    st = L.kc_mrg_rounds(_ptr(p), n, d, k, m, _ptr(off), int(capacity), _ptr(centers), _ptr(k_out), _ptr(radius),
-                         ct.byref(rounds), ct.byref(o))
+    st = L.kc_mrg_rounds(_ptr(p), n, d, k, m, _ptr(off), int(capacity), _ptr(centers), *at, ct.byref(rounds),
+                         ct.byref(o))
     _check(L, st)
-    kk = int(_item(k_out))
-    return GonResult(centers[:kk], kk, float(_item(radius))), rounds.value
+    return GonResult(centers[:k_out.value], k_out.value, radius.value), rounds.value
 
 
 def kc_eim(points, k: int, eps: float = 0.1, phi: float = 6.0, seed: int = 0, *, stream=None,
@@ -396,13 +415,10 @@ def kc_eim(points, k: int, eps: float = 0.1, phi: float = 6.0, seed: int = 0, *,
     L = load()
     p, n, d, code = _points(points)
     centers = _empty_like_place(p, k, np.int64)
-    k_out = _empty_like_place(p, 1, np.int32)
-    radius = _empty_like_place(p, 1, np.float64)
+    (k_out, radius), at = _host_scalars(ct.c_int32, ct.c_double)
     o = _opts(code, p, stream, 0, timeout_ms, seed=seed, phi=phi, sweep=sweep)
-    st = L.kc_eim(_ptr(p), n, d, k, float(eps), _ptr(centers), _ptr(k_out), _ptr(radius), ct.byref(o))
-    _check(L, st)
-    kk = int(_item(k_out))
-    return GonResult(centers[:kk], kk, float(_item(radius)))
+    _check(L, L.kc_eim(_ptr(p), n, d, k, float(eps), _ptr(centers), *at, ct.byref(o)))
+    return GonResult(centers[:k_out.value], k_out.value, radius.value)
 
 
 def kc_gonzalez_batch(points_list, ks, *, stream=None, flags: int = 0, timeout_ms: int = 0,
