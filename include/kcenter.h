@@ -269,12 +269,12 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
  * whose work exceeds the fair share of one resident CTA (FP32: or whose points
  * exceed its part of the L2 cache) is solved by a group of CTAs (cooperative
  * launch), and groups solve further instances one after another; the others go
- * through a queue, one CTA each, longest first.  With KC_BATCH_THETA or
- * KC_AUTOTUNE each group solves one instance: those whose work exceeds theta
- * times the fair share, as long as half of the CTAs suffice.  With
+ * through a queue, one CTA each, longest first.  With KC_BATCH_THETA each
+ * group solves one instance: those whose work exceeds theta times the fair
+ * share, as long as half of the CTAs suffice.  With
  * KC_AUTOTUNE in opts->flags the first call for a batch shape (count, dtype,
- * sweep and every (n, d, k)) solves the batch once per candidate theta
- * (plain queue, 4, 2, 1, 0.5), keeps the fastest for later calls in the
+ * sweep and every (n, d, k)) solves the batch once per candidate
+ * (the default; theta = inf, 4, 2, 1, 0.5), keeps the fastest for later calls in the
  * process, and returns the result of a final solve with it.  Every launch
  * shape selects the same centers.  KC_AUTOTUNE does not combine with
  * KC_ASYNC.  Errors: as kc_gonzalez, per instance; KC_ERR_ARG for the fp8
@@ -292,8 +292,8 @@ kc_status kc_gonzalez_batch(int32_t count, const void *const *pts, const int64_t
  *
  * kc_batch_plan_create takes the arguments of kc_gonzalez_batch, all of them
  * device memory of the current device (KC_ERR_ARG otherwise), checks them,
- * picks the launch shape (KC_AUTOTUNE: builds and times a plan per candidate
- * theta: a warm-up replay, then the fastest of five, and keeps the fastest), allocates the plan's
+ * picks the launch shape (KC_AUTOTUNE: builds and times a plan per
+ * candidate: a warm-up replay, then the fastest of five, and keeps the fastest), allocates the plan's
  * own scratch (freed by kc_batch_plan_destroy), uploads the instance
  * descriptors and captures pack + GON + radius into a CUDA graph.  The
  * pointers are bound at creation: each run reads the current contents of
@@ -303,7 +303,7 @@ kc_status kc_gonzalez_batch(int32_t count, const void *const *pts, const int64_t
  * must not overlap (they share scratch): order them on one stream.
  * kc_batch_plan_wait waits for the last run and returns its device status
  * (KC_ERR_RANGE, KC_ERR_NONFINITE, KC_ERR_TIMEOUT as kc_gonzalez).
- * kc_batch_plan_info reports the chosen theta (1 if none was set or timed),
+ * kc_batch_plan_info reports the chosen theta (1 for the default),
  * the number of group-solved instances, the CTAs of their groups (the first
  * ones of the grid), and the grid size.
  * kc_batch_plan_destroy waits for the last run and frees the plan (NULL is

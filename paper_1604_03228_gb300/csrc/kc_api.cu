@@ -1788,17 +1788,23 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
 // bf16 does not group by L2: it is issue-bound, with two exchanges a step
 // (4096: 62.5 -> 83 ms).
 //
-// KC_BATCH_THETA and KC_AUTOTUNE take the one-level split instead: an instance
-// with w > theta W / S is heavy and solved by a CTA group of
-// G = ceil(w / (W / S)) CTAs at the front of a cooperative grid, while the
-// groups take at most half of the CTAs; the others go through the queue.
-// theta = +inf is the plain queue.  KC_AUTOTUNE times every theta of kThetas
-// on the batch itself and keeps the fastest per batch shape.
+// KC_BATCH_THETA takes the one-level split instead: an instance with
+// w > theta W / S is heavy and solved by a CTA group of G = ceil(w / (W / S))
+// CTAs at the front of a cooperative grid, while the groups take at most half
+// of the CTAs; the others go through the queue.  theta = +inf is the plain
+// queue.  KC_AUTOTUNE times the default and this split with several thetas
+// (kSplits) on the batch itself and keeps the fastest per batch shape.
 namespace {
 
 constexpr double kThetaQueue = 1e300;
-constexpr double kThetas[] = {kThetaQueue, 4.0, 2.0, 1.0, 0.5};
 constexpr double kThetaDefault = 1.0;
+// A launch shape: the one-level split with theta, or the default groups
+// (teams; theta then stands for itself in kc_batch_plan_info only).
+struct Split {
+    double theta = kThetaDefault;
+    bool teams = true;
+};
+constexpr Split kSplits[] = {{kThetaQueue, false}, {4.0, false}, {2.0, false}, {1.0, false}, {0.5, false}, {1.0, true}};
 
 struct BatchShape {
     int count = 0, dtype = 0, lp = 0, dc = 0, dmax = 0;
@@ -1902,7 +1908,8 @@ bool slot_room(const BatchShape &b, const int64_t *n, const int32_t *d, const in
     return slots <= packed / 16 + 16.0 * 1048576;
 }
 
-void batch_policy(BatchShape &b, const int64_t *n, const int32_t *d, const int32_t *k, double theta, bool teams) {
+void batch_policy(BatchShape &b, const int64_t *n, const int32_t *d, const int32_t *k, const Split &split) {
+    const double theta = split.theta;
     const int count = b.count;
     const double bpc = b.lp == KC_SWEEP_BF16 ? 2.0 : 4.0;
     std::vector<double> w((size_t)count);
@@ -1921,8 +1928,8 @@ void batch_policy(BatchShape &b, const int64_t *n, const int32_t *d, const int32
     b.cta0.clear();
     b.nheavy = b.gheavy = 0;
     b.theta = theta;
-    b.teams = teams;
-    if (teams) {
+    b.teams = split.teams;
+    if (split.teams) {
         batch_teams(b, n, k, w, lpt, slots, share);
         if (slot_room(b, n, d, k)) return;
         b.order.clear();
@@ -1979,37 +1986,32 @@ uint64_t batch_signature(const BatchShape &b, const int64_t *n, const int32_t *d
 }
 
 std::mutex g_tune_mu;
-std::map<uint64_t, double> g_tune;   // batch signature -> fastest theta
+std::map<uint64_t, Split> g_tune;   // batch signature -> fastest split
 
-
-bool tuned_theta(uint64_t sig, double *theta) {
+bool tuned_split(uint64_t sig, Split *split) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(sig);
     if (it == g_tune.end()) return false;
-    *theta = it->second;
+    *split = it->second;
     return true;
 }
 
-void remember_theta(uint64_t sig, double theta) {
+void remember_split(uint64_t sig, const Split &split) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune[sig] = theta;
+    g_tune[sig] = split;
 }
 
-// The theta for a batch: KC_BATCH_THETA if set ("inf": the plain queue;
-// it also skips tuning), else the tuned one for this shape, else the
-// default.  Returns whether the choice is settled (no tuning needed).
-bool pick_theta(uint64_t sig, double *theta, bool *teams) {
-    *teams = false;
+// The split for a batch: KC_BATCH_THETA if set ("inf": the plain queue; it
+// also skips tuning), else the tuned one for this shape, else the default.
+// Returns whether the choice is settled (no tuning needed).
+bool pick_split(uint64_t sig, Split *split) {
     const char *e = getenv("KC_BATCH_THETA");
     if (e && *e) {
         const double v = strcmp(e, "inf") == 0 ? kThetaQueue : atof(e);
-        *theta = v > 0 ? v : kThetaDefault;
+        *split = {v > 0 ? v : kThetaDefault, false};
         return true;
     }
-    *theta = kThetaDefault;
-    const bool tuned = tuned_theta(sig, theta);
-    *teams = !tuned;
-    return tuned;
+    return tuned_split(sig, split);
 }
 
 // Device buffers of one batch, carved from one allocation.  The zero region
@@ -2244,14 +2246,13 @@ kc_status kc_gonzalez_batch(int32_t count, const void *const *pts, const int64_t
     const bool tune = (c.o.flags & KC_AUTOTUNE) != 0;
     if (tune && c.async) return fail(KC_ERR_ARG, "KC_AUTOTUNE times the batch and does not take KC_ASYNC");
     const uint64_t sig = batch_signature(b, n, d, k);
-    double theta = kThetaDefault;
-    bool teams = false;
-    const bool known = pick_theta(sig, &theta, &teams);
+    Split split;
+    const bool known = pick_split(sig, &split);
 
     BatchBufs B;
-    // One solve with the given theta: layout, inputs, descriptors, launches.
-    auto solve = [&](double th, bool teams, float *ms) -> kc_status {
-        batch_policy(b, n, d, k, th, teams);
+    // One solve with the given split: layout, inputs, descriptors, launches.
+    auto solve = [&](const Split &sp, float *ms) -> kc_status {
+        batch_policy(b, n, d, k, sp);
         Carve sizing(nullptr);
         batch_layout(sizing, b, B, n, d, k, centers, k_out, radii, dev_pts.data(), dev_cen.data(), dev_kout, dev_rad);
         kc_status rr = arena_reserve(c.arena, sizing.off, c.s);
@@ -2288,21 +2289,20 @@ kc_status kc_gonzalez_batch(int32_t count, const void *const *pts, const int64_t
 
     if (tune && !known) {
         // Every candidate solves the batch exactly (selection does not depend
-        // on the launch shape); the fastest theta is remembered.
+        // on the launch shape); the fastest split is remembered.
         float best_ms = 0.f;
-        for (double th : kThetas) {
+        for (const Split &sp : kSplits) {
             float ms = 0.f;
-            if ((r = solve(th, false, &ms)) != KC_OK) return r;
+            if ((r = solve(sp, &ms)) != KC_OK) return r;
             if ((r = finish(c.arena, c.s)) != KC_OK) return r;
-            if (th == kThetas[0] || ms < best_ms) {
+            if (&sp == kSplits || ms < best_ms) {
                 best_ms = ms;
-                theta = th;
+                split = sp;
             }
         }
-        remember_theta(sig, theta);
-        teams = false;
+        remember_split(sig, split);
     }
-    if ((r = solve(theta, teams, nullptr)) != KC_OK) return r;
+    if ((r = solve(split, nullptr)) != KC_OK) return r;
     for (int i = 0; i < count; ++i)
         if (!dev_cen[i])
             KC_CUDA(cudaMemcpyAsync(centers[i], B.per[i].cen, (size_t)std::min<int64_t>(k[i], n[i]) * sizeof(int64_t),
@@ -2330,6 +2330,7 @@ struct kc_batch_plan {
     cudaStream_t last = nullptr;
     bool ran = false;
     double theta = 0;
+    bool teams = false;
     int nheavy = 0, gheavy = 0, grid = 0;
 };
 
@@ -2346,10 +2347,10 @@ void plan_free(kc_batch_plan *p) {
 // Build one plan: its own device allocation (outside the per-stream arena,
 // so later calls cannot move it), descriptors uploaded once, and the solve
 // captured into a CUDA graph.
-kc_status plan_build(BatchShape &b, double theta, bool teams, int32_t count, const void *const *pts, const int64_t *n,
+kc_status plan_build(BatchShape &b, const Split &split, int32_t count, const void *const *pts, const int64_t *n,
                      const int32_t *d, const int32_t *k, int64_t *const *centers, int32_t *k_out, double *radii,
                      const kc_opts &o, kc_batch_plan **out) {
-    batch_policy(b, n, d, k, theta, teams);
+    batch_policy(b, n, d, k, split);
     std::vector<char> dev_pts((size_t)count, 1), dev_cen((size_t)count, 1);
     BatchBufs B;
     Carve sizing(nullptr);
@@ -2398,7 +2399,8 @@ kc_status plan_build(BatchShape &b, double theta, bool teams, int32_t count, con
         plan_free(p);
         return r;
     }
-    p->theta = theta;
+    p->theta = split.theta;
+    p->teams = b.teams;
     p->nheavy = b.nheavy;
     p->gheavy = b.gheavy;
     p->grid = b.grid;
@@ -2437,9 +2439,8 @@ kc_status kc_batch_plan_create(int32_t count, const void *const *pts, const int6
         if (!is_device_ptr(pts[i], c.dev) || !is_device_ptr(centers[i], c.dev))
             return fail(KC_ERR_ARG, "instance %d: a plan needs device memory for points and centers", i);
     const uint64_t sig = batch_signature(b, n, d, k);
-    double theta = kThetaDefault;
-    bool teams = false;
-    const bool known = pick_theta(sig, &theta, &teams);
+    Split split;
+    const bool known = pick_split(sig, &split);
     if ((c.o.flags & KC_AUTOTUNE) && !known) {
         // Time each candidate's graph (one warm-up replay, then the fastest of
         // five replays timed one by one: a mean of a few replays let one slow
@@ -2449,9 +2450,9 @@ kc_status kc_batch_plan_create(int32_t count, const void *const *pts, const int6
         cudaEvent_t e0, e1;
         KC_CUDA(cudaEventCreate(&e0), "cudaEventCreate");
         KC_CUDA(cudaEventCreate(&e1), "cudaEventCreate");
-        for (double th : kThetas) {
+        for (const Split &sp : kSplits) {
             kc_batch_plan *p = nullptr;
-            if ((r = plan_build(b, th, false, count, pts, n, d, k, centers, k_out, radii, c.o, &p)) != KC_OK) break;
+            if ((r = plan_build(b, sp, count, pts, n, d, k, centers, k_out, radii, c.o, &p)) != KC_OK) break;
             float ms = 0.f;
             cudaError_t e = cudaGraphLaunch(p->exec, c.s);
             for (int rep = 0; rep < 5 && e == cudaSuccess; ++rep) {
@@ -2486,11 +2487,11 @@ kc_status kc_batch_plan_create(int32_t count, const void *const *pts, const int6
             plan_free(best);
             return r;
         }
-        remember_theta(sig, best->theta);
+        remember_split(sig, {best->theta, best->teams});
         *plan = best;
         return KC_OK;
     }
-    return plan_build(b, theta, teams, count, pts, n, d, k, centers, k_out, radii, c.o, plan);
+    return plan_build(b, split, count, pts, n, d, k, centers, k_out, radii, c.o, plan);
 }
 
 kc_status kc_batch_plan_run(kc_batch_plan *plan, void *stream) {
