@@ -682,7 +682,8 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
     const bool bad_index = (c.o.flags & KC_TEST_BAD_INDEX) != 0;
 
     const bool dev_pts = is_device_ptr(pts, c.dev);
-    const void *pin_pts = dev_pts ? nullptr : pinned_device_ptr(pts);   // read in place by the pack
+    const void *const pinned = dev_pts ? nullptr : pinned_device_ptr(pts);
+    const void *pin_pts = pinned;   // read in place by the pack
     const bool dev_cen = is_device_ptr(centers, c.dev);
     const bool dev_kout = is_device_ptr(k_out, c.dev);
     const bool dev_rad = is_device_ptr(radius, c.dev);
@@ -703,11 +704,16 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
                      nblocks(n) >= 4 * (int64_t)grid * gon_warps_per_cta();   // claimed blocks pay off
     bool use_tail = dyn && grid > 1 && nblocks(n) * 7 / 8 / ((int64_t)grid * gon_warps_per_cta()) >= 2;
     if (const char *env = getenv("KC_GON_TAIL")) use_tail = use_tail && atoi(env) != 0;
-    // large float sets whose rows are in device memory may change over to the
-    // skip kernel after one of these steps
+    // large float sets may change over to the skip kernel after one of these
+    // steps; it reads rows in device memory, so pinned points are then copied
+    // there (8M x 64, k = 1024 from pinned memory: 317 ms a call read in place,
+    // with every step streaming, 52 with the copy).  The copy is one more pass,
+    // 2% of a streaming solve at k = 64 (8M x 64 uniform 29.9 -> 30.7 ms), so
+    // only from k = 256 on.
     int seg_end[8];
-    const int nseg = !res_grid && !pin_pts && !bad_index
-                         ? gon_skip_segments(c.o.dtype, d, n, keff, grid, seg_end, 8) : 0;
+    int nseg = !res_grid && !bad_index ? gon_skip_segments(c.o.dtype, d, n, keff, grid, seg_end, 8) : 0;
+    if (pin_pts && keff < 256) nseg = 0;
+    if (nseg) pin_pts = nullptr;
     const int64_t nb = nblocks(n);
     const size_t esz = 4;
     LPBufs LB;
@@ -791,6 +797,16 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
         Carve sizing(nullptr);
         layout(sizing, g, ra, &staging, &cen_dev, &kout_dev, &rad_dev, &zero_bytes);
         r = arena_reserve(c.arena, sizing.off, c.s);
+        if (r == KC_ERR_OOM && nseg) {   // the streaming kernels alone need less
+            g_err.clear();
+            nseg = 0;
+            pin_pts = pinned;
+            g = GonArgs{};
+            ra = RadiusArgs{};
+            Carve less(nullptr);
+            layout(less, g, ra, &staging, &cen_dev, &kout_dev, &rad_dev, &zero_bytes);
+            r = arena_reserve(c.arena, less.off, c.s);
+        }
         if (r != KC_OK) return r;
     }
     Carve cv(c.arena->dev);
@@ -1423,15 +1439,15 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
     // tensor cores above; pivots (cells) at most
     const char *cenv = getenv("KC_EIM_CELLS");
     const bool cells_ok = c.o.dtype == KC_F32 && !(cenv && atoi(cenv) == 0);
-    const int Pmax = !cells_ok ? 0 : (d < 16 ? CELLS_MAX : EIM_PIVOTS_TC);
-    const int64_t npad = n + (int64_t)Pmax * (TC_CELL_UNIT - 1);   // a list sorted by cell
+    int Pmax = !cells_ok ? 0 : (d < 16 ? CELLS_MAX : EIM_PIVOTS_TC);
+    int64_t npad = n + (int64_t)Pmax * (TC_CELL_UNIT - 1);   // a list sorted by cell
     constexpr int64_t PSAMPLE = 8192;                              // rows of S the pivots are chosen from (d >= 16)
     CellBufs CB;
     CellSort CR, CS;
     int *ctiles = nullptr, *cntile = nullptr;
     bool assigned = false;
     SkipBufs SB{};
-    const bool skip_ok = !lp && gon_skip_possible(c.o.dtype, d, n, keff_max, grid);
+    bool skip_ok = !lp && gon_skip_possible(c.o.dtype, d, n, keff_max, grid);
     LPBufs LB;
     float *cenT = nullptr, *ecmax = nullptr;
     RadiusArgs Rtc{}, Ptc{};
@@ -1564,6 +1580,15 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         Carve sizing(nullptr);
         layout(sizing);
         r = arena_reserve(c.arena, sizing.off, c.s);
+        if (r == KC_ERR_OOM && (Pmax || skip_ok)) {   // without cells and the skip kernel it takes less
+            g_err.clear();
+            Pmax = 0;
+            npad = n;
+            skip_ok = false;
+            Carve less(nullptr);
+            layout(less);
+            r = arena_reserve(c.arena, less.off, c.s);
+        }
         if (r != KC_OK) return r;
     }
     Carve cv(c.arena->dev);

@@ -55,6 +55,18 @@ def test_skip_unaligned_rows(kc):
     _check(kc, pts, 90, x=x)
 
 
+@pytest.mark.parametrize("sweep", ["f32", "bf16"])
+def test_skip_host_points(kc, sweep):
+    # pinned points are copied to the device rather than read in place
+    import torch
+    pts = I.gauss_mixture(30_001, 9, 714, 12, 0.5, -10.0, 10.0)
+    ref = O.gonzalez(pts, 300, mode="f32")
+    for x in (torch.from_numpy(pts).pin_memory(), torch.from_numpy(pts), pts):
+        r = kc.kc_gonzalez(x, 300, sweep=sweep)
+        assert np.asarray(r.centers).tolist() == ref.centers.tolist()
+        assert r.radius == O.radius(pts, ref.centers, mode="f64")[0]
+
+
 def test_skip_ties_duplicates_and_early_stop(kc):
     grid = I.int_points(30_000, 3, 712, 0, 4).astype(np.float32)   # 125 distinct points
     _check(kc, grid, 100)
