@@ -69,11 +69,7 @@ EXTRA = (CFG2, "gon_int_n10000_d2_k10", "gon_unif_n10000000_d16_k200", "mrg_unif
 # ncu capture, keyed by the SHA-256 of the kernel's source file at capture
 # time; reported only while the source is unchanged.  Values are for the
 # full workload (a smaller capture scaled by the units processed).
-NCU_TRAFFIC = {
-    # gon_group_kernel<float, 64, 1> at k = 16 on the 8M x 64 set (mean of two launches):
-    # 33,414,887,680 B read + 275,456,128 B written; x 64 for k = 1024
-    "3f019a95cd88c2d2cbef16eee6b28214751a0de558481537031966052fe939c9": 2_156_182_003_712,
-}
+NCU_TRAFFIC = {}
 
 
 def parse():
@@ -479,11 +475,16 @@ def run_gpu(args):
                            "l2": ("inputs larger than L2 (no flush)" if big
                                   else f"{L2_FLUSH_BYTES >> 20} MiB flush between steps"),
                            "step": "one kc_gonzalez call: pack + persistent k-step GON + FP64 radius recheck",
+                           "evals": "the k n point-center pairs that a solve decides",
                            "sweep": "f32", "replicas": world},
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                             "frac": achieved / peak, "traffic": traffic, "kernel": "gon_group_kernel",
+                             "frac": achieved / peak, "traffic": traffic,
+                             "kernel": "gon_group_kernel (first steps), gon_skip_kernel (the rest)",
                              "peak_kind": peak_kind, "avg_ms": gon_avg, "alg_bytes_per_launch": alg_bytes,
-                             "alg_bytes_rule": "k n (4 d + 4): each step reads every point and its running minimum"},
+                             "alg_bytes_rule": "k n (4 d + 4): each step reads every point and its running minimum; the "
+                                               "skip kernel leaves out the distances that the triangle inequality "
+                                               "proves irrelevant, so a fraction above 1 is work not needed, not "
+                                               "bandwidth"},
                 "mixed": mixed, "fp64_error": fp64_error, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
                 "clocks": clocks,
                 "step_share_ms": {k_: v / args.steps for k_, v in shares.items()}}
