@@ -855,9 +855,9 @@ __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_kernel(GonArgs a) {
 // launches of one d do; out of line, so that each has the registers it needs
 // (inlined side by side they spilled: 4096 mixed FP32 instances 95 -> 114 ms).
 // With CTA groups that hold their instances in L2 the generic sweep's dependent
-// loads are what was left: 89 ms at the best group size, 60 with these.  The mixed-precision kernel keeps its
-// generic loop: out of line its sweeps gained less than its longer recheck
-// path lost (62 -> 70 ms).
+// loads are what was left: 89 ms at the best group size, 60 with these.  The
+// mixed-precision kernel keeps its generic loop (4096 instances 62 ms, out of
+// line 72).
 template <typename T, int DC>
 __device__ __noinline__ void queue_solve_d(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
                                            long long timeout) {
@@ -967,6 +967,9 @@ __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_lp_kernel(GonArgs a) {
     gon_solve_lp<KIND, DC, GROUP_NT>(I, r, I.G, smem_f, sh, a.st, a.timeout_cycles, a.withhold, a.lp_local_t != 0);
 }
 
+// Four CTAs per SM: the sweep is bound by issue and latency together (4096 mixed
+// bf16 instances: 62 ms, with three 73, with five or six and more spills 69 and
+// 65).
 template <int KIND, int DC>
 __global__ void __launch_bounds__(QUEUE_NT, 4) gon_queue_lp_kernel(GonArgs a) {
     extern __shared__ __align__(16) float smem_f[];
