@@ -1806,10 +1806,10 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
 // once, and what did not fit there was left to single CTAs.  Measured on
 // mixed batches (d 3, 8, 32; k 8 to 128; GON launch alone, before / now, ms):
 //   instances x points         FP32           bf16
-//   4096 x 1k..200k          87.6 / 60.6    62.4 / 62.5
+//   4096 x 1k..200k          87.6 / 60.6    62.4 / 59.1
 //    512 x 1k..200k          17.8 /  8.2    25.4 / 13.4
 //     69 x 1k..200k           6.2 /  1.9    13.9 /  2.8
-//    905 x 1k..20k            2.6 /  1.9     3.9 /  3.2
+//    905 x 1k..20k            2.6 /  1.9     3.9 /  3.4
 // bf16 does not group by L2: it is issue-bound, with two exchanges a step
 // (4096: 62.5 -> 83 ms).
 //

@@ -536,7 +536,8 @@ __device__ __forceinline__ void lp_load_center(const GonInst &I, int64_t c, int 
     *ec = e;
 }
 
-template <int KIND, int DC, int NT>
+// UNR: words per point in flight in the generic loop (DC = 0).
+template <int KIND, int DC, int NT, int UNR = 2>
 __device__ void gon_solve_lp(const GonInst &I, int r, int G, float *smem, ShLP &sh, DevStatus *st, long long timeout,
                              int withhold = 0, bool local_t = false) {
     constexpr int W = NT / 32;
@@ -613,6 +614,7 @@ __device__ void gon_solve_lp(const GonInst &I, int r, int G, float *smem, ShLP &
                     }
                 }
             } else {
+#pragma unroll UNR
                 for (int jg = 0; jg < ng; ++jg) {
                     const uint4 w = __ldg(src + jg * (BLK / 4));
                     const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
@@ -857,7 +859,7 @@ __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_kernel(GonArgs a) {
 // With CTA groups that hold their instances in L2 the generic sweep's dependent
 // loads are what was left: 89 ms at the best group size, 60 with these.  The
 // mixed-precision kernel keeps its generic loop (4096 instances 62 ms, out of
-// line 72).
+// line 72; with four words in flight 59).
 template <typename T, int DC>
 __device__ __noinline__ void queue_solve_d(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
                                            long long timeout) {
@@ -991,7 +993,10 @@ __global__ void __launch_bounds__(QUEUE_NT, 4) gon_queue_lp_kernel(GonArgs a) {
         if (s_i >= a.ninst) return;
         copy_instance(I, a.insts + s_i);
         if (ld_volatile_i32(&a.st->code) != 0) return;
-        gon_solve_lp<KIND, DC, QUEUE_NT>(I, 0, 1, smem_f, sh, a.st, a.timeout_cycles);
+        // instances of single CTAs stream from memory: more loads in flight (4096
+        // mixed instances of up to 200k points 62.5 -> 59.1 ms, 905 of up to 20k
+        // 3.26 -> 3.41; in the groups above 512 of up to 200k 13.4 -> 14.1)
+        gon_solve_lp<KIND, DC, QUEUE_NT, 4>(I, 0, 1, smem_f, sh, a.st, a.timeout_cycles);
         __syncthreads();
     }
 }
