@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "kc_internal.cuh"
+#include "kc_nearest.cuh"
 
 namespace kc {
 
@@ -25,62 +26,16 @@ namespace {
 constexpr uint32_t NO_POINT = 0xFFFFFFFFu;
 
 // ----------------------------------------------------------------- assign
-// Nearest pivot of every point of the packed array (lowest on ties) and its
-// canonical distance.  A warp takes a block, its lanes four points each;
-// pivots go sixteen at a time (64 running sums), staged in shared memory.
-constexpr int AS_NT = 256, AS_C = 16;
+// Nearest pivot of every point of the packed array and its canonical distance
+// (three CTAs per SM for d = 2; with two EIM on 1M x 2 takes 1.76 ms, not 1.73).
 template <int DC>
-__global__ void __launch_bounds__(AS_NT, 2) cells_assign_kernel(const float *__restrict__ pk, int64_t n, int d_,
-                                                                const float *__restrict__ piv, int P,
-                                                                uint16_t *__restrict__ cell, uint32_t *__restrict__ dist) {
-    extern __shared__ __align__(16) float as_c[];   // [d][AS_C]
-    const int d = DC > 0 ? DC : d_;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t nb = nblocks(n);
-    for (int64_t g = blockIdx.x; g * (AS_NT / 32) < nb; g += gridDim.x) {
-        const int64_t b = g * (AS_NT / 32) + warp;
-        uint32_t m[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
-        uint32_t a[4] = {0u, 0u, 0u, 0u};
-        for (int c0 = 0; c0 < P; c0 += AS_C) {
-            __syncthreads();
-            for (int e = threadIdx.x; e < AS_C * d; e += AS_NT) {
-                const int c = c0 + e % AS_C, j = e / AS_C;
-                as_c[e] = c < P ? piv[(int64_t)c * d + j] : 0.f;
-            }
-            __syncthreads();
-            if (b >= nb) continue;
-            float acc[AS_C][4];
-#pragma unroll
-            for (int c = 0; c < AS_C; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.f;
-            const float4 *src = reinterpret_cast<const float4 *>(pk + b * d * BLK) + lane;
-#pragma unroll 4
-            for (int j = 0; j < d; ++j) {
-                const float4 v = __ldg(src + j * (BLK / 4));
-#pragma unroll
-                for (int c = 0; c < AS_C; ++c) {
-                    const float cc = as_c[j * AS_C + c];
-                    acc[c][0] = sq_step(acc[c][0], v.x, cc);
-                    acc[c][1] = sq_step(acc[c][1], v.y, cc);
-                    acc[c][2] = sq_step(acc[c][2], v.z, cc);
-                    acc[c][3] = sq_step(acc[c][3], v.w, cc);
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < AS_C; ++c)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint32_t s = __float_as_uint(acc[c][q]);
-                    if (c0 + c < P && s < m[q]) {
-                        m[q] = s;
-                        a[q] = (uint32_t)(c0 + c);
-                    }
-                }
-        }
-        if (b < nb) {
-            reinterpret_cast<uint4 *>(dist + b * BLK)[lane] = make_uint4(m[0], m[1], m[2], m[3]);
-            reinterpret_cast<uint2 *>(cell + b * BLK)[lane] = make_uint2(a[0] | (a[1] << 16), a[2] | (a[3] << 16));
-        }
-    }
+__global__ void __launch_bounds__(NEAREST_NT, DC == 2 ? 3 : 2) cells_assign_kernel(const float *__restrict__ pk, int64_t n, int d,
+                                                                     const float *__restrict__ piv, int P,
+                                                                     uint16_t *__restrict__ cell,
+                                                                     uint32_t *__restrict__ dist) {
+    extern __shared__ __align__(16) float as_c[];
+    const int dd = DC > 0 ? DC : d;
+    nearest_centers<DC>(pk, n, d, P, as_c, [=](int c, int j) { return __ldg(piv + (int64_t)c * dd + j); }, dist, cell);
 }
 
 // ------------------------------------------------------------------- sort
@@ -336,12 +291,11 @@ cudaError_t launch_pivot_rows(const float *rows, int64_t n, int d, const int64_t
 }
 
 cudaError_t launch_cells_assign(const float *pk, int64_t n, int d, const CellBufs &C, cudaStream_t s) {
-    const size_t smem = (size_t)AS_C * d * sizeof(float);
-    const int64_t groups = (nblocks(n) + AS_NT / 32 - 1) / (AS_NT / 32);
-    const int g = (int)std::min<int64_t>(groups, (int64_t)sm_count() * 8);
-    if (d == 64) cells_assign_kernel<64><<<g, AS_NT, smem, s>>>(pk, n, d, C.piv, C.P, C.cell, C.dist);
-    else if (d == 2) cells_assign_kernel<2><<<g, AS_NT, smem, s>>>(pk, n, d, C.piv, C.P, C.cell, C.dist);
-    else cells_assign_kernel<0><<<g, AS_NT, smem, s>>>(pk, n, d, C.piv, C.P, C.cell, C.dist);
+    const size_t smem = nearest_smem(d);
+    const int g = nearest_grid(n, sm_count());
+    if (d == 64) cells_assign_kernel<64><<<g, NEAREST_NT, smem, s>>>(pk, n, d, C.piv, C.P, C.cell, C.dist);
+    else if (d == 2) cells_assign_kernel<2><<<g, NEAREST_NT, smem, s>>>(pk, n, d, C.piv, C.P, C.cell, C.dist);
+    else cells_assign_kernel<0><<<g, NEAREST_NT, smem, s>>>(pk, n, d, C.piv, C.P, C.cell, C.dist);
     note_launches(1);
     return cudaGetLastError();
 }

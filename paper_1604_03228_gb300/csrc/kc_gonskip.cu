@@ -28,6 +28,7 @@
 #include <cstdlib>
 
 #include "kc_gon.cuh"
+#include "kc_nearest.cuh"
 
 namespace kc {
 
@@ -143,63 +144,14 @@ __global__ void __launch_bounds__(PROBE_NT) gon_probe_kernel(const float *__rest
 
 // ----------------------------------------------------------------- assign
 // Minimum over the first *route centers of every point of the packed array
-// (bits into mind) and the position of the center that gives it (asg, lowest
-// on ties).  A warp takes a block, its lanes four points each; centers go
-// sixteen at a time (64 running sums), staged in shared memory.
-constexpr int ASSIGN_NT = 256, ASSIGN_C = 16;
+// (into mind) and the position of the center that gives it (asg).
 template <int DC>
-__global__ void __launch_bounds__(ASSIGN_NT, 2) gon_assign_kernel(GonInst I, const int *route, const DevStatus *st) {
-    extern __shared__ __align__(16) float as_cen[];   // [d][ASSIGN_C]
+__global__ void __launch_bounds__(NEAREST_NT, 2) gon_assign_kernel(GonInst I, const int *route, const DevStatus *st) {
+    extern __shared__ __align__(16) float as_cen[];
     const int it0 = ld_volatile_i32(route);
     if (it0 == 0 || ld_volatile_i32(&st->code) != 0) return;
-    const int d = DC > 0 ? DC : I.d;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float *__restrict__ pk = (const float *)I.pk;
-    const int64_t nb = nblocks(I.n);
-    for (int64_t g = blockIdx.x; g * (ASSIGN_NT / 32) < nb; g += gridDim.x) {
-        const int64_t b = g * (ASSIGN_NT / 32) + warp;
-        uint32_t m[4] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
-        uint32_t a[4] = {0u, 0u, 0u, 0u};
-        for (int c0 = 0; c0 < it0; c0 += ASSIGN_C) {
-            __syncthreads();
-            for (int e = threadIdx.x; e < ASSIGN_C * d; e += ASSIGN_NT) {
-                const int c = c0 + e % ASSIGN_C, j = e / ASSIGN_C;
-                as_cen[e] = c < it0 ? I.cenT[(int64_t)j * I.kcap + c] : 0.f;
-            }
-            __syncthreads();
-            if (b >= nb) continue;
-            float acc[ASSIGN_C][4];
-#pragma unroll
-            for (int c = 0; c < ASSIGN_C; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.f;
-            const float4 *src = reinterpret_cast<const float4 *>(pk + b * d * BLK) + lane;
-#pragma unroll 4
-            for (int j = 0; j < d; ++j) {
-                const float4 v = __ldg(src + j * (BLK / 4));
-#pragma unroll
-                for (int c = 0; c < ASSIGN_C; ++c) {
-                    const float cc = as_cen[j * ASSIGN_C + c];
-                    acc[c][0] = sq_step(acc[c][0], v.x, cc);
-                    acc[c][1] = sq_step(acc[c][1], v.y, cc);
-                    acc[c][2] = sq_step(acc[c][2], v.z, cc);
-                    acc[c][3] = sq_step(acc[c][3], v.w, cc);
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < ASSIGN_C; ++c)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint32_t s = __float_as_uint(acc[c][q]);
-                    if (c0 + c < it0 && s < m[q]) {
-                        m[q] = s;
-                        a[q] = (uint32_t)(c0 + c);
-                    }
-                }
-        }
-        if (b < nb) {   // rows past n are written too (padding, never read as points)
-            reinterpret_cast<uint4 *>(I.mind + b * BLK)[lane] = make_uint4(m[0], m[1], m[2], m[3]);
-            reinterpret_cast<uint2 *>(I.asg + b * BLK)[lane] = make_uint2(a[0] | (a[1] << 16), a[2] | (a[3] << 16));
-        }
-    }
+    nearest_centers<DC>((const float *)I.pk, I.n, I.d, it0, as_cen,
+                        [&](int c, int j) { return I.cenT[(int64_t)j * I.kcap + c]; }, I.mind, I.asg);
 }
 
 // The first *route centers' coordinates, transposed ([d][kcap]).
@@ -811,11 +763,10 @@ cudaError_t launch_gon_skip(GonArgs &a, int last, cudaStream_t s) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     gon_center_rows_kernel<<<(int)std::min<int64_t>(sms, ((int64_t)last * I.d + 255) / 256), 256, 0, s>>>(I, a.route, a.st);
-    const size_t asm_ = (size_t)ASSIGN_C * I.d * sizeof(float);
-    const int64_t groups = (nblocks(I.n) + ASSIGN_NT / 32 - 1) / (ASSIGN_NT / 32);
-    const int ga = (int)std::min<int64_t>(groups, (int64_t)sms * 8);
-    if (I.d == 64) gon_assign_kernel<64><<<ga, ASSIGN_NT, asm_, s>>>(I, a.route, a.st);
-    else gon_assign_kernel<0><<<ga, ASSIGN_NT, asm_, s>>>(I, a.route, a.st);
+    const size_t smem_a = nearest_smem(I.d);
+    const int ga = nearest_grid(I.n, sms);
+    if (I.d == 64) gon_assign_kernel<64><<<ga, NEAREST_NT, smem_a, s>>>(I, a.route, a.st);
+    else gon_assign_kernel<0><<<ga, NEAREST_NT, smem_a, s>>>(I, a.route, a.st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     void *fn = pick_skip(I.d);

@@ -41,6 +41,32 @@ def test_skip_equals_oracle(kc, n, d, k, shape):
     _check(kc, pts, k, first=n // 3)
 
 
+@pytest.mark.parametrize("n,d,k", [(4_000, 256, 40), (4_000, 257, 40), (3_000, 768, 30), (3_000, 769, 30),
+                                   (2_500, 1100, 70), (1_500, 3700, 30)])
+def test_skip_large_d(kc, n, d, k):
+    # the assignment stages centers in parts of 256 coordinates
+    _check(kc, I.gauss_mixture(n, d, 720 + d, 20, 0.5, -10.0, 10.0), k, first=5)
+
+
+@pytest.mark.parametrize("sweep", ["f32", "bf16"])
+@pytest.mark.parametrize("shape", ["gau", "unif"])
+def test_skip_large_d_with_the_default_switches(kc, monkeypatch, shape, sweep):
+    # large enough for the segments by itself (n d k >= 1e10): the same as the
+    # streaming kernels, whether it changes over or not
+    import torch
+    n, d, k = 200_000, 1024, 64
+    g = torch.Generator(device="cuda").manual_seed(730)
+    x = torch.randn(n, d, generator=g, device="cuda")
+    if shape == "gau":
+        x += 20.0 * torch.rand(10, d, generator=g, device="cuda")[torch.randint(0, 10, (n,), generator=g, device="cuda")]
+    monkeypatch.delenv("KC_GON_SKIP")
+    a = kc.kc_gonzalez(x, k, sweep=sweep)
+    monkeypatch.setenv("KC_GON_SKIP", "0")
+    b = kc.kc_gonzalez(x, k, sweep=sweep)
+    assert a.centers.cpu().tolist() == b.centers.cpu().tolist() and (a.k_out, a.radius) == (b.k_out, b.radius)
+    assert kc.kc_radius(x, a.centers).radius == a.radius
+
+
 @pytest.mark.parametrize("sweep", ["bf16", "fp16", "fp8"])
 def test_skip_behind_a_low_precision_sweep(kc, sweep):
     _check(kc, I.gauss_mixture(40_000, 24, 710, 30, 0.5, -10.0, 10.0), 120, sweep=sweep)
