@@ -1383,11 +1383,25 @@ static size_t smem_for(int dtype, int lp, int dmax, bool queue) {
     return (size_t)(dmax > 0 ? dmax : 1) * 4;
 }
 
-// Occupancy of a GON kernel with its dynamic shared memory (opted in first
-// when above the default 48 KB).
+// A kernel whose static and dynamic shared memory together exceed the default
+// 48 KB is opted in to its dynamic part (the static one is below 2 KB in all of
+// them; with a limit on the dynamic part alone the mixed-precision kernels were
+// refused for 1925 <= d <= 2048).
+static cudaError_t opt_in_smem(void *fn, size_t smem) {
+    constexpr size_t STATIC_MAX = 4096;
+    static_assert(sizeof(ShLP) + sizeof(GonInst) + 64 <= STATIC_MAX && sizeof(ShRes) + sizeof(GonInst) + 64 <= STATIC_MAX,
+                  "static shared memory");
+    if (smem + STATIC_MAX <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
+// Occupancy of a GON kernel with its dynamic shared memory.
 static int gon_occupancy(void *fn, int nt, size_t smem) {
-    if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 0;
+    if (opt_in_smem(fn, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, nt, smem) != cudaSuccess) {
         cudaGetLastError();
         occ = 0;
@@ -1436,7 +1450,7 @@ int gon_resident_plan(int dtype, int d, int64_t n, int *cap, int *slot_words) {
     const int64_t c = npmax > GROUP_NT ? npmax - GROUP_NT : 1;
     const size_t smem = (size_t)c * d * 4;
     if (smem + sizeof(ShRes) + 1024 > (size_t)optin) return 0;
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (opt_in_smem(fn, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1456,10 +1470,7 @@ cudaError_t launch_gon(GonArgs &a, cudaStream_t s) {
         void *fn = pick_resident(a.dtype, a.dc);
         if (!fn) return cudaErrorInvalidValue;
         const size_t smem = (size_t)a.res_cap * a.dc * 4;
-        if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
+        if (const cudaError_t e = opt_in_smem(fn, smem)) return e;
         note_launches(1);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(a.grid);
@@ -1476,10 +1487,7 @@ cudaError_t launch_gon(GonArgs &a, cudaStream_t s) {
     }
     const size_t smem = smem_for(a.dtype, a.lp_kind, a.dmax, a.queue != 0);
     void *fn = pick_fn(a.dtype, a.lp_kind, a.dc, a.queue != 0, a.dyn != 0, a.grid > LEADER_MIN);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = opt_in_smem(fn, smem)) return e;
     note_launches(1);
     // Groups that wait on one another need a cooperative launch (all CTAs
     // co-resident); the attribute form is also accepted by stream capture.

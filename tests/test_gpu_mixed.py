@@ -131,3 +131,26 @@ def test_lp_rechecks_read_rows_or_packed_copy(kc):
         same(kc.kc_gonzalez(unal, 120, sweep=sw), ref)
         r = kc.kc_gonzalez(hp, 120, sweep=sw)
         assert r.centers.tolist() == ref.centers.cpu().tolist() and r.radius == ref.radius
+
+
+@pytest.mark.parametrize("d", [1924, 1925, 1937, 2000, 2047, 2048, 2049])
+@pytest.mark.parametrize("sweep", SWEEPS)
+def test_lp_shared_memory_around_48_kb(kc, sweep, d):
+    # the group kernels' dynamic shared memory (32 KB and 8 bytes a coordinate)
+    # passes 48 KB at d = 2048, with the static part at d = 1925
+    x = _dev(I.gauss_mixture(600, d, 511, 6, 0.5, -10, 10))
+    same(kc.kc_gonzalez(x, 30, sweep=sweep), kc.kc_gonzalez(x, 30))
+
+
+def test_shared_memory_around_48_kb_batch_and_f32(kc):
+    xs = [_dev(I.gauss_mixture(150 + i, d, 512 + i, 4, 0.5, -10, 10)) for i, d in enumerate((4994, 5000, 5100, 5120))]
+    for xd in ([xs[1]], xs):
+        for a, b in zip(kc.kc_gonzalez_batch(xd, [12] * len(xd), sweep="bf16"), kc.kc_gonzalez_batch(xd, [12] * len(xd))):
+            same(a, b)
+    for d in (12_100, 12_200, 12_288, 12_289):
+        pts = I.gauss_mixture(300, d, 520, 4, 0.5, -10, 10)
+        ref = O.gonzalez(pts, 12, mode="f32")
+        assert kc.kc_gonzalez(_dev(pts), 12).centers.cpu().tolist() == ref.centers.tolist()
+    for n in (2214, 2230, 2252, 2253):   # the resident kernel's columns
+        pts = I.gauss_mixture(n, 10, 521, 4, 0.5, -10, 10)
+        assert kc.kc_gonzalez(_dev(pts), 40).centers.cpu().tolist() == O.gonzalez(pts, 40, mode="f32").centers.tolist()
