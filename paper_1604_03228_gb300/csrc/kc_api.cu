@@ -86,11 +86,11 @@ kc_status fail(kc_status s, const char *fmt, ...) {
     return s;
 }
 
+// The error is taken from CUDA's own record too: the launchers read that record
+// after theirs, and a refused call's error would be reported by the next one.
 kc_status cuda_fail(cudaError_t e, const char *what) {
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        return fail(KC_ERR_OOM, "%s: %s", what, cudaGetErrorString(e));
-    }
+    cudaGetLastError();
+    if (e == cudaErrorMemoryAllocation) return fail(KC_ERR_OOM, "%s: %s", what, cudaGetErrorString(e));
     return fail(KC_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 

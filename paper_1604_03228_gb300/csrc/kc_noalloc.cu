@@ -60,7 +60,10 @@ kc_status na_fail(kc_status s, const char *fmt, ...) {
 #define NA_CUDA(call, what)                                                                   \
     do {                                                                                      \
         cudaError_t e_ = (call);                                                              \
-        if (e_ != cudaSuccess) return na_fail(KC_ERR_CUDA, "%s: %s", (what), cudaGetErrorString(e_)); \
+        if (e_ != cudaSuccess) {                                                              \
+            cudaGetLastError();                                                               \
+            return na_fail(KC_ERR_CUDA, "%s: %s", (what), cudaGetErrorString(e_));            \
+        }                                                                                     \
     } while (0)
 
 // Device address of the static array for the current device (looked up once

@@ -440,3 +440,19 @@ def test_fp32_radius_against_fp64_per_result(kc):
     ipts = I.gon_int_10k().points
     gi = kc.kc_gonzalez(_dev(ipts), 10)
     assert kc.kc_last_fp32_radius() == gi.radius
+
+
+@pytest.mark.parametrize("noalloc", [False, True])
+def test_refused_launch_leaves_no_error_behind(kc, noalloc):
+    # 240 KB of coordinates of one center pass an SM's shared memory: the call
+    # is refused, and the next one is not told so again
+    big = _dev(I.gauss_mixture(64, 60_000, 31, 4, 0.5, -10, 10))
+    pts = I.gauss_mixture(3000, 5, 32, 4, 0.5, -10, 10)
+    x = _dev(pts)
+    solve = kc.kc_gonzalez_noalloc if noalloc else kc.kc_gonzalez
+    ref = O.gonzalez(pts, 9, mode="f32").centers.tolist()
+    assert solve(x, 9).centers.cpu().tolist() == ref
+    with pytest.raises(kc.KCError) as e:
+        solve(big, 8)
+    assert e.value.status == kc.KC_ERR_CUDA
+    assert solve(x, 9).centers.cpu().tolist() == ref
