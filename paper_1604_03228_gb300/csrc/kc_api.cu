@@ -2240,7 +2240,12 @@ kc_status batch_check(int32_t count, const void *const *pts, const int64_t *n, c
     if (b.lp == KC_SWEEP_FP8 || b.lp == KC_SWEEP_FP16)
         return fail(KC_ERR_ARG,
                     "the batched form takes KC_SWEEP_F32 or KC_SWEEP_BF16 (fp8 and fp16 need per-instance scales)");
-    b.dc = (dcommon == 3 || dcommon == 8 || dcommon == 32) && o.dtype == KC_F32 ? dcommon : 0;
+    // 0: several d, and a single one for which that kernel's loops of 128
+    // registers are the faster ones (two CTAs per SM against four, ms: 600
+    // instances of up to 50k points d = 10 6.6 / 5.5, 24 12.1 / 13.6, 37 20.8 /
+    // 27.9, 64 44.3 / 52.5; 100 of up to 100k d = 80 23.8 / 22.4, 128 34.5 / 34.1;
+    // 1791 of up to 1000 d = 10 0.64 / 0.44, 24 0.84 / 0.74, 37 1.21 / 1.17)
+    b.dc = dcommon > 24 && dcommon < 96 && dcommon != 32 ? 0 : dcommon;
     b.dmax = dmax;
     return KC_OK;
 }

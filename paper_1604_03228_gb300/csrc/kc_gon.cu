@@ -68,7 +68,7 @@ __device__ __forceinline__ void pc_publish(const long long *c) {
 namespace {
 
 // One step's sweep of this CTA's share (rank r of G) of [lo, lo + n).
-template <typename T, int DC, int NT>
+template <typename T, int DC, int NT, int UNR>
 __device__ __forceinline__ uint64_t sweep(const T *__restrict__ pk, uint32_t *__restrict__ mind,
                                           int64_t lo, int64_t n, int d, const T *cs, bool first_step,
                                           int r, int G, int *ctr, int *gtail) {
@@ -99,7 +99,7 @@ __device__ __forceinline__ uint64_t sweep(const T *__restrict__ pk, uint32_t *__
             }
         }
         typename AccOf<T>::type acc[4];
-        dist4<T, DC>(pk + b * d * BLK, d, cs, lane, acc);
+        dist4<T, DC, UNR>(pk + b * d * BLK, d, cs, lane, acc);
         uint32_t m[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) m[q] = min(o[q], acc_bits(acc[q]));
@@ -160,8 +160,12 @@ struct Shared {
 // the instance is large enough for claimed blocks and the shared tail (a
 // separate instantiation, so that small instances run the plain loop).  LEAD:
 // the exchange may go through the leader (its own instantiation as well: one
-// CTA on 3608 x 16 takes 2.35 us a step without its code, 2.73 with it).
-template <typename T, int DC, int NT, bool DYN = false, bool LEAD = false>
+// CTA on 3608 x 16 takes 2.35 us a step without its code, 2.73 with it).  UNR:
+// coordinates in flight in the generic loop, 8 in queue launches of one d (MRG
+// on 2M x 64 with 4 / 8: 20.0 / 18.4 ms, int32 29.7 / 28.7; batches of int32
+// 1791 x 64 2.64 / 2.31), 4 elsewhere (streaming float 4M x 40 110 / 119 us a
+// step, batches through the kernel of several d at d = 37 20.9 / 22.9 ms).
+template <typename T, int DC, int NT, bool DYN = false, bool LEAD = false, int UNR = 4>
 __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
                           long long timeout, int withhold = 0, bool bad_index = false) {
     constexpr int W = NT / 32;
@@ -195,15 +199,14 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
     const bool lead = LEAD && G > LEADER_MIN && I.bc != nullptr &&
                       (I.lo + I.n - 1) / BLK - I.lo / BLK + 1 < 4 * (int64_t)G * W;
 
-    const int it1 = I.it1;
     int it;
     uint64_t K = 0;
-    for (it = I.it0; it < it1; ++it) {
+    for (it = I.it0; it < I.it1; ++it) {
         // claimed blocks in the 1024-thread group CTAs when every warp has
         // several (measured: GON on 8M x 64, k = 1024, 313 -> 308 ms); the
         // fixed assignment in the 256-thread queue CTAs (MRG round 1 on
         // 10M x 16 was 5% slower with claims) and for small instances
-        uint64_t best = sweep<T, DC, NT>(pk, I.mind, I.lo, I.n, d, cs, it == 0, r, G,
+        uint64_t best = sweep<T, DC, NT, UNR>(pk, I.mind, I.lo, I.n, d, cs, it == 0, r, G,
                                          claim ? &sh.ctr[it & 1] : nullptr, tail ? I.tail + it : nullptr);
         best = warp_max_u64(best);
         if (lane == 0) sh.red[warp] = best;
@@ -214,7 +217,7 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
             v = warp_max_u64(v);
             uint64_t g = v;
             bool ab = false;
-            const bool more = it + 1 < it1;
+            const bool more = it + 1 < I.it1;
             const uint64_t tagw = (uint64_t)(it + 1) << 32;
             if (G > 1) {
                 uint64_t *row = I.slots + (int64_t)it * slot_stride(G);
@@ -853,22 +856,27 @@ __global__ void __launch_bounds__(GROUP_NT, 1) gon_group_kernel(GonArgs a) {
     gon_solve<T, DC, GROUP_NT, DYN, LEAD>(I, r, I.G, cs, sh, a.st, a.timeout_cycles, a.withhold, a.bad_index != 0);
 }
 
-// A launch of mixed d solves each instance with the sweep made for its d, as
-// launches of one d do; out of line, so that each has the registers it needs
-// (inlined side by side they spilled: 4096 mixed FP32 instances 95 -> 114 ms).
-// With CTA groups that hold their instances in L2 the generic sweep's dependent
-// loads are what was left: 89 ms at the best group size, 60 with these.  The
-// mixed-precision kernel keeps its generic loop (4096 instances 62 ms, out of
-// line 72; with four words in flight 59).
+// A batch of several d (MIX) solves each instance with the sweep made for its
+// d, as launches of one d do; out of line, so that each has the registers it
+// needs (inlined side by side they spilled: 4096 mixed FP32 instances 95 -> 114
+// ms).  With CTA groups that hold their instances in L2 the generic sweep's
+// dependent loads are what was left: 89 ms at the best group size, 60 with
+// these.  The calls cost registers (128 a thread, two CTAs per SM, against 64
+// and four), so launches of one d have an instantiation without them: MRG, whose
+// round 1 streams from memory, with the calls / without: 10M x 2 7.9 / 4.9 ms,
+// 10M x 10 21.9 / 17.2, 4M x 37 25.0 / 21.5, 2M x 64 20.9 / 19.9.
+// The mixed-precision kernel keeps its generic loop (4096 instances 62 ms, out
+// of line 72; with four words in flight 59).
 template <typename T, int DC>
 __device__ __noinline__ void queue_solve_d(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
                                            long long timeout) {
     gon_solve<T, DC, QUEUE_NT>(I, r, G, cs, sh, st, timeout);
 }
-template <typename T, int DC>
+template <typename T, int DC, bool MIX>
 __device__ __forceinline__ void queue_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
                                             long long timeout) {
-    if constexpr (DC == 0 && std::is_same<T, float>::value) {
+    if constexpr (MIX) {
+        static_assert(DC == 0, "a launch of several d");
         switch (I.d) {
             case 3: queue_solve_d<T, 3>(I, r, G, cs, sh, st, timeout); return;
             case 8: queue_solve_d<T, 8>(I, r, G, cs, sh, st, timeout); return;
@@ -877,7 +885,7 @@ __device__ __forceinline__ void queue_solve(const GonInst &I, int r, int G, T *c
             default: queue_solve_d<T, 0>(I, r, G, cs, sh, st, timeout); return;
         }
     } else {
-        gon_solve<T, DC, QUEUE_NT>(I, r, G, cs, sh, st, timeout);
+        gon_solve<T, DC, QUEUE_NT, false, false, 8>(I, r, G, cs, sh, st, timeout);
     }
 }
 
@@ -929,7 +937,7 @@ __device__ __forceinline__ bool join_group(const GonInst &I, long long timeout, 
 // CTAs (the launch is then cooperative, so the groups are co-resident); a CTA
 // solves those whose group it is in, in order; every CTA then takes the
 // remaining instances insts[nheavy, ninst) one at a time, in order.
-template <typename T, int DC>
+template <typename T, int DC, bool MIX>
 __global__ void __launch_bounds__(QUEUE_NT) gon_queue_kernel(GonArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *cs = reinterpret_cast<T *>(smem_raw);
@@ -941,7 +949,7 @@ __global__ void __launch_bounds__(QUEUE_NT) gon_queue_kernel(GonArgs a) {
             copy_instance(I, a.insts + q);
             if (!join_group(I, a.timeout_cycles, a.st)) return;
             if (instance_ok<T>(I, a.st))
-                queue_solve<T, DC>(I, (int)blockIdx.x - I.cta0, I.G, cs, sh, a.st, a.timeout_cycles);
+                queue_solve<T, DC, MIX>(I, (int)blockIdx.x - I.cta0, I.G, cs, sh, a.st, a.timeout_cycles);
             __syncthreads();
         }
     }
@@ -951,7 +959,7 @@ __global__ void __launch_bounds__(QUEUE_NT) gon_queue_kernel(GonArgs a) {
         if (s_i >= a.ninst) return;
         copy_instance(I, a.insts + s_i);
         if (ld_volatile_i32(&a.st->code) != 0) return;
-        if (instance_ok<T>(I, a.st)) queue_solve<T, DC>(I, 0, 1, cs, sh, a.st, a.timeout_cycles);
+        if (instance_ok<T>(I, a.st)) queue_solve<T, DC, MIX>(I, 0, 1, cs, sh, a.st, a.timeout_cycles);
         __syncthreads();
     }
 }
@@ -1277,7 +1285,7 @@ void *pick_resident(int dtype, int d) {
 }
 
 template <typename T, int DC, bool DYN, bool LEAD> void *group_fn() { return (void *)gon_group_kernel<T, DC, DYN, LEAD>; }
-template <typename T, int DC> void *queue_fn() { return (void *)gon_queue_kernel<T, DC>; }
+template <typename T, int DC, bool MIX = false> void *queue_fn() { return (void *)gon_queue_kernel<T, DC, MIX>; }
 template <int KIND, int DC> void *group_lp_fn() { return (void *)gon_group_lp_kernel<KIND, DC>; }
 template <int KIND, int DC> void *queue_lp_fn() { return (void *)gon_queue_lp_kernel<KIND, DC>; }
 
@@ -1345,9 +1353,10 @@ void *pick_group(int dtype, int dc, bool dyn, bool lead) {
     return lead ? pick_group_f32<false, true>(dc) : pick_group_f32<false, false>(dc);
 }
 
-void *pick_queue(int dtype, int dc) {
+void *pick_queue(int dtype, int dc) {   // dc = 0: several d
     if (dtype == KC_F32) {
         switch (dc) {
+            case 0: return queue_fn<float, 0, true>();
             case 3: return queue_fn<float, 3>();
             case 8: return queue_fn<float, 8>();
             case 16: return queue_fn<float, 16>();

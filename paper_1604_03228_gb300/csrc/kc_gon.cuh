@@ -27,7 +27,8 @@ __device__ __forceinline__ void st_relaxed_u64(uint64_t *p, uint64_t v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-template <typename T, int DC>
+// UNR: coordinates in flight in the generic loop (DC = 0).
+template <typename T, int DC, int UNR = 4>
 __device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T *cs, int lane,
                                       typename AccOf<T>::type acc[4]) {
     using V4 = typename Vec4<T>::type;
@@ -45,7 +46,7 @@ __device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T 
             a3 = sq_step(a3, v.w, c);
         }
     } else {
-#pragma unroll 4
+#pragma unroll UNR
         for (int j = 0; j < d; ++j) {
             const V4 v = __ldg(src + j * (BLK / 4));
             const T c = cs[j];

@@ -76,3 +76,24 @@ def test_batch_groups_keep_scratch(kc, monkeypatch, sweep):
     kc.kc_batch_plan_run(plan)
     assert [(r.centers.cpu().tolist(), r.k_out, r.radius) for r in kc.kc_batch_plan_wait(plan)] == got
     kc.kc_batch_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("d,integer", [(2, False), (10, False), (16, False), (24, False), (100, False), (7, True), (64, True)])
+def test_one_d_batches_keep_four_ctas_per_sm(kc, d, integer):
+    """A batch of one d has a kernel of its own, not the one of several d with
+    its loops out of line (128 registers a thread): as many CTAs as at d = 8."""
+    import torch
+
+    def solve(dd):
+        make = (lambda i: I.int_points(200, dd, 60 + i, -99, 99)) if integer else (lambda i: I.gauss_mixture(200, dd, 60 + i, 5, 0.2, 0, 1))
+        pts = [make(i % 7) for i in range(2000)]
+        plan = kc.kc_batch_plan_create([torch.from_numpy(p).cuda() for p in pts], [9] * len(pts))
+        grid = kc.kc_batch_plan_info(plan)[3]
+        kc.kc_batch_plan_run(plan)
+        got = [r.centers.cpu().tolist() for r in kc.kc_batch_plan_wait(plan)]
+        kc.kc_batch_plan_destroy(plan)
+        assert got[:7] == [O.gonzalez(p, 9, mode="i64" if integer else "f32").centers.tolist() for p in pts[:7]]
+        assert all(g == got[i % 7] for i, g in enumerate(got))
+        return grid
+
+    assert solve(d) == solve(8)
