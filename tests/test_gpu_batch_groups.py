@@ -97,3 +97,19 @@ def test_one_d_batches_keep_four_ctas_per_sm(kc, d, integer):
         return grid
 
     assert solve(d) == solve(8)
+
+
+@pytest.mark.parametrize("integer,d", [(False, 10), (False, 24), (False, 25), (False, 64), (False, 95), (False, 96),
+                                       (False, 130), (True, 47), (True, 48)])
+def test_one_d_batch_groups_match_queue(kc, monkeypatch, integer, d):
+    """Around the lines between the kernels (d = 24 and 96) and of the grouping
+    by L2 (96, int32 48)."""
+    import torch
+    insts, ks = _batch(700, (d,), 3, integer, 7100 + d)
+    xs = [torch.from_numpy(p).cuda() for p in insts]
+    got = [(r.centers.cpu().tolist(), r.k_out, r.radius) for r in kc.kc_gonzalez_batch(xs, ks)]
+    monkeypatch.setenv("KC_BATCH_THETA", "inf")
+    assert [(r.centers.cpu().tolist(), r.k_out, r.radius) for r in kc.kc_gonzalez_batch(xs, ks)] == got
+    for i in range(11):
+        o = O.gonzalez(insts[i], ks[i], mode="i64" if integer else "f32")
+        assert got[i][0] == o.centers.tolist()
