@@ -490,7 +490,7 @@ cudaError_t launch_gon_segments(GonArgs &g, const int *ends, int nseg, int *rout
         g.single.it1 = i < nseg ? ends[i] : 0;
         e = launch_gon(g, s);
         if (i < nseg && e == cudaSuccess)
-            e = launch_gon_probe(g.single, ends[i], route, (unsigned *)route + 4, g.st, s);
+            e = launch_gon_probe(g.single, ends[i], i == nseg - 1, route, (unsigned *)route + 4, g.st, s);
     }
     if (nseg && e == cudaSuccess) e = launch_gon_skip(g, ends[nseg - 1], s);
     return e;

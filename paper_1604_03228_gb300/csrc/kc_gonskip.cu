@@ -46,10 +46,20 @@ constexpr int SKIP_TILE = UNIT * 33;    // words of a warp's transpose tile
 // last CTA then bins the sample as the regrouping would (by a, near or far)
 // and counts the points in bins that the newest center c (the winner of step
 // it0 - 1) touches: d(a, c) < 2 sqrt(largest m of the bin).  With that share
-// of the points touched per step, a step is expected to take
-//   fixed_us + share^2 unit_us (the share falls as clusters get centers),
-// and the change-over (assignment, two regroupings) `once` microseconds; *route
-// is set to it0 when that saves at least a tenth of the remaining steps' time.
+// of the points touched a step takes fixed_us + share unit_us, the change-over
+// (assignment, two regroupings) `once`.  What becomes of the share:
+//  - where a fifth of the points or more are near (m at most a quarter of the
+//    largest), the centers so far cover that part of the clusters, a new one
+//    touches the other points only, and covering them takes about it0 (1 / near
+//    - 1) more steps, over which the share falls to the few points of a cluster
+//    (where nearly all are, outliers are being taken, and the others are still
+//    to show what they are: a tenth);
+//  - elsewhere (no clusters, or each has its center) it stays about what it is.
+// *route is set to it0 when the steps left would take a tenth less time that
+// way and the next ones no longer than a sweep (at the last probe they may, if
+// all together take a seventh less).  Taking the share to fall on any points (its square) cost 10M x 8
+// uniform, k = 500, 61 ms against 30, and one cluster of 10M x 10, k = 1024, 152
+// against 72; there is no way back.
 constexpr int PROBE_NT = 256, PROBE_CTAS = 128, PROBE_S = PROBE_CTAS * PROBE_NT / 32;
 constexpr int PROBE_MAX = 256;         // most centers at a probe
 
@@ -75,9 +85,9 @@ __device__ __forceinline__ float row_dist_any(const float *__restrict__ x, const
 __global__ void __launch_bounds__(PROBE_NT) gon_probe_kernel(const float *__restrict__ rm,
                                                              const int64_t *__restrict__ rmap, int64_t n, int d,
                                                              const int64_t *__restrict__ centers, const uint64_t *key,
-                                                             int it0, float sweep_us, float unit_us, float fixed_us, float once_us, int left,
-                                                             int *route, unsigned *done, uint2 *sample,
-                                                             const DevStatus *st) {
+                                                             int it0, float sweep_us, float unit_us, float fixed_us,
+                                                             float once_us, int left, bool last_probe, int *route,
+                                                             unsigned *done, uint2 *sample, const DevStatus *st) {
     if (ld_volatile_i32(&st->code) != 0 || ld_volatile_i32(route) != 0) return;
     const uint64_t K = *key;
     if (key_val(K) == 0) return;   // the solve has stopped early
@@ -121,24 +131,33 @@ __global__ void __launch_bounds__(PROBE_NT) gon_probe_kernel(const float *__rest
         if (s.y < (uint32_t)it0) atomicMax(&rmax[2 * s.y + (s.x > far)], s.x);
     }
     __syncthreads();
-    int touched = 0, total = 0;
+    int touched = 0, total = 0, near = 0;
     for (int q = threadIdx.x; q < PROBE_S; q += PROBE_NT) {
         const uint2 s = __ldcg(sample + q);
         if (s.y >= (uint32_t)it0) continue;
         ++total;
+        near += s.x <= far;
         touched += dc[s.y] < 2.f * sqrtf(__uint_as_float(rmax[2 * s.y + (s.x > far)]));
     }
-    __shared__ int sum[2];
-    if (threadIdx.x < 2) sum[threadIdx.x] = 0;
+    __shared__ int sum[3];
+    if (threadIdx.x < 3) sum[threadIdx.x] = 0;
     __syncthreads();
     atomicAdd(&sum[0], touched);
     atomicAdd(&sum[1], total);
+    atomicAdd(&sum[2], near);
     __syncthreads();
     if (threadIdx.x == 0) {
         *done = 0u;   // ready for the next probe
-        const float share = (float)sum[0] / (float)max(sum[1], 1);
-        const float save = (float)left * (sweep_us - share * share * unit_us - fixed_us) - once_us;
-        if (save > 0.1f * (float)left * sweep_us) *route = it0;
+        const float share = (float)sum[0] / (float)max(sum[1], 1), nearf = (float)sum[2] / (float)max(sum[1], 1);
+        float later = share;   // mean over the steps left
+        if (nearf >= 0.2f) {
+            const float cover = (float)it0 * (1.f / nearf - 1.f), l = (float)left;
+            later *= fmaxf(l < cover ? 1.f - 0.5f * l / cover : 0.5f * cover / l, 0.1f);
+            if (nearf > 0.9f) later = fmaxf(later, 0.1f);
+        }
+        const float save = (float)left * (sweep_us - later * unit_us - fixed_us) - once_us;
+        const bool soon = share * unit_us + fixed_us <= 1.1f * sweep_us;   // from the next step on
+        if ((soon || last_probe) && save > (soon ? 0.1f : 0.15f) * (float)left * sweep_us) *route = it0;
     }
 }
 
@@ -739,20 +758,29 @@ bool gon_skip_possible(int dtype, int d, int64_t n, int k, int grid) {
     return gon_skip_segments(dtype, d, n, k, grid, ends, 8) > 0;
 }
 
-cudaError_t launch_gon_probe(const GonInst &I, int it0, int *route, unsigned *words, DevStatus *st, cudaStream_t s) {
-    // microseconds: a whole sweep at the HBM rate (half the bytes in mixed
-    // precision), the assignment at the FP32 rate and two regroupings
-    const double n = (double)I.n;
-    const float sweep = (float)(n * (I.d * (I.lp_kind ? 2.0 : 4.0) + 4.0) / 6.9e6);
+cudaError_t launch_gon_probe(const GonInst &I, int it0, bool last, int *route, unsigned *words, DevStatus *st,
+                             cudaStream_t s) {
+    // microseconds: a whole sweep at the HBM rate, or the one of L2 where the
+    // points stay there (half the bytes in mixed precision), the assignment at
+    // the FP32 rate and two regroupings
+    const double n = (double)I.n, bytes = n * (I.d * (I.lp_kind ? 2.0 : 4.0) + 4.0);
+    const float sweep = (float)(bytes / (bytes < 100e6 ? 14e6 : 6.9e6));
     // all units touched: perm and assignment too, and less even than a sweep
-    // (8M x 64: a quarter of the units in 90 us)
-    const float unit = (float)(1.25 * n * (I.d * 4.0 + 12.0) / 6.9e6);
+    // (8M x 64: a quarter of the units in 90 us); or a warp's waits, about 2 us
+    // for a unit's first batch of loads and 1 for each further one (a tenth of the
+    // units of 10M x 10, one batch, in 26 us, of 4M x 32, two, in 12)
+    const int batches = I.d / 64 + (I.d % 64 + 15) / 16;
+    const float unit = (float)std::max(1.25 * n * (I.d * 4.0 + 12.0) / 6.9e6,
+                                       n / UNIT / (SKIP_W * (double)I.G) * (1.0 + batches));
     const float once = (float)(n * I.d * it0 / 1.2e7 + 2.0 * n * (8.0 * I.d + 100.0) / 4e6 + 60.0);
     const char *env = getenv("KC_GON_SKIP");   // testing: 1 = change over at the first probe
     const bool force = env && atoi(env) > 0;
-    const float fixed = (float)(8.0 + n / 2e6);   // beyond a streaming step's, with the tests of all units
+    // beyond a streaming step's exchange, with the tests of all units (10M x 10, a tenth
+    // of the units touched: 36 us a step, 26 of them the units, 3.5 the exchange)
+    const float fixed = (float)(3.0 + n / 2e6);
     gon_probe_kernel<<<PROBE_CTAS, PROBE_NT, 0, s>>>(I.rm, I.rmap, I.n, I.d, I.centers, I.final_key, it0,
-                                                     force ? 1e9f : sweep, unit, fixed, once, I.k - it0, route, words, reinterpret_cast<uint2 *>(words + 4), st);
+                                                     force ? 1e9f : sweep, unit, fixed, once, I.k - it0, last, route,
+                                                     words, reinterpret_cast<uint2 *>(words + 4), st);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -346,7 +346,8 @@ int64_t skip_route_words();          // the route word, the probe's counter and 
 int64_t skip_slot_rows();            // slot rows behind the k exchange rows
 bool gon_skip_possible(int dtype, int d, int64_t n, int k, int grid);   // for n points at most
 int gon_skip_segments(int dtype, int d, int64_t n, int k, int grid, int *ends, int cap);
-cudaError_t launch_gon_probe(const GonInst &I, int it0, int *route, unsigned *words, DevStatus *st, cudaStream_t s);
+cudaError_t launch_gon_probe(const GonInst &I, int it0, bool last, int *route, unsigned *words, DevStatus *st,
+                             cudaStream_t s);
 cudaError_t launch_gon_skip(GonArgs &a, int last, cudaStream_t s);
 // Resident form for one instance of n points (row-major rows in device
 // memory): the grid (0 when the instance does not fit on chip or d has no

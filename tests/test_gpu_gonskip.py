@@ -111,3 +111,36 @@ def test_skip_tiny_and_huge_coordinates(kc, monkeypatch, scale):
     b = kc.kc_gonzalez(x, 60)
     assert a.centers.cpu().tolist() == b.centers.cpu().tolist() == O.gonzalez(pts, 60, mode="f32").centers.tolist()
     assert (a.k_out, a.radius) == (b.k_out, b.radius)
+
+
+@pytest.mark.parametrize("n,d,k,clusters,gain", [(10_000_000, 8, 500, 0, 0.0), (10_000_000, 10, 1024, 1, 0.0),
+                                                 (4_000_000, 16, 512, 40, 0.5)])
+def test_probe_changes_over_only_where_it_pays(kc, monkeypatch, n, d, k, clusters, gain):
+    """Points without clusters stay on the streaming kernel (two of the slowest
+    mistakes took 2.0 and 2.1 times as long), clustered ones leave it."""
+    import time
+
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(740)
+    if clusters:
+        x = torch.randn(n, d, generator=g, device="cuda").mul_(0.5)
+        x += (20.0 * torch.rand(clusters, d, generator=g, device="cuda"))[torch.randint(0, clusters, (n,), generator=g, device="cuda")]
+    else:
+        x = torch.rand(n, d, generator=g, device="cuda")
+
+    def solve(switch):
+        if switch:
+            monkeypatch.setenv("KC_GON_SKIP", switch)
+        else:
+            monkeypatch.delenv("KC_GON_SKIP")
+        best = float("inf")
+        for _ in range(4):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            r = kc.kc_gonzalez(x, k)
+            best = min(best, time.perf_counter() - t)
+        return best, r.centers.cpu().tolist()
+
+    (t, c), (t0, c0) = solve(None), solve("0")
+    assert c == c0
+    assert t < (1.0 - gain if gain else 1.25) * t0, (t, t0)
