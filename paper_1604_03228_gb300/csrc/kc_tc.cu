@@ -1396,29 +1396,30 @@ __global__ void tc_pair_kernel(const float *__restrict__ src, int d, bool v4, co
 }
 
 // Pending rows: removed on a hit; a row whose pairs overflowed the buffer is
-// scanned against every center (one warp, lanes over centers); the rest are
-// kept.
-__global__ void tc_resolve_kernel(const float *__restrict__ src, int d, bool v4, const uint32_t *__restrict__ R,
-                                  const float *__restrict__ cen, const uint32_t *__restrict__ cidx, int64_t sn,
-                                  const uint32_t *__restrict__ pend,
-                                  const unsigned long long *npend, const uint8_t *__restrict__ flag,
-                                  const uint8_t *__restrict__ hit, const uint32_t *thr, uint32_t *Rn,
-                                  unsigned long long *rnn) {
-    const int64_t np = (int64_t)*npend;
+// scanned against every center of the tiles it met (one warp, lanes over
+// centers; by cells that is the near cells' alone); the rest are kept.
+__global__ void tc_resolve_kernel(const float *__restrict__ src, bool v4, const float *__restrict__ cen,
+                                  const uint32_t *__restrict__ cidx, TcArgs a, const uint8_t *__restrict__ hit,
+                                  const uint32_t *thr, uint32_t *Rn, unsigned long long *rnn) {
+    const int64_t np = (int64_t)*a.npend;
     const uint32_t T = *thr;
-    const int lane = threadIdx.x & 31;
+    const int d = a.d, lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t j = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); j < np; j += warps) {
-        const uint32_t pi = pend[j];
-        const int64_t gx = (int64_t)R[pi];
+        const uint32_t pi = a.pend[j];
+        const int64_t gx = (int64_t)a.R[pi];
         bool rm = hit[pi] != 0;
-        if (!rm && (flag[pi] & 2)) {
-            for (int64_t cb = 0; cb < sn && !rm; cb += 32) {
-                const int64_t ci = cb + lane;
-                const bool in = ci < sn && (!cidx || cidx[ci] != 0xFFFFFFFFu);
-                const float *c = in && cidx ? src + (int64_t)cidx[ci] * d : cen + ci * d;
-                const bool h = in && __float_as_uint(row_dist(src + gx * d, c, d, v4)) <= T;
-                rm = __any_sync(0xFFFFFFFFu, h);
+        if (!rm && (a.pflag[pi] & 2)) {
+            const PairTiles pt(a, pi / TC_CELL_UNIT);
+            for (int li = 0; li < pt.count && !rm; ++li) {
+                const int64_t c0 = (int64_t)pt[li] * TC_N;
+                for (int64_t cb = c0; cb < c0 + TC_N && cb < a.kc && !rm; cb += 32) {
+                    const int64_t ci = cb + lane;
+                    const bool in = ci < a.kc && (!cidx || cidx[ci] != 0xFFFFFFFFu);
+                    const float *c = in && cidx ? src + (int64_t)cidx[ci] * d : cen + ci * d;
+                    const bool h = in && __float_as_uint(row_dist(src + gx * d, c, d, v4)) <= T;
+                    rm = __any_sync(0xFFFFFFFFu, h);
+                }
             }
         }
         if (!rm && lane == 0) Rn[atomicAdd(rnn, 1ull)] = (uint32_t)gx;
@@ -1682,7 +1683,7 @@ cudaError_t launch_tc_prune(const float *src, int d, const uint32_t *R, int64_t 
     const bool v4 = (d & 3) == 0 && ((uintptr_t)src & 15) == 0 && (cells || ((uintptr_t)Scen & 15) == 0);
     const int g2 = sms() * 8;
     tc_pair_kernel<<<g2, 256, 0, s>>>(src, d, v4, R, Scen, cidx, P.pairs, P.npairs, P.pcap, thr, P.hit);
-    tc_resolve_kernel<<<g2, 256, 0, s>>>(src, d, v4, R, Scen, cidx, sn, P.pend, P.npend, P.flag, P.hit, thr, Rn, rnn);
+    tc_resolve_kernel<<<g2, 256, 0, s>>>(src, v4, Scen, cidx, a, P.hit, thr, Rn, rnn);
     note_launches(3);
     return cudaGetLastError();
 }

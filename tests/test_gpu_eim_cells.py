@@ -55,3 +55,47 @@ def test_cells_equal_the_whole_block(kc, monkeypatch, n, d, k):
         r = kc.kc_eim(x, k, seed=3)
         got.append((r.centers.cpu().tolist(), r.radius))
     assert got[0] == got[1]
+
+
+@pytest.mark.parametrize("d", [16, 20, 64])
+@pytest.mark.parametrize("cap", [1, 300])
+def test_cells_rescan_after_pair_overflow(kc, monkeypatch, d, cap):
+    # rows whose undecided pairs do not fit the buffer are scanned against the
+    # centers of their near cells
+    monkeypatch.setenv("KC_EIM_CELLS", "1")
+    monkeypatch.setenv("KC_TC_STREAM_CENTERS", "1")
+    monkeypatch.setenv("KC_PRUNE_PAIR_CAP", str(cap))
+    _check(kc, I.gauss_mixture(30_011, d, 850 + d, 30, 0.5, -10.0, 10.0, heavy_frac=0.5), 4, 850 + d)
+
+
+def _timed(kc, monkeypatch, x, k, cells):
+    import time
+
+    import torch
+    if cells is not None:
+        monkeypatch.setenv("KC_EIM_CELLS", cells)
+    else:
+        monkeypatch.delenv("KC_EIM_CELLS", raising=False)
+    best = float("inf")
+    for _ in range(3):
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        r = kc.kc_eim(x, k, seed=3)
+        best = min(best, time.perf_counter() - t)
+    return best, r.centers.cpu().tolist()
+
+
+def test_cells_with_many_undecided_pairs_pay(kc, monkeypatch):
+    """Half of the points in one cluster: 20M undecided pairs overflow the
+    buffer.  Scanning those rows against all of S took twice the whole block's
+    time; the near cells' part of it takes a third."""
+    import torch
+    n, d = 2_000_000, 20
+    g = torch.Generator(device="cuda").manual_seed(11)
+    c = torch.randint(0, 40, (n,), generator=g, device="cuda")
+    c[torch.rand(n, generator=g, device="cuda") < 0.5] = 0
+    x = torch.randn(n, d, generator=g, device="cuda").mul_(0.5)
+    x += (20 * torch.rand(40, d, generator=g, device="cuda"))[c]
+    (t, a), (t0, b) = _timed(kc, monkeypatch, x, 200, None), _timed(kc, monkeypatch, x, 200, "0")
+    assert a == b
+    assert t < 0.8 * t0, (t, t0)
