@@ -55,7 +55,8 @@
  *                            |S| >= 256)
  *  KC_EIM_CELLS=0|1          EIM's prune never / wherever S has 1024 points by
  *                            Voronoi cells of pivots (default: float points,
- *                            when the block |R| x |S| is large)
+ *                            when the block |R| x |S| is large and a sample
+ *                            shows that cells leave out enough of it)
  *  KC_TC_STREAM_CENTERS=1    tensor-core blocks stream the center tiles through
  *                            a two-stage ring even when all of them fit in
  *                            shared memory

@@ -1441,11 +1441,13 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
     const bool cells_ok = c.o.dtype == KC_F32 && !(cenv && atoi(cenv) == 0);
     int Pmax = !cells_ok ? 0 : (d < 16 ? CELLS_MAX : EIM_PIVOTS_TC);
     int64_t npad = n + (int64_t)Pmax * (TC_CELL_UNIT - 1);   // a list sorted by cell
-    constexpr int64_t PSAMPLE = 8192;                              // rows of S the pivots are chosen from (d >= 16)
+    constexpr int64_t PSAMPLE = 8192;   // rows of S the pivots are chosen from (d >= 16)
+    constexpr int64_t CSAMPLE = 32768;  // rows of S that show whether cells pay (4 < d < 16)
     CellBufs CB;
     CellSort CR, CS;
     int *ctiles = nullptr, *cntile = nullptr;
-    bool assigned = false;
+    unsigned long long *cpairs = nullptr;
+    bool assigned = false, no_cells = false;
     SkipBufs SB{};
     bool skip_ok = !lp && gon_skip_possible(c.o.dtype, d, n, keff_max, grid);
     LPBufs LB;
@@ -1524,6 +1526,7 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
                 o->start = cv.take<unsigned>((size_t)Pmax + 1);
                 o->cursor = cv.take<unsigned>((size_t)Pmax);
             }
+            cpairs = cv.take<unsigned long long>(1);
             if (d < 16) {
                 Lo.Ss = cv.take<float>((size_t)n * d);
             } else {
@@ -1652,9 +1655,26 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
             g_prune_pairs += (unsigned long long)rn * (unsigned long long)sn;
             const bool tcp = Ptc.tc_at && sn >= 256;
             // by cells when the whole block costs more than assigning and sorting
-            bool cells = Pmax > 0 && (assigned || sn >= 1024) && (tcp ? d >= 16 && tc_prune_pairs(d, sn) : d < 16) &&
+            bool cells = Pmax > 0 && !no_cells && (assigned || sn >= 1024) &&
+                         (tcp ? d >= 16 && tc_prune_pairs(d, sn) : d < 16) &&
                          (cenv || (double)rn * (double)sn * d >= (tcp ? 2e12 : 4e9));
-            if (cells && !assigned) {
+            // Cells that are nearly all near one another cost more than they
+            // leave out.  What share of all pairs they leave is counted once a
+            // call; whole block / by cells, ms, d < 16: share 0.42 (1M x 6
+            // uniform) 42.3 / 24.6, 0.59 (106k x 7) 2.7 / 3.1, 0.75 (1M x 5, one
+            // cluster) 20.4 / 22.3, 1 (500k x 12) 20.9 / 27.0; tensor cores 0.5
+            // (4M x 32, 70% in one cluster) 3007 / 1738, 0.64 (80%) 3349 / 3058,
+            // 0.98 (500 clusters) 106 / 115, 1 (uniform) 101 / 113.
+            auto cells_pay = [&](CellSort &R, int64_t nr, CellSort &S, int64_t ns, double share) -> kc_status {
+                KC_CUDA(launch_cells_pairs(CB, R, S, cpairs, c.s), "near pairs");
+                unsigned long long left = 0;
+                const kc_status e = read_u64(cpairs, &left);
+                cells = (double)left <= share * (double)nr * (double)ns;
+                no_cells = !cells;
+                return e;
+            };
+            const bool first = cells && !assigned;
+            if (first) {
                 if (d < 16) {
                     // pivots: the first rows of S (a random sample of the points)
                     CB.P = (int)std::min<int64_t>(CELLS_MAX, std::max<int64_t>(64, sn / 16));
@@ -1675,14 +1695,27 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
                     KC_CUDA(launch_pivot_rows((const float *)Lo.Sc, M, d, Lo.pcen, Lo.pk_out, CB.P, CB.piv, c.s),
                             "pivot rows");
                 }
-                KC_CUDA(launch_cells_assign((const float *)Lo.pk, n, d, CB, c.s), "cell assignment");
-                assigned = true;
+                // Below d = 16 the assignment to up to 1024 pivots is a few
+                // percent of the block, so part of S stands for both sides; its
+                // cells reach less far, and its share is a sixth to a third
+                // lower.  Up to d = 4 no point set gave more than 0.3.
+                if (!cenv && d > 4 && d < 16) {
+                    const int64_t M = std::min<int64_t>(sn, CSAMPLE);
+                    KC_CUDA(launch_cells_sample((const float *)Lo.Sc, M, d, CB, CR, c.s), "sample cells");
+                    KC_CUDA(launch_cells_near(d, CB, CR, CR, Lo.thr, c.s), "sample near cells");
+                    if ((r = cells_pay(CR, M, CR, M, 0.4)) != KC_OK) return r;
+                }
+                if (cells) {
+                    KC_CUDA(launch_cells_assign((const float *)Lo.pk, n, d, CB, c.s), "cell assignment");
+                    assigned = true;
+                }
             }
             if (cells) {
                 const int ru = tcp ? TC_CELL_UNIT : cells_prune_unit(), su = tcp ? TC_CELL_UNIT : 1;
                 KC_CUDA(launch_cells_sort(Rc, rn, ru, CB, CR, c.s), "sort R");
                 KC_CUDA(launch_cells_sort(Lo.S, sn, su, CB, CS, c.s), "sort S");
                 KC_CUDA(launch_cells_near(d, CB, CR, CS, Lo.thr, c.s), "near cells");
+                if (first && tcp && !cenv && (r = cells_pay(CR, rn, CS, sn, 0.7)) != KC_OK) return r;
             }
             if (cells && tcp) {
                 const int64_t rp = rn + (int64_t)CB.P * (TC_CELL_UNIT - 1), sp = sn + (int64_t)CB.P * (TC_CELL_UNIT - 1);

@@ -38,6 +38,37 @@ __global__ void __launch_bounds__(NEAREST_NT, DC == 2 ? 3 : 2) cells_assign_kern
     nearest_centers<DC>(pk, n, d, P, as_c, [=](int c, int j) { return __ldg(piv + (int64_t)c * dd + j); }, dist, cell);
 }
 
+// The same for a few thousand rows (d < 16): a CTA takes 32 of them, a lane one,
+// and its warps share the pivots, so that it takes the time of P / 8 pivots
+// (the kernel above walks all P in each warp: 8853 x 12, P = 553, 70 us of 1.5
+// ms of an EIM call).
+constexpr int SAMPLE_NT = 256, SAMPLE_D = 16;
+__global__ void __launch_bounds__(SAMPLE_NT) cells_sample_kernel(const float *__restrict__ rows, int64_t n, int d,
+                                                                 const float *__restrict__ piv, int P,
+                                                                 uint16_t *__restrict__ cell, uint32_t *__restrict__ dist) {
+    __shared__ unsigned long long best[SAMPLE_NT / 32][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    float x[SAMPLE_D];
+#pragma unroll
+    for (int j = 0; j < SAMPLE_D; ++j) x[j] = i < n && j < d ? rows[i * d + j] : 0.f;
+    unsigned long long b = ~0ull;   // (distance bits, pivot), smallest
+    for (int p = warp; p < P; p += SAMPLE_NT / 32) {
+        float acc = 0.f;
+#pragma unroll
+        for (int j = 0; j < SAMPLE_D; ++j) acc = sq_step(acc, x[j], j < d ? __ldg(piv + (int64_t)p * d + j) : 0.f);
+        const unsigned long long k = ((unsigned long long)__float_as_uint(acc) << 32) | (unsigned)p;
+        b = k < b ? k : b;
+    }
+    best[warp][lane] = b;
+    __syncthreads();
+    if (warp == 0 && i < n) {
+        for (int w = 1; w < SAMPLE_NT / 32; ++w) b = best[w][lane] < b ? best[w][lane] : b;
+        cell[i] = (uint16_t)b;
+        dist[i] = (uint32_t)(b >> 32);
+    }
+}
+
 // ------------------------------------------------------------------- sort
 // Counting sort of a list of points by cell.  Counts and the largest distance
 // of each cell, then (one CTA) the cells' starts, padded to `unit`, then the
@@ -56,7 +87,7 @@ __global__ void __launch_bounds__(SORT_NT) cells_count_kernel(const uint32_t *__
         const int64_t c1 = c0 + SORT_CHUNK < cnt ? c0 + SORT_CHUNK : cnt;
 #pragma unroll 4
         for (int64_t i = c0 + threadIdx.x; i < c1; i += SORT_NT) {
-            const uint32_t x = list[i];
+            const uint32_t x = list ? list[i] : (uint32_t)i;
             const int p = cell[x];
             const uint32_t v = dist[x];
             atomicAdd(&sc[p], 1u);
@@ -159,6 +190,21 @@ __global__ void __launch_bounds__(NEAR_NT) cells_near_kernel(const float *__rest
     }
     __syncthreads();
     if (threadIdx.x == 0) nnear[p] = cnt;
+}
+
+// Pairs that the near lists leave: the sum over the cells p of R's points of p
+// times S's points of the cells near p.  One CTA per p.
+constexpr int PAIRS_NT = 128;
+__global__ void __launch_bounds__(PAIRS_NT) cells_pairs_kernel(const uint16_t *__restrict__ near,
+                                                               const int *__restrict__ nnear, int P,
+                                                               const unsigned *__restrict__ rcount,
+                                                               const unsigned *__restrict__ scount,
+                                                               unsigned long long *pairs) {
+    const int p = blockIdx.x, m = nnear[p];
+    unsigned sum = 0;
+    for (int e = threadIdx.x; e < m; e += PAIRS_NT) sum += scount[near[(int64_t)p * P + e]];
+    sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(pairs, (unsigned long long)sum * rcount[p]);
 }
 
 // The near lists as center tiles of `tile` positions of sorted S (whose cells
@@ -319,6 +365,24 @@ cudaError_t launch_cells_near(int d, const CellBufs &C, const CellSort &R, const
     cells_near_kernel<<<C.P, NEAR_NT, (size_t)d * sizeof(float), s>>>(
         C.piv, C.P, d, R.count, R.count + C.P, S.count, S.count + C.P, thr, (float)(2.0 * g) + 0x1p-22f,
         (float)(1.0 - 2.0 * g - 0x1p-18), C.near, C.nnear);
+    note_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cells_sample(const float *rows, int64_t cnt, int d, const CellBufs &C, CellSort &O, cudaStream_t s) {
+    cells_sample_kernel<<<(int)((cnt + 31) / 32), SAMPLE_NT, 0, s>>>(rows, cnt, d, C.piv, C.P, C.cell, C.dist);
+    cudaMemsetAsync(O.count, 0, 2 * (size_t)C.P * sizeof(unsigned), s);
+    const int g = (int)std::min<int64_t>((cnt + SORT_CHUNK - 1) / SORT_CHUNK, (int64_t)sm_count() * 4);
+    cells_count_kernel<<<g, SORT_NT, 2 * (size_t)C.P * sizeof(unsigned), s>>>(nullptr, cnt, C.P, C.cell, C.dist, O.count,
+                                                                              O.count + C.P);
+    note_launches(2);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cells_pairs(const CellBufs &C, const CellSort &R, const CellSort &S, unsigned long long *pairs,
+                               cudaStream_t s) {
+    cudaMemsetAsync(pairs, 0, sizeof(unsigned long long), s);
+    cells_pairs_kernel<<<C.P, PAIRS_NT, 0, s>>>(C.near, C.nnear, C.P, R.count, S.count, pairs);
     note_launches(1);
     return cudaGetLastError();
 }

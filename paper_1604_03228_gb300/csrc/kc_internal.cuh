@@ -548,6 +548,11 @@ cudaError_t launch_cells_sort(const uint32_t *list, int64_t cnt, int unit, const
                               cudaStream_t s);
 cudaError_t launch_cells_near(int d, const CellBufs &C, const CellSort &R, const CellSort &S, const uint32_t *thr,
                               cudaStream_t s);
+// Cells, counts and radii of the rows [0, cnt) (d < 16; O's list is not made);
+// and the pairs of two lists that the near cells leave.
+cudaError_t launch_cells_sample(const float *rows, int64_t cnt, int d, const CellBufs &C, CellSort &O, cudaStream_t s);
+cudaError_t launch_cells_pairs(const CellBufs &C, const CellSort &R, const CellSort &S, unsigned long long *pairs,
+                               cudaStream_t s);
 cudaError_t launch_cells_tiles(const CellBufs &C, const CellSort &S, int tile, int cap, int *tiles, int *ntile,
                                cudaStream_t s);
 int cells_prune_unit();

@@ -99,3 +99,14 @@ def test_cells_with_many_undecided_pairs_pay(kc, monkeypatch):
     (t, a), (t0, b) = _timed(kc, monkeypatch, x, 200, None), _timed(kc, monkeypatch, x, 200, "0")
     assert a == b
     assert t < 0.8 * t0, (t, t0)
+
+
+@pytest.mark.parametrize("n,d,k", [(500_000, 12, 20), (2_000_000, 8, 25)])
+def test_cells_only_where_a_sample_shows_that_they_pay(kc, monkeypatch, n, d, k):
+    """Uniform points, whose cells are all near one another, take the whole
+    block (by cells 1.1 to 1.3 times its time)."""
+    import torch
+    x = torch.rand(n, d, generator=torch.Generator(device="cuda").manual_seed(860), device="cuda")
+    (t, a), (t0, b) = _timed(kc, monkeypatch, x, k, None), _timed(kc, monkeypatch, x, k, "0")
+    assert a == b
+    assert t < 1.07 * t0, (t, t0)
