@@ -57,9 +57,9 @@ constexpr int SKIP_TILE = UNIT * 33;    // words of a warp's transpose tile
 //  - elsewhere (no clusters, or each has its center) it stays about what it is.
 // *route is set to it0 when the steps left would take a tenth less time that
 // way and the next ones no longer than a sweep (at the last probe they may, if
-// all together take a seventh less).  Taking the share to fall on any points (its square) cost 10M x 8
-// uniform, k = 500, 61 ms against 30, and one cluster of 10M x 10, k = 1024, 152
-// against 72; there is no way back.
+// all together take a seventh less); there is no way back.  Taking the share to
+// fall on any points (its square) cost 10M x 8 uniform, k = 500, 61 ms against
+// 30, and one cluster of 10M x 10, k = 1024, 153 against 72.
 constexpr int PROBE_NT = 256, PROBE_CTAS = 128, PROBE_S = PROBE_CTAS * PROBE_NT / 32;
 constexpr int PROBE_MAX = 256;         // most centers at a probe
 
