@@ -67,8 +67,9 @@ __device__ __forceinline__ void pc_publish(const long long *c) {
 
 namespace {
 
-// One step's sweep of this CTA's share (rank r of G) of [lo, lo + n).
-template <typename T, int DC, int NT, int UNR>
+// One step's sweep of this CTA's share (rank r of G) of [lo, lo + n); UNR and
+// BATCH as in dist4.
+template <typename T, int DC, int NT, int UNR, int BATCH>
 __device__ __forceinline__ uint64_t sweep(const T *__restrict__ pk, uint32_t *__restrict__ mind,
                                           int64_t lo, int64_t n, int d, const T *cs, bool first_step,
                                           int r, int G, int *ctr, int *gtail) {
@@ -99,7 +100,7 @@ __device__ __forceinline__ uint64_t sweep(const T *__restrict__ pk, uint32_t *__
             }
         }
         typename AccOf<T>::type acc[4];
-        dist4<T, DC, UNR>(pk + b * d * BLK, d, cs, lane, acc);
+        dist4<T, DC, UNR, BATCH>(pk + b * d * BLK, d, cs, lane, acc);
         uint32_t m[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) m[q] = min(o[q], acc_bits(acc[q]));
@@ -163,8 +164,9 @@ struct Shared {
 // CTA on 3608 x 16 takes 2.35 us a step without its code, 2.73 with it).  UNR:
 // coordinates in flight in the generic loop, 8 in queue launches of one d (MRG
 // on 2M x 64 with 4 / 8: 20.0 / 18.4 ms, int32 29.7 / 28.7; batches of int32
-// 1791 x 64 2.64 / 2.31), 4 elsewhere (streaming float 4M x 40 110 / 119 us a
-// step, batches through the kernel of several d at d = 37 20.9 / 22.9 ms).
+// 1791 x 64 2.64 / 2.31), 4 elsewhere (streaming float 800k x 37 23.6 / 26.0 us a
+// step, 800k x 256 129 / 127; batches through the kernel of several d at d = 37
+// 20.9 / 22.9 ms).
 template <typename T, int DC, int NT, bool DYN = false, bool LEAD = false, int UNR = 4>
 __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
                           long long timeout, int withhold = 0, bool bad_index = false) {
@@ -190,15 +192,7 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
     __syncthreads();
     const bool claim = DYN && NT == GROUP_NT && (I.lo + I.n - 1) / BLK - I.lo / BLK + 1 >= 4 * (int64_t)G * W;
     const bool tail = DYN && G > 1 && I.tail != nullptr;
-    // Through the leader while a step's sweep is short, fewer than four blocks
-    // a warp: behind longer ones the CTAs arrive apart, do not slow each other's
-    // polling, and the leader's second hop is what shows (int32 6.4M x 55,
-    // 230 us a step: 1% slower; float 8M x 64: 0.7%).  Not between queue CTAs,
-    // which share their SM with other groups: nothing gained, and the sweep's
-    // code grew (MRG round 1 on 10M x 16 20.2 -> 20.7 ms).
-    const bool lead = LEAD && G > LEADER_MIN && I.bc != nullptr &&
-                      (I.lo + I.n - 1) / BLK - I.lo / BLK + 1 < 4 * (int64_t)G * W;
-
+    constexpr bool lead = LEAD;   // gon_lead
     int it;
     uint64_t K = 0;
     for (it = I.it0; it < I.it1; ++it) {
@@ -206,7 +200,7 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
         // several (measured: GON on 8M x 64, k = 1024, 313 -> 308 ms); the
         // fixed assignment in the 256-thread queue CTAs (MRG round 1 on
         // 10M x 16 was 5% slower with claims) and for small instances
-        uint64_t best = sweep<T, DC, NT, UNR>(pk, I.mind, I.lo, I.n, d, cs, it == 0, r, G,
+        uint64_t best = sweep<T, DC, NT, UNR, NT == GROUP_NT ? (DYN ? 2 : 1) : 0>(pk, I.mind, I.lo, I.n, d, cs, it == 0, r, G,
                                          claim ? &sh.ctr[it & 1] : nullptr, tail ? I.tail + it : nullptr);
         best = warp_max_u64(best);
         if (lane == 0) sh.red[warp] = best;
@@ -1336,7 +1330,6 @@ template <bool DYN, bool LEAD> void *pick_group_f32(int dc) {
         case 10: return group_fn<float, 10, DYN, LEAD>();
         case 16: return group_fn<float, 16, DYN, LEAD>();
         case 32: return group_fn<float, 32, DYN, LEAD>();
-        case 64: return group_fn<float, 64, DYN, LEAD>();
         default: return group_fn<float, 0, DYN, LEAD>();
     }
 }
@@ -1473,6 +1466,20 @@ int gon_resident_plan(int dtype, int d, int64_t n, int *cap, int *slot_words) {
     return G;
 }
 
+// Does a single instance's exchange go through the leader?  Where a step's
+// sweep is short: behind longer ones the CTAs arrive apart, do not slow each
+// other's polling, and the leader's second hop and the code it adds to the sweep
+// are what shows (not between queue CTAs either, which share their SM with other
+// groups: MRG round 1 on 10M x 16 20.2 -> 20.7 ms).  All polling / leader, us a
+// step, float: 200k x 2 (49 CTAs) 2.65 / 3.2, x 10 3.4 / 4.0, x 16 5.4 / 4.6; 600k x
+// 2 4.7 / 3.4, 1M x 10 7.2 / 5.7, 600k x 37 (89 MB) 11.3 / 8.8, 2.4M x 16 30.0 /
+// 28.4; beyond L2 1.5M x 64 68.6 / 72.4, 800k x 128 83 / 87; 200k x 100 14.6 / 15.3.
+// int32: 1.5M x 64 76 / 66, 1M x 100 74 / 66.
+static bool gon_lead(int dtype, int d, int64_t n, int G) {
+    if (G <= (d <= 10 ? 64 : LEADER_MIN) || nblocks(n) >= 4 * (int64_t)G * (GROUP_NT / 32)) return false;
+    return dtype == KC_I32 || d <= 16 || (d <= 64 && 4.0 * (double)n * d <= 100e6);
+}
+
 cudaError_t launch_gon(GonArgs &a, cudaStream_t s) {
     if (a.res_cap > 0) {
         // resident single instance: one CTA per SM, all co-resident
@@ -1495,7 +1502,8 @@ cudaError_t launch_gon(GonArgs &a, cudaStream_t s) {
         return cudaLaunchKernelExC(&cfg, fn, args);
     }
     const size_t smem = smem_for(a.dtype, a.lp_kind, a.dmax, a.queue != 0);
-    void *fn = pick_fn(a.dtype, a.lp_kind, a.dc, a.queue != 0, a.dyn != 0, a.grid > LEADER_MIN);
+    const bool lead = !a.insts && !a.lp_kind && a.single.bc && gon_lead(a.dtype, a.dc, a.single.n, a.grid);
+    void *fn = pick_fn(a.dtype, a.lp_kind, a.dc, a.queue != 0, a.dyn != 0, lead);
     if (const cudaError_t e = opt_in_smem(fn, smem)) return e;
     note_launches(1);
     // Groups that wait on one another need a cooperative launch (all CTAs

@@ -27,8 +27,17 @@ __device__ __forceinline__ void st_relaxed_u64(uint64_t *p, uint64_t v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// UNR: coordinates in flight in the generic loop (DC = 0).
-template <typename T, int DC, int UNR = 4>
+// UNR: coordinates in flight in the generic loop (DC = 0).  BATCH: their loads
+// written out ahead of the terms, with one more batch for the remainder (1) or a
+// load at a time (2), or (0) left to the compiler.  In the 1024-thread kernels it
+// mixed loads and terms of a plain unrolled loop differently from build to build
+// (us a step: 800k x 256 on 98 CTAs 147 or 160, written out 129; 1.5M x 24 30.5
+// or 32, 27.8; 4M x 40 111, 98), and the loop written out beats the full unrolling
+// of d = 64 too (1.5M x 64 70.2 / 65.2, 8M x 64 309 / 297).  The remainder as a
+// batch made the claimed-block instantiation a third slower (5M x 37 128 -> 173,
+// one by one 116).  In the 256-thread kernels the plain loop is the better one
+// (MRG on 2M x 64 18.4 ms, written out 22.2).
+template <typename T, int DC, int UNR, int BATCH>
 __device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T *cs, int lane,
                                       typename AccOf<T>::type acc[4]) {
     using V4 = typename Vec4<T>::type;
@@ -44,6 +53,47 @@ __device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T 
             a1 = sq_step(a1, v.y, c);
             a2 = sq_step(a2, v.z, c);
             a3 = sq_step(a3, v.w, c);
+        }
+    } else if constexpr (BATCH != 0) {
+        int j = 0;
+#pragma unroll 1
+        for (; j + UNR <= d; j += UNR) {
+            V4 v[UNR];
+#pragma unroll
+            for (int t = 0; t < UNR; ++t) v[t] = __ldg(src + (j + t) * (BLK / 4));
+#pragma unroll
+            for (int t = 0; t < UNR; ++t) {
+                const T c = cs[j + t];
+                a0 = sq_step(a0, v[t].x, c);
+                a1 = sq_step(a1, v[t].y, c);
+                a2 = sq_step(a2, v[t].z, c);
+                a3 = sq_step(a3, v[t].w, c);
+            }
+        }
+        if constexpr (BATCH == 2) {
+#pragma unroll 1
+            for (; j < d; ++j) {
+                const V4 v = __ldg(src + j * (BLK / 4));
+                const T c = cs[j];
+                a0 = sq_step(a0, v.x, c);
+                a1 = sq_step(a1, v.y, c);
+                a2 = sq_step(a2, v.z, c);
+                a3 = sq_step(a3, v.w, c);
+            }
+        } else if (j < d) {
+            V4 v[UNR - 1];
+#pragma unroll
+            for (int t = 0; t < UNR - 1; ++t)
+                if (j + t < d) v[t] = __ldg(src + (j + t) * (BLK / 4));
+#pragma unroll
+            for (int t = 0; t < UNR - 1; ++t)
+                if (j + t < d) {
+                    const T c = cs[j + t];
+                    a0 = sq_step(a0, v[t].x, c);
+                    a1 = sq_step(a1, v[t].y, c);
+                    a2 = sq_step(a2, v[t].z, c);
+                    a3 = sq_step(a3, v[t].w, c);
+                }
         }
     } else {
 #pragma unroll UNR

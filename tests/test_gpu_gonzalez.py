@@ -456,3 +456,26 @@ def test_refused_launch_leaves_no_error_behind(kc, noalloc):
         solve(big, 8)
     assert e.value.status == kc.KC_ERR_CUDA
     assert solve(x, 9).centers.cpu().tolist() == ref
+
+
+@pytest.mark.parametrize("d", [4, 5, 6, 7, 64, 65])
+@pytest.mark.parametrize("n", [3_000, 262_144, 262_273, 2_600_001])
+def test_streaming_loop_remainders_and_exchange_forms(kc, monkeypatch, n, d):
+    """The generic loop's batches of four coordinates and their remainders; 24, 64
+    and 65 CTAs (all poll / leader) and claimed blocks with a shared tail."""
+    if n > 1_000_000 and d > 7:
+        n = 2_500_001
+    monkeypatch.setenv("KC_GON_RESIDENT", "0")
+    pts = I.unif_points(n, d, 33)
+    ref = O.gonzalez(pts, 6, mode="f32")
+    r = kc.kc_gonzalez(_dev(pts), 6)
+    assert r.centers.cpu().tolist() == ref.centers.tolist() and r.radius == O.radius(pts, ref.centers, mode="f64")[0]
+
+
+@pytest.mark.parametrize("n,d", [(163_841, 11), (390_000, 64), (391_000, 64), (170_000, 65), (300_000, 16)])
+@pytest.mark.parametrize("integer", [False, True])
+def test_leader_rule_edges(kc, monkeypatch, n, d, integer):
+    monkeypatch.setenv("KC_GON_RESIDENT", "0")
+    pts = I.int_points(n, d, 34, -100, 100) if integer else I.gauss_mixture(n, d, 34, 9, 0.5, -10, 10)
+    ref = O.gonzalez(pts, 12, mode="i64" if integer else "f32")
+    assert kc.kc_gonzalez(_dev(pts), 12).centers.cpu().tolist() == ref.centers.tolist()
