@@ -1101,7 +1101,7 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
     struct L {
         int32_t *range2;
         unsigned long long *key32, *max64, *arg64;
-        uint64_t *slots1, *slots2, *fk2, *bc1, *bc2;
+        uint64_t *slots1, *slots2, *fk2;
         int64_t *nU;
         int *counter;
         void *staging, *pk, *pkU, *cen;
@@ -1128,8 +1128,6 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
         Lo.counter = cv.take<int>(1);
         Lo.slots1 = cv.take<uint64_t>((size_t)std::max<int64_t>(1, slot_off[m]));
         Lo.slots2 = cv.take<uint64_t>((size_t)slot_words(k, G2, false));
-        Lo.bc1 = cv.take<uint64_t>((size_t)bc_words(d) * m);
-        Lo.bc2 = cv.take<uint64_t>((size_t)bc_words(d));
         Lo.zero_bytes = cv.off;
         Lo.staging = (dev_pts || pin_pts) ? nullptr : cv.take<char>((size_t)n * d * esz);
         Lo.pk = cv.take<char>((size_t)nb * BLK * d * esz);
@@ -1179,7 +1177,6 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
             I.pk = Lo.pk;
             I.mind = Lo.mind;
             I.slots = Lo.slots1 + slot_off[i];
-            I.bc = Lo.bc1 + bc_words(d) * i;
             I.centers = Lo.c1 + (int64_t)i * k;
             I.k_out = Lo.k1 + i;
             I.final_key = Lo.fk1 + i;
@@ -1204,7 +1201,6 @@ kc_status mrg_run(const void *pts, int64_t n, int32_t d, int32_t k, int32_t m, c
     proto.pk = Lo.pkU;
     proto.mind = Lo.mindU;
     proto.slots = Lo.slots2;
-    proto.bc = Lo.bc2;
     proto.centers = Lo.cen_dev;
     proto.k_out = Lo.kout_dev;
     proto.final_key = Lo.fk2;

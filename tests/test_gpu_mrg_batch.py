@@ -281,3 +281,18 @@ def test_mrg_rounds_bf16_first_round(kc):
     ref = O.mrg_rounds(pts, 12, off, 100, mode="f32")
     got, rounds = kc.kc_mrg_rounds(_dev(pts), 12, 50, 100, _dev(off), sweep="bf16")
     assert rounds == ref.rounds and got.centers.cpu().tolist() == ref.centers.tolist()
+
+
+def test_mrg_scratch_of_many_parts(kc):
+    # 200,000 parts of two points: scratch is the packed points, the union's copy
+    # and a descriptor per part, no words of an exchange that no part has
+    import torch
+    n, d, m = 400_000, 64, 200_000
+    x = torch.rand(n, d, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    r = kc.kc_mrg(x, 1, m, stream=stream.cuda_stream)
+    used = before - torch.cuda.mem_get_info()[0]
+    assert r.k_out == 1
+    assert used < 9 / 8 * (n * d * 4 * 1.5 + 512 * m) + 32e6, used
