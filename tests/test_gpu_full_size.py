@@ -152,6 +152,14 @@ def test_eim_8m_tensor_core_prune_equals_cuda_cores(kc, gau8m, monkeypatch):
     assert radius_checks(pts, ca, rr.radius, rr.argmax, sample_rows(len(pts), 4000, 15)) == []
 
 
+def test_eim_8m_skip_kernel_equals_streaming_on_the_sample(kc, gau8m, monkeypatch):
+    x = _dev(gau8m)
+    a = kc.kc_eim(x, 1024, eps=0.1, phi=6.0, seed=40)
+    monkeypatch.setenv("KC_GON_SKIP", "0")
+    b = kc.kc_eim(x, 1024, eps=0.1, phi=6.0, seed=40)
+    assert _centers(a).tolist() == _centers(b).tolist() and a.radius == b.radius
+
+
 def test_batch_4096_plan(kc):
     insts = [I.batch_instance(i) for i in range(4096)]
     xs = [_dev(z.points) for z in insts]

@@ -113,6 +113,38 @@ def test_skip_tiny_and_huge_coordinates(kc, monkeypatch, scale):
     assert (a.k_out, a.radius) == (b.k_out, b.radius)
 
 
+@pytest.mark.parametrize("kind", ["gau", "dup", "unaligned", "host"])
+def test_skip_on_eims_sample_equals_oracle(kc, kind):
+    # the rows of the sample are found through its index
+    import torch
+    n, d, k = 40_009, 9, 24
+    pts = I.gauss_mixture(n, d, 750, 15, 0.5, -10.0, 10.0)
+    if kind == "dup":
+        pts = np.ascontiguousarray(pts[np.arange(n) % 20_000])
+    x = pts
+    if kind == "unaligned":
+        x = torch.empty(pts.size + 1, dtype=torch.float32, device="cuda")[1:].view(pts.shape)
+        x.copy_(torch.from_numpy(pts))
+    elif kind != "host":
+        x = _dev(pts)
+    r = kc.kc_eim(x, k, eps=0.1, phi=6.0, seed=7)
+    ref = O.eim(pts, k, 0.1, 6.0, 7, mode="f32")
+    assert np.asarray(r.centers if kind == "host" else r.centers.cpu()).tolist() == ref.centers.tolist()
+    assert r.radius == O.radius(pts, ref.centers, mode="f64")[0]
+
+
+@pytest.mark.parametrize("n,d,k", [(800_000, 12, 200), (60_000, 1000, 30), (1_500_001, 33, 300)])
+def test_skip_on_eims_sample_equals_streaming(kc, monkeypatch, n, d, k):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(751)
+    x = torch.randn(n, d, generator=g, device="cuda").mul_(0.5)
+    x += (20.0 * torch.rand(40, d, generator=g, device="cuda"))[torch.randint(0, 40, (n,), generator=g, device="cuda")]
+    a = kc.kc_eim(x, k, seed=3)
+    monkeypatch.setenv("KC_GON_SKIP", "0")
+    b = kc.kc_eim(x, k, seed=3)
+    assert a.centers.cpu().tolist() == b.centers.cpu().tolist() and (a.k_out, a.radius) == (b.k_out, b.radius)
+
+
 @pytest.mark.parametrize("n,d,k,clusters,gain", [(10_000_000, 8, 500, 0, 0.0), (10_000_000, 10, 1024, 1, 0.0),
                                                  (4_000_000, 16, 512, 40, 0.5)])
 def test_probe_changes_over_only_where_it_pays(kc, monkeypatch, n, d, k, clusters, gain):
