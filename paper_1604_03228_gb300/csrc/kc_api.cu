@@ -262,6 +262,12 @@ const char *where_name(int w) {
         case KC_AT_EIM_INDEX: return "EIM point index (checked build)";
         case KC_AT_RADIUS_LIST: return "radius recheck list (checked build)";
         case KC_AT_SLOT: return "exchange slot (checked build)";
+        case KC_AT_SKIP_BIN: return "regrouping bin or position (checked build)";
+        case KC_AT_SKIP_UNIT: return "skip kernel unit (checked build)";
+        case KC_AT_SKIP_ROW: return "regrouped point (checked build)";
+        case KC_AT_CELL: return "EIM cell (checked build)";
+        case KC_AT_CELL_POS: return "EIM sorted position (checked build)";
+        case KC_AT_TILE: return "near center tile (checked build)";
         default: return "device";
     }
 }
@@ -1697,8 +1703,8 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
                 // lower.  Up to d = 4 no point set gave more than 0.3.
                 if (!cenv && d > 4 && d < 16) {
                     const int64_t M = std::min<int64_t>(sn, CSAMPLE);
-                    KC_CUDA(launch_cells_sample((const float *)Lo.Sc, M, d, CB, CR, c.s), "sample cells");
-                    KC_CUDA(launch_cells_near(d, CB, CR, CR, Lo.thr, c.s), "sample near cells");
+                    KC_CUDA(launch_cells_sample((const float *)Lo.Sc, M, d, CB, CR, st, c.s), "sample cells");
+                    KC_CUDA(launch_cells_near(d, CB, CR, CR, Lo.thr, st, c.s), "sample near cells");
                     if ((r = cells_pay(CR, M, CR, M, 0.4)) != KC_OK) return r;
                 }
                 if (cells) {
@@ -1708,22 +1714,23 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
             }
             if (cells) {
                 const int ru = tcp ? TC_CELL_UNIT : cells_prune_unit(), su = tcp ? TC_CELL_UNIT : 1;
-                KC_CUDA(launch_cells_sort(Rc, rn, ru, CB, CR, c.s), "sort R");
-                KC_CUDA(launch_cells_sort(Lo.S, sn, su, CB, CS, c.s), "sort S");
-                KC_CUDA(launch_cells_near(d, CB, CR, CS, Lo.thr, c.s), "near cells");
+                KC_CUDA(launch_cells_sort(Rc, rn, ru, CB, CR, st, c.s), "sort R");
+                KC_CUDA(launch_cells_sort(Lo.S, sn, su, CB, CS, st, c.s), "sort S");
+                KC_CUDA(launch_cells_near(d, CB, CR, CS, Lo.thr, st, c.s), "near cells");
                 if (first && tcp && !cenv && (r = cells_pay(CR, rn, CS, sn, 0.7)) != KC_OK) return r;
             }
             if (cells && tcp) {
                 const int64_t rp = rn + (int64_t)CB.P * (TC_CELL_UNIT - 1), sp = sn + (int64_t)CB.P * (TC_CELL_UNIT - 1);
                 const int cap = tc_center_tiles(sp);
-                KC_CUDA(launch_cells_tiles(CB, CS, TC_CELL_UNIT, cap, ctiles, cntile, c.s), "center tiles");
+                KC_CUDA(launch_cells_tiles(CB, CS, TC_CELL_UNIT, cap, ctiles, cntile, st, c.s), "center tiles");
                 const TcCells tcc{&CR, &CS, CB.P, ctiles, cntile, cap};
                 KC_CUDA(launch_tc_prune((const float *)src, d, nullptr, rp, Lo.mask, nullptr, sp, tc_bufs(Ptc), Lo.pb,
                                         Lo.thr, Rx, Lo.rnn, st, c.s, &tcc),
                         "prune");
             } else if (cells) {
                 KC_CUDA(launch_eim_gather_rows(src, c.o.dtype, d, CS.idx, 0, sn, Lo.Ss, c.s), "sorted S");
-                KC_CUDA(launch_cells_prune((const float *)src, d, rn, Lo.mask, Lo.Ss, CB, CR, CS, Lo.thr, Rx, Lo.rnn, c.s),
+                KC_CUDA(launch_cells_prune((const float *)src, d, rn, Lo.mask, Lo.Ss, CB, CR, CS, Lo.thr, Rx, Lo.rnn, n, sn, st,
+                                           c.s),
                         "prune");
             } else if (tcp) {
                 // tensor-core R x S block with exact rechecks of undecided pairs

@@ -78,7 +78,7 @@ constexpr int SORT_NT = 512, SORT_CHUNK = 8192;
 __global__ void __launch_bounds__(SORT_NT) cells_count_kernel(const uint32_t *__restrict__ list, int64_t cnt, int P,
                                                               const uint16_t *__restrict__ cell,
                                                               const uint32_t *__restrict__ dist, unsigned *count,
-                                                              unsigned *rad) {
+                                                              unsigned *rad, DevStatus *st) {
     extern __shared__ unsigned sc[];   // [P] counts, [P] radii
     unsigned *sr = sc + P;
     for (int i = threadIdx.x; i < 2 * P; i += SORT_NT) sc[i] = 0;
@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(SORT_NT) cells_count_kernel(const uint32_t *__
         for (int64_t i = c0 + threadIdx.x; i < c1; i += SORT_NT) {
             const uint32_t x = list ? list[i] : (uint32_t)i;
             const int p = cell[x];
+            if (!KC_IN_RANGE(st, p, P, KC_AT_CELL)) continue;
             const uint32_t v = dist[x];
             atomicAdd(&sc[p], 1u);
             if (v > sr[p]) atomicMax(&sr[p], v);
@@ -132,7 +133,8 @@ __global__ void __launch_bounds__(1024) cells_starts_kernel(const unsigned *__re
 
 __global__ void __launch_bounds__(SORT_NT) cells_scatter_kernel(const uint32_t *__restrict__ list, int64_t cnt, int P,
                                                                 const uint16_t *__restrict__ cell, unsigned *cursor,
-                                                                uint32_t *__restrict__ out) {
+                                                                uint32_t *__restrict__ out, int64_t extent,
+                                                                DevStatus *st) {
     extern __shared__ unsigned sc[];   // [P]
     for (int64_t c0 = (int64_t)blockIdx.x * SORT_CHUNK; c0 < cnt; c0 += (int64_t)gridDim.x * SORT_CHUNK) {
         const int64_t c1 = c0 + SORT_CHUNK < cnt ? c0 + SORT_CHUNK : cnt;
@@ -147,7 +149,8 @@ __global__ void __launch_bounds__(SORT_NT) cells_scatter_kernel(const uint32_t *
 #pragma unroll 4
         for (int64_t i = c0 + threadIdx.x; i < c1; i += SORT_NT) {
             const uint32_t x = list[i];
-            out[atomicAdd(&sc[cell[x]], 1u)] = x;
+            const unsigned p = atomicAdd(&sc[cell[x]], 1u);
+            if (KC_IN_RANGE(st, p, extent, KC_AT_CELL_POS)) out[p] = x;
         }
         __syncthreads();
     }
@@ -164,7 +167,8 @@ __global__ void __launch_bounds__(NEAR_NT) cells_near_kernel(const float *__rest
                                                              const unsigned *__restrict__ scount,
                                                              const unsigned *__restrict__ srad,
                                                              const uint32_t *thr_p, float g2, float f,
-                                                             uint16_t *__restrict__ near, int *__restrict__ nnear) {
+                                                             uint16_t *__restrict__ near, int *__restrict__ nnear,
+                                                             DevStatus *st) {
     extern __shared__ float np[];   // [d] pivot p
     __shared__ int cnt;
     const int p = blockIdx.x;
@@ -186,7 +190,8 @@ __global__ void __launch_bounds__(NEAR_NT) cells_near_kernel(const float *__rest
         for (int j = 0; j < d; ++j) t = sq_step(t, np[j], __ldg(piv + (int64_t)q * d + j));
         const float h = t >= 0x1p-100f && t <= 3.0e38f ? __fmul_rd(__fsqrt_rd(t), f) : 0.f;
         if (h > __fadd_ru(need, up(srad[q]))) continue;
-        near[(int64_t)p * P + atomicAdd(&cnt, 1)] = (uint16_t)q;
+        const int at = atomicAdd(&cnt, 1);
+        if (KC_IN_RANGE(st, at, P, KC_AT_CELL)) near[(int64_t)p * P + at] = (uint16_t)q;
     }
     __syncthreads();
     if (threadIdx.x == 0) nnear[p] = cnt;
@@ -211,7 +216,7 @@ __global__ void __launch_bounds__(PAIRS_NT) cells_pairs_kernel(const uint16_t *_
 // start at multiples of it): tiles[p][0 .. ntile[p]).
 __global__ void __launch_bounds__(256) cells_tiles_kernel(const uint16_t *__restrict__ near, const int *__restrict__ nnear,
                                                           int P, const unsigned *__restrict__ sstart, int tile, int cap,
-                                                          int *__restrict__ tiles, int *__restrict__ ntile) {
+                                                          int *__restrict__ tiles, int *__restrict__ ntile, DevStatus *st) {
     __shared__ int cnt;
     const int p = blockIdx.x, m = nnear[p];
     if (threadIdx.x == 0) cnt = 0;
@@ -221,7 +226,8 @@ __global__ void __launch_bounds__(256) cells_tiles_kernel(const uint16_t *__rest
         const int t0 = (int)(sstart[q] / tile), t1 = (int)(sstart[q + 1] / tile);
         const int at = cnt;
         __syncthreads();
-        for (int t = t0 + threadIdx.x; t < t1; t += 256) tiles[(int64_t)p * cap + at + t - t0] = t;
+        for (int t = t0 + threadIdx.x; t < t1; t += 256)
+            if (KC_IN_RANGE(st, at + t - t0, cap, KC_AT_TILE)) tiles[(int64_t)p * cap + at + t - t0] = t;
         if (threadIdx.x == 0) cnt = at + t1 - t0;
         __syncthreads();
     }
@@ -243,7 +249,8 @@ __global__ void __launch_bounds__(CP_NT) cells_prune_kernel(const float *__restr
                                                             const unsigned *__restrict__ sstart,
                                                             const uint16_t *__restrict__ near,
                                                             const int *__restrict__ nnear, const uint32_t *thr_p,
-                                                            uint32_t *__restrict__ Rn, unsigned long long *rnn) {
+                                                            uint32_t *__restrict__ Rn, unsigned long long *rnn, int64_t n,
+                                                            int64_t sn, int64_t rn, DevStatus *st) {
     __shared__ __align__(16) float cs[CP_TILE_BYTES / 4];
     constexpr int TILE = CP_TILE_BYTES / (DR * 4);
     const uint32_t thr = *thr_p;
@@ -258,7 +265,8 @@ __global__ void __launch_bounds__(CP_NT) cells_prune_kernel(const float *__restr
         }
         const int p = lo;
         const uint32_t x = R[r0 + threadIdx.x];
-        bool removed = x == NO_POINT || inS[x];   // d(x, S) = 0 for sampled points
+        // d(x, S) = 0 for sampled points
+        bool removed = x == NO_POINT || !KC_IN_RANGE(st, x, n, KC_AT_EIM_INDEX) || inS[x];
         float xc[DR];
 #pragma unroll
         for (int j = 0; j < DR; ++j) xc[j] = (!removed && j < d) ? src[(int64_t)x * d + j] : 0.f;
@@ -274,7 +282,7 @@ __global__ void __launch_bounds__(CP_NT) cells_prune_kernel(const float *__restr
                 const int take = len < TILE - fill ? len : TILE - fill;
                 for (int i = threadIdx.x; i < take * DR; i += CP_NT) {
                     const int c = i / DR, j = i - c * DR;
-                    cs[(fill + c) * DR + j] = j < d ? Ss[(s0 + c) * d + j] : 0.f;
+                    cs[(fill + c) * DR + j] = j < d && KC_IN_RANGE(st, s0 + c, sn, KC_AT_CELL_POS) ? Ss[(s0 + c) * d + j] : 0.f;
                 }
                 fill += take;
                 if (take == len) {
@@ -302,7 +310,8 @@ __global__ void __launch_bounds__(CP_NT) cells_prune_kernel(const float *__restr
         unsigned long long at = 0;
         if (lane == 0 && keep) at = atomicAdd(rnn, (unsigned long long)__popc(keep));
         at = __shfl_sync(0xFFFFFFFFu, at, 0);
-        if (!removed) Rn[at + __popc(keep & ((1u << lane) - 1u))] = x;
+        at += __popc(keep & ((1u << lane) - 1u));
+        if (!removed && KC_IN_RANGE(st, at, rn, KC_AT_CELL_POS)) Rn[at] = x;
         __syncthreads();
     }
 }
@@ -346,35 +355,36 @@ cudaError_t launch_cells_assign(const float *pk, int64_t n, int d, const CellBuf
     return cudaGetLastError();
 }
 
-cudaError_t launch_cells_sort(const uint32_t *list, int64_t cnt, int unit, const CellBufs &C, CellSort &O,
+cudaError_t launch_cells_sort(const uint32_t *list, int64_t cnt, int unit, const CellBufs &C, CellSort &O, DevStatus *st,
                               cudaStream_t s) {
     cudaMemsetAsync(O.count, 0, 2 * (size_t)C.P * sizeof(unsigned), s);   // counts and radii
     cudaMemsetAsync(O.idx, 0xFF, (size_t)(cnt + (int64_t)C.P * (unit - 1)) * sizeof(uint32_t), s);
     const int g = (int)std::min<int64_t>((cnt + SORT_CHUNK - 1) / SORT_CHUNK, (int64_t)sm_count() * 4);
     const size_t sm = (size_t)C.P * sizeof(unsigned);
-    cells_count_kernel<<<g, SORT_NT, 2 * sm, s>>>(list, cnt, C.P, C.cell, C.dist, O.count, O.count + C.P);
+    cells_count_kernel<<<g, SORT_NT, 2 * sm, s>>>(list, cnt, C.P, C.cell, C.dist, O.count, O.count + C.P, st);
     cells_starts_kernel<<<1, 1024, 0, s>>>(O.count, C.P, unit, O.start, O.cursor);
-    cells_scatter_kernel<<<g, SORT_NT, sm, s>>>(list, cnt, C.P, C.cell, O.cursor, O.idx);
+    cells_scatter_kernel<<<g, SORT_NT, sm, s>>>(list, cnt, C.P, C.cell, O.cursor, O.idx, cnt + (int64_t)C.P * (unit - 1), st);
     note_launches(3);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cells_near(int d, const CellBufs &C, const CellSort &R, const CellSort &S, const uint32_t *thr,
-                              cudaStream_t s) {
+                              DevStatus *st, cudaStream_t s) {
     const double g = f32_gamma(d);   // on the host: FP64 is slow on the device
     cells_near_kernel<<<C.P, NEAR_NT, (size_t)d * sizeof(float), s>>>(
         C.piv, C.P, d, R.count, R.count + C.P, S.count, S.count + C.P, thr, (float)(2.0 * g) + 0x1p-22f,
-        (float)(1.0 - 2.0 * g - 0x1p-18), C.near, C.nnear);
+        (float)(1.0 - 2.0 * g - 0x1p-18), C.near, C.nnear, st);
     note_launches(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_cells_sample(const float *rows, int64_t cnt, int d, const CellBufs &C, CellSort &O, cudaStream_t s) {
+cudaError_t launch_cells_sample(const float *rows, int64_t cnt, int d, const CellBufs &C, CellSort &O, DevStatus *st,
+                                cudaStream_t s) {
     cells_sample_kernel<<<(int)((cnt + 31) / 32), SAMPLE_NT, 0, s>>>(rows, cnt, d, C.piv, C.P, C.cell, C.dist);
     cudaMemsetAsync(O.count, 0, 2 * (size_t)C.P * sizeof(unsigned), s);
     const int g = (int)std::min<int64_t>((cnt + SORT_CHUNK - 1) / SORT_CHUNK, (int64_t)sm_count() * 4);
     cells_count_kernel<<<g, SORT_NT, 2 * (size_t)C.P * sizeof(unsigned), s>>>(nullptr, cnt, C.P, C.cell, C.dist, O.count,
-                                                                              O.count + C.P);
+                                                                              O.count + C.P, st);
     note_launches(2);
     return cudaGetLastError();
 }
@@ -388,8 +398,8 @@ cudaError_t launch_cells_pairs(const CellBufs &C, const CellSort &R, const CellS
 }
 
 cudaError_t launch_cells_tiles(const CellBufs &C, const CellSort &S, int tile, int cap, int *tiles, int *ntile,
-                               cudaStream_t s) {
-    cells_tiles_kernel<<<C.P, 256, 0, s>>>(C.near, C.nnear, C.P, S.start, tile, cap, tiles, ntile);
+                               DevStatus *st, cudaStream_t s) {
+    cells_tiles_kernel<<<C.P, 256, 0, s>>>(C.near, C.nnear, C.P, S.start, tile, cap, tiles, ntile, st);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -398,11 +408,12 @@ int cells_prune_unit() { return CP_NT; }
 
 cudaError_t launch_cells_prune(const float *src, int d, int64_t rn, const uint8_t *inS, const float *Ss,
                                const CellBufs &C, const CellSort &R, const CellSort &S, const uint32_t *thr, uint32_t *Rn,
-                               unsigned long long *rnn, cudaStream_t s) {
+                               unsigned long long *rnn, int64_t n, int64_t sn, DevStatus *st, cudaStream_t s) {
     const int64_t ctas = (rn + (int64_t)C.P * (CP_NT - 1)) / CP_NT;
     const int g = (int)std::min<int64_t>(ctas, (int64_t)sm_count() * 64);
     auto run = [&](auto kern) {
-        kern<<<g, CP_NT, 0, s>>>(src, d, R.idx, R.start, C.P, inS, Ss, S.start, C.near, C.nnear, thr, Rn, rnn);
+        kern<<<g, CP_NT, 0, s>>>(src, d, R.idx, R.start, C.P, inS, Ss, S.start, C.near, C.nnear, thr, Rn, rnn, n, sn, rn,
+                                 st);
     };
     if (d <= 2) run(cells_prune_kernel<2>);
     else if (d <= 4) run(cells_prune_kernel<4>);

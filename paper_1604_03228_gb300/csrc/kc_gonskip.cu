@@ -209,6 +209,9 @@ __global__ void gon_center_rows_kernel(GonInst I, const int *route, const DevSta
 // separated by the group's own barrier (slot rows behind the k exchange rows).
 constexpr int SKIP_ROUNDS = 6;   // regrouping decisions
 
+// Positions of the regrouped arrays, at most: a unit per bin is begun for nothing.
+__host__ __device__ inline int64_t skip_extent(int64_t n) { return nblocks(n + (int64_t)(UNIT - 1) * SKIP_BINS) * BLK; }
+
 struct ShSkip {
     uint64_t red[32];
     uint64_t key;
@@ -278,11 +281,14 @@ __device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I,
     unsigned *cnt = M.bins, *off = M.bins + SKIP_BINS;
     for (int b = tid; b < nbin; b += SKIP_NT) cnt[b] = 0;
     __syncthreads();
-    const int64_t p0 = npos * r / G, p1 = npos * (r + 1) / G;
+    const int64_t p0 = npos * r / G, p1 = npos * (r + 1) / G, extent = skip_extent(I.n);
     auto bin_of = [&](int64_t i) { return 2 * (int)__ldcg(from.asg + i) + (__ldcg(from.mind + i) > far ? 1 : 0); };
 #pragma unroll 4
     for (int64_t i = p0 + tid; i < p1; i += SKIP_NT)
-        if (!from.perm || __ldcg(from.perm + i) != NO_POINT) atomicAdd(&cnt[bin_of(i)], 1u);
+        if (!from.perm || __ldcg(from.perm + i) != NO_POINT) {
+            const int b = bin_of(i);
+            if (KC_IN_RANGE(a.st, b, nbin, KC_AT_SKIP_BIN)) atomicAdd(&cnt[b], 1u);
+        }
     __syncthreads();
     for (int b = tid; b < nbin; b += SKIP_NT) __stcg(I.skip_hist + (int64_t)r * SKIP_BINS + b, cnt[b]);
     __syncthreads();
@@ -355,6 +361,7 @@ __device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I,
         const uint32_t x = from.perm ? __ldcg(from.perm + i) : (uint32_t)i;
         if (x == NO_POINT) continue;
         const unsigned p = atomicAdd(&off[bin_of(i)], 1u);
+        if (!KC_IN_RANGE(a.st, p, extent, KC_AT_SKIP_BIN)) continue;
         __stcg(to.perm + p, x);
         __stcg(to.mind + p, __ldcg(from.mind + i));
         __stcg(to.asg + p, __ldcg(from.asg + i));
@@ -371,6 +378,7 @@ __device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I,
     const int64_t nb = out / BLK;
     // the CTA's units: their centers (before the tiles overwrite the bins) ...
     const int nu = (int)((nb - r + G - 1) / G) * (BLK / UNIT);
+    if (!KC_IN_RANGE(a.st, nu, a.skip_units + 1, KC_AT_SKIP_UNIT) || !KC_IN_RANGE(a.st, out, extent + 1, KC_AT_SKIP_BIN)) return 0;
     for (int u = tid; u < nu; u += SKIP_NT) {
         const unsigned gu = (unsigned)((int64_t)(u / (BLK / UNIT)) * G + r) * (BLK / UNIT) + u % (BLK / UNIT);
         int lo = 0, hi = nbin - 1;   // the last bin that starts at or before the unit
@@ -389,7 +397,8 @@ __device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I,
     for (int u = warp; u < nu; u += SKIP_W) {
         const int64_t b = (int64_t)(u / (BLK / UNIT)) * G + r;
         const int64_t p = b * BLK + (u % (BLK / UNIT)) * UNIT + lane;
-        const uint32_t x = __ldcg(to.perm + p);
+        uint32_t x = __ldcg(to.perm + p);
+        if (x != NO_POINT && !KC_IN_RANGE(a.st, x, I.n, KC_AT_SKIP_ROW)) x = NO_POINT;
         const uint32_t m = x != NO_POINT ? __ldcg(to.mind + p) : 0u;
         const int64_t row = x != NO_POINT ? row_of(I, x) : -1;
         const uint64_t key = warp_max_u64(x != NO_POINT ? make_key(m, x) : 0);
@@ -468,12 +477,14 @@ __device__ __forceinline__ void skip_bounds(const GonInst &I, const SkipMem &M, 
 // The touched units (list[0, n)): distances, minima, assignments, keys.  A
 // warp takes a unit, a lane one point, up to 64 coordinate loads in flight.
 template <int DC>
-__device__ __forceinline__ void skip_units(const GonInst &I, const SkipMem &M, const SkipState &S, int n, int r, int it) {
+__device__ __forceinline__ void skip_units(const GonArgs &a, const GonInst &I, const SkipMem &M, const SkipState &S, int n,
+                                           int r, int it) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int d = DC > 0 ? DC : I.d, G = I.G;
     const float *pk = (const float *)I.pk;
     for (int e = warp; e < n; e += SKIP_W) {
         const int u = (int)M.list[e];
+        if (!KC_IN_RANGE(a.st, u, a.skip_units, KC_AT_SKIP_UNIT)) continue;
         const int64_t b = (int64_t)(u / (BLK / UNIT)) * G + r;
         const int q = (u % (BLK / UNIT)) * UNIT + lane;
         const int64_t p = b * BLK + q;
@@ -559,12 +570,15 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
     SkipState S[2] = {{nullptr, I.mind, I.asg}, {I.skip_perm[0], I.skip_mind[0], I.skip_asg}};
     // slot rows of the regroupings: behind the exchange rows of the k steps
     uint64_t *xrow = I.slots + (int64_t)k * slot_stride(G) * (I.lp_kind ? 2 : 1);
+    uint64_t *const xrow0 = xrow;
     int cur = 0, ncen = 0, nu = 0, it;
     int64_t npos = I.n;
     int next = it0, rounds = 0;   // step of the next regrouping decision
     for (it = it0; it < k; ++it) {
         if (it == next) {
             bool go = rounds == 0;
+            // this decision's rows: the touched units' sum, two of a regrouping, the centers
+            if (!KC_IN_RANGE(a.st, (xrow - xrow0) / G + 3, 4 * SKIP_ROUNDS, KC_AT_SLOT)) break;
             if (!go) {
                 // regroup again when the units touched since the last one are
                 // more than a few percent and enough steps remain
@@ -621,11 +635,12 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
             int at = 0;
             if (lane == 0 && bal) at = atomicAdd(&sh.ntouch, __popc(bal));
             at = __shfl_sync(0xFFFFFFFFu, at, 0);
-            if (touch) M.list[at + __popc(bal & ((1u << lane) - 1u))] = (uint32_t)u;
+            at += __popc(bal & ((1u << lane) - 1u));
+            if (touch && KC_IN_RANGE(a.st, at, a.skip_units, KC_AT_SKIP_UNIT)) M.list[at] = (uint32_t)u;
         }
         __syncthreads();
         const int nt = sh.ntouch;
-        skip_units<DC>(I, M, S[cur], nt, r, it);
+        skip_units<DC>(a, I, M, S[cur], nt, r, it);
         __syncthreads();
         uint64_t best = 0;
         for (int u = tid; u < nu; u += SKIP_NT) best = umax64(best, M.key[u]);
@@ -700,7 +715,7 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
     for (int u = warp; u < nu; u += SKIP_W) {
         const int64_t p = ((int64_t)(u / (BLK / UNIT)) * G + r) * BLK + (u % (BLK / UNIT)) * UNIT + lane;
         const uint32_t x = __ldcg(S[cur].perm + p);
-        if (x != NO_POINT) I.mind[x] = __ldcg(S[cur].mind + p);
+        if (x != NO_POINT && KC_IN_RANGE(a.st, x, I.n, KC_AT_SKIP_ROW)) I.mind[x] = __ldcg(S[cur].mind + p);
     }
     if (r == 0 && tid == 0) {
         *I.k_out = it;
@@ -728,7 +743,7 @@ size_t skip_smem(int d, int units) {
 
 }  // namespace
 
-int64_t skip_positions(int64_t n) { return nblocks(n + (int64_t)(UNIT - 1) * SKIP_BINS) * BLK; }
+int64_t skip_positions(int64_t n) { return skip_extent(n); }
 int64_t skip_route_words() { return 8 + 2 * PROBE_S; }
 int64_t skip_hist_words(int G) { return (int64_t)G * SKIP_BINS; }
 int64_t skip_slot_rows() { return 4 * SKIP_ROUNDS; }

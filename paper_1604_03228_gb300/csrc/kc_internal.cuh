@@ -79,7 +79,13 @@ enum {
     KC_AT_CENTER_COPY = 15,   // a center slot of the transposed FP32 center copy
     KC_AT_EIM_INDEX = 16,     // an index into the points in EIM's kernels
     KC_AT_RADIUS_LIST = 17,   // an entry of the radius recheck's point list
-    KC_AT_SLOT = 18           // a GON exchange slot
+    KC_AT_SLOT = 18,          // a GON exchange slot
+    KC_AT_SKIP_BIN = 19,      // a bin or position of the skip kernel's regrouping
+    KC_AT_SKIP_UNIT = 20,     // a unit of its CTA's share
+    KC_AT_SKIP_ROW = 21,      // a point of its regrouped state
+    KC_AT_CELL = 22,          // a cell of EIM's prune by cells, or a near-list entry
+    KC_AT_CELL_POS = 23,      // a position of its sorted lists
+    KC_AT_TILE = 24           // a center tile of a near list
 };
 
 // ---------------------------------------------------------------- keys
@@ -544,22 +550,23 @@ struct CellSort {
 cudaError_t launch_pivot_rows(const float *rows, int64_t n, int d, const int64_t *centers, const int32_t *k_out, int P,
                               float *piv, cudaStream_t s);
 cudaError_t launch_cells_assign(const float *pk, int64_t n, int d, const CellBufs &C, cudaStream_t s);
-cudaError_t launch_cells_sort(const uint32_t *list, int64_t cnt, int unit, const CellBufs &C, CellSort &O,
+cudaError_t launch_cells_sort(const uint32_t *list, int64_t cnt, int unit, const CellBufs &C, CellSort &O, DevStatus *st,
                               cudaStream_t s);
 cudaError_t launch_cells_near(int d, const CellBufs &C, const CellSort &R, const CellSort &S, const uint32_t *thr,
-                              cudaStream_t s);
+                              DevStatus *st, cudaStream_t s);
 // Cells, counts and radii of the rows [0, cnt) (d < 16; O's list is not made);
 // and the pairs of two lists that the near cells leave.
-cudaError_t launch_cells_sample(const float *rows, int64_t cnt, int d, const CellBufs &C, CellSort &O, cudaStream_t s);
+cudaError_t launch_cells_sample(const float *rows, int64_t cnt, int d, const CellBufs &C, CellSort &O, DevStatus *st,
+                                cudaStream_t s);
 cudaError_t launch_cells_pairs(const CellBufs &C, const CellSort &R, const CellSort &S, unsigned long long *pairs,
                                cudaStream_t s);
 cudaError_t launch_cells_tiles(const CellBufs &C, const CellSort &S, int tile, int cap, int *tiles, int *ntile,
-                               cudaStream_t s);
+                               DevStatus *st, cudaStream_t s);
 int cells_prune_unit();
 // Float points, d <= 16; R sorted with that unit, S with unit 1, Ss its rows.
 cudaError_t launch_cells_prune(const float *src, int d, int64_t rn, const uint8_t *inS, const float *Ss,
                                const CellBufs &C, const CellSort &R, const CellSort &S, const uint32_t *thr, uint32_t *Rn,
-                               unsigned long long *rnn, cudaStream_t s);
+                               unsigned long long *rnn, int64_t n, int64_t sn, DevStatus *st, cudaStream_t s);
 
 struct RadiusArgs {
     const void *pk;

@@ -572,8 +572,10 @@ struct TcArgs {
 // The center tiles of point-tile pair pp: how many, and the i-th.
 struct PairTiles {
     const int *list;
-    int count;
-    __device__ __forceinline__ PairTiles(const TcArgs &a, int64_t pp) : list(nullptr), count(a.ntiles) {
+    int count, ntiles;
+    DevStatus *st;
+    __device__ __forceinline__ PairTiles(const TcArgs &a, int64_t pp)
+        : list(nullptr), count(a.ntiles), ntiles(a.ntiles), st(a.st) {
         if (!a.tiles) return;
         const int64_t r0 = pp * TC_CELL_UNIT;
         int lo = 0, hi = a.P;   // the last cell that starts at or before row r0 (P: past the last row)
@@ -583,9 +585,13 @@ struct PairTiles {
             else hi = mid - 1;
         }
         count = lo < a.P ? __ldg(a.ntile + lo) : 0;
+        if (!KC_IN_RANGE(st, count, a.tcap + 1, KC_AT_TILE)) count = 0;
         list = a.tiles + (int64_t)lo * a.tcap;
     }
-    __device__ __forceinline__ int operator[](int i) const { return list ? __ldg(list + i) : i; }
+    __device__ __forceinline__ int operator[](int i) const {
+        const int t = list ? __ldg(list + i) : i;
+        return KC_IN_RANGE(st, t, ntiles, KC_AT_TILE) ? t : 0;
+    }
 };
 
 __device__ __forceinline__ float tc_eta(int d, int kp) {

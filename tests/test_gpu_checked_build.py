@@ -96,6 +96,50 @@ def test_checked_build_runs_clean_and_catches_a_planted_index(kc):
     assert p.returncode == 0 and "checked build: OK" in p.stdout, p.stdout[-3000:] + p.stderr[-3000:]
 
 
+CHILD_SKIP = r'''
+import os
+import numpy as np
+import torch
+import paper_1604_03228_gb300 as kc
+from oracle import oracle as O
+from paper_1604_03228_gb300 import inputs as I
+
+assert kc.load()._name.endswith("libkcenter_checks.so")
+dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+os.environ.update(KC_GON_SKIP="1", KC_GON_RESIDENT="0", KC_EIM_CELLS="1")
+
+for n, d, k in ((60_000, 64, 300), (50_000, 2, 600), (33_333, 37, 100), (3_000, 1100, 30), (31, 3, 30)):
+    p = I.gauss_mixture(n, d, 900 + d, 20, 0.5, -10.0, 10.0)
+    ref = O.gonzalez(p, k, mode="f32")
+    for sw in ("f32", "bf16"):
+        r = kc.kc_gonzalez(dev(p), k, sweep=sw)
+        assert r.centers.cpu().numpy().tolist() == ref.centers.tolist(), (n, d, k, sw)
+for d, stream, cap in ((3, "0", None), (9, "0", None), (20, "1", None), (64, "1", "1")):
+    if d >= 16:
+        os.environ["KC_TC_STREAM_CENTERS"] = "1"
+    if cap:
+        os.environ["KC_PRUNE_PAIR_CAP"] = cap
+    p = I.gauss_mixture(30_011, d, 920 + d, 30, 0.5, -10.0, 10.0)
+    e = kc.kc_eim(dev(p), 4, eps=0.1, phi=6.0, seed=920 + d)
+    assert e.centers.cpu().numpy().tolist() == O.eim(p, 4, 0.1, 6.0, 920 + d, mode="f32").centers.tolist(), d
+x = dev(I.gauss_mixture(800_000, 12, 930, 40, 0.5, -10.0, 10.0))   # EIM's sample through the skip kernel
+a = kc.kc_eim(x, 200, seed=3)
+os.environ["KC_GON_SKIP"] = os.environ["KC_EIM_CELLS"] = "0"
+b = kc.kc_eim(x, 200, seed=3)
+assert a.centers.cpu().tolist() == b.centers.cpu().tolist() and a.radius == b.radius
+print("checked build: OK")
+'''
+
+
+def test_checked_build_of_the_kernels_that_leave_out_distances(kc):
+    """Gonzalez with several regroupings, alone and on EIM's sample, and EIM's
+    prune by cells on the CUDA and the tensor cores: no check fires."""
+    from paper_1604_03228_gb300 import build
+    env = dict(os.environ, KC_LIBRARY=build.build(checks=True))
+    p = subprocess.run([sys.executable, "-c", CHILD_SKIP], env=env, cwd=ROOT, capture_output=True, text=True, timeout=1500)
+    assert p.returncode == 0 and "checked build: OK" in p.stdout, p.stdout[-3000:] + p.stderr[-3000:]
+
+
 def test_regular_build_rejects_the_checked_build_flag(kc):
     import torch
     x = torch.from_numpy(I.gauss_mixture(20_000, 4, 9, 3, 1.0, 0, 1)).cuda()
