@@ -96,8 +96,24 @@ __device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T 
                 }
         }
     } else {
-#pragma unroll UNR
-        for (int j = 0; j < d; ++j) {
+        // whole groups of UNR coordinates, then by fours: a loop unrolled by eight
+        // loads what is left one at a time (MRG on 10M x 4, m = 64: 5.4 ms, so 3.7,
+        // by fours alone 4.1; 3M x 30 14.3, 13.3, 15.1)
+        int j = 0;
+#pragma unroll 1
+        for (; j + UNR <= d; j += UNR) {
+#pragma unroll
+            for (int t = 0; t < UNR; ++t) {
+                const V4 v = __ldg(src + (j + t) * (BLK / 4));
+                const T c = cs[j + t];
+                a0 = sq_step(a0, v.x, c);
+                a1 = sq_step(a1, v.y, c);
+                a2 = sq_step(a2, v.z, c);
+                a3 = sq_step(a3, v.w, c);
+            }
+        }
+#pragma unroll 4
+        for (; j < d; ++j) {
             const V4 v = __ldg(src + j * (BLK / 4));
             const T c = cs[j];
             a0 = sq_step(a0, v.x, c);

@@ -41,6 +41,13 @@ def test_mrg_float_even(kc, n, d, m, k):
     check_mrg(kc, pts, k, I.even_offsets(n, m))
 
 
+@pytest.mark.parametrize("d", [1, 4, 5, 6, 7, 9, 11, 12, 13, 15])
+def test_mrg_coordinate_remainders(kc, d):
+    """The queue kernels' loop: groups of eight coordinates, then by fours."""
+    check_mrg(kc, I.gauss_mixture(9_001, d, 440 + d, 8, 1.0, -10, 10), 9, I.even_offsets(9_001, 5))
+    check_mrg(kc, I.int_points(9_001, d, 441 + d, -60, 60), 9, I.even_offsets(9_001, 5))
+
+
 def test_mrg_zipf_parts(kc):
     n, m, k = 300_000, 64, 20
     pts = I.unif_points(n, 16, 41)
