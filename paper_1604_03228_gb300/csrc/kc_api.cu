@@ -1444,7 +1444,7 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
     int Pmax = !cells_ok ? 0 : (d < 16 ? CELLS_MAX : EIM_PIVOTS_TC);
     int64_t npad = n + (int64_t)Pmax * (TC_CELL_UNIT - 1);   // a list sorted by cell
     constexpr int64_t PSAMPLE = 8192;   // rows of S the pivots are chosen from (d >= 16)
-    constexpr int64_t CSAMPLE = 32768;  // rows of S that show whether cells pay (4 < d < 16)
+    constexpr int64_t CSAMPLE = 32768;  // rows of S that show whether cells pay (2 < d < 16)
     CellBufs CB;
     CellSort CR, CS;
     int *ctiles = nullptr, *cntile = nullptr;
@@ -1700,8 +1700,8 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
                 // Below d = 16 the assignment to up to 1024 pivots is a few
                 // percent of the block, so part of S stands for both sides; its
                 // cells reach less far, and its share is a sixth to a third
-                // lower.  Up to d = 4 no point set gave more than 0.3.
-                if (!cenv && d > 4 && d < 16) {
+                // lower.  In the plane no point set came near the line.
+                if (!cenv && d > 2 && d < 16) {
                     const int64_t M = std::min<int64_t>(sn, CSAMPLE);
                     KC_CUDA(launch_cells_sample((const float *)Lo.Sc, M, d, CB, CR, st, c.s), "sample cells");
                     KC_CUDA(launch_cells_near(d, CB, CR, CR, Lo.thr, st, c.s), "sample near cells");

@@ -110,3 +110,12 @@ def test_cells_only_where_a_sample_shows_that_they_pay(kc, monkeypatch, n, d, k)
     (t, a), (t0, b) = _timed(kc, monkeypatch, x, k, None), _timed(kc, monkeypatch, x, k, "0")
     assert a == b
     assert t < 1.07 * t0, (t, t0)
+
+
+def test_cells_of_few_pivots_are_counted_too(kc, monkeypatch):
+    # one cluster in four dimensions and a small S: few pivots, most cells near
+    import torch
+    x = torch.randn(478_764, 4, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+    (t, a), (t0, b) = _timed(kc, monkeypatch, x, 12, None), _timed(kc, monkeypatch, x, 12, "0")
+    assert a == b
+    assert t < 1.07 * t0, (t, t0)
