@@ -35,7 +35,6 @@ phi on 2-D sets shaped like the paper's experiments instead.
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import statistics
@@ -64,13 +63,6 @@ CPU_K_SHARD = 32      # oracle sample, all cores: GON with 32 centers on each co
 # same instances as one kc_gonzalez call each (the unbatched baseline).
 EXTRA = (CFG2, "gon_int_n10000_d2_k10", "gon_unif_n10000000_d16_k200", "mrg_unif_n10000000_d16_m64_k200",
          "radius_gau_n8000000_d64_k1024", "eim_gau_n8000000_d64_k1024", "batch_4096", "batch_4096_per_call")
-
-# DRAM traffic (read + write bytes) per launch of the dominant kernel from an
-# ncu capture, keyed by the SHA-256 of the kernel's source file at capture
-# time; reported only while the source is unchanged.  Values are for the
-# full workload (a smaller capture scaled by the units processed).
-NCU_TRAFFIC = {}
-
 
 def parse():
     ap = argparse.ArgumentParser()
@@ -412,8 +404,6 @@ def run_gpu(args):
     alg_bytes = k * n * (4 * D + 4)
     achieved = alg_bytes / (gon_avg / 1e3) / 1e9
     peak, peak_kind = peaks()
-    src = open(os.path.join(ROOT, "paper_1604_03228_gb300", "csrc", "kc_gon.cu"), "rb").read()
-    traffic = NCU_TRAFFIC.get(hashlib.sha256(src).hexdigest()) if (n, k) == (N, K) else None
     shares = {}
     for name, nk, ms in trace:
         shares[name] = shares.get(name, 0.0) + ms
@@ -478,7 +468,7 @@ def run_gpu(args):
                            "evals": "the k n point-center pairs that a solve decides",
                            "sweep": "f32", "replicas": world},
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                             "frac": achieved / peak, "traffic": traffic,
+                             "frac": achieved / peak, "traffic": None,
                              "kernel": "gon_group_kernel (first steps), gon_skip_kernel (the rest)",
                              "peak_kind": peak_kind, "avg_ms": gon_avg, "alg_bytes_per_launch": alg_bytes,
                              "alg_bytes_rule": "k n (4 d + 4): each step reads every point and its running minimum; the "

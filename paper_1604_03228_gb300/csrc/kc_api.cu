@@ -502,7 +502,9 @@ cudaError_t launch_gon_segments(GonArgs &g, const int *ends, int nseg, int *rout
     return e;
 }
 
-// Pivots of EIM's prune on the tensor cores.
+// Pivots of EIM's prune on the tensor cores: each cell's list is padded to tiles
+// of 256, so at most 128 x 255 positions are added.  Sets of many more clusters
+// keep nearly all pairs near and take the whole block.
 constexpr int EIM_PIVOTS_TC = 128;
 
 int choose_gon_grid(int dtype, int d, int64_t n, int lp = 0) {
@@ -1838,14 +1840,13 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
 // longest-first, which the CTAs join when their list is done.  If groups of
 // any size fit side by side they are not rounded and all start at once.  Batches
 // whose slots would take much scratch use the one-level split below, theta 1.
-// Before, instances above the share took groups of the first half of the CTAs
-// once, and what did not fit there was left to single CTAs.  Measured on
-// mixed batches (d 3, 8, 32; k 8 to 128; GON launch alone, before / now, ms):
+// Measured on mixed batches (d 3, 8, 32; k 8 to 128; GON launch alone, one-level
+// split and the generic sweep / these groups and the sweep of each d, ms):
 //   instances x points         FP32           bf16
-//   4096 x 1k..200k          87.6 / 60.6    62.4 / 59.1
-//    512 x 1k..200k          17.8 /  8.2    25.4 / 13.4
-//     69 x 1k..200k           6.2 /  1.9    13.9 /  2.8
-//    905 x 1k..20k            2.6 /  1.9     3.9 /  3.4
+//   4096 x 1k..200k          95.5 / 60.6    71.4 / 59.1
+//    512 x 1k..200k          33.5 /  8.2    36.2 / 13.4
+//     69 x 1k..200k          13.3 /  1.6    22.1 /  2.7
+//    905 x 1k..20k            4.2 /  1.9     5.4 /  3.4
 // bf16 does not group by L2: it is issue-bound, with two exchanges a step
 // (4096: 62.5 -> 83 ms).
 //
@@ -1888,9 +1889,10 @@ void batch_teams(BatchShape &b, const int64_t *n, const int32_t *d, const int32_
     int dev = 0, l2 = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
-    // From d = 96 on a step's sweep from memory is as fast (3000 instances of
-    // up to 5000 points, ms with / without this criterion: d = 64 18.3 / 23.8, 80
-    // 26.4 / 30.6, 90 34.7 / 34.6, 100 41.4 / 38.0, 128 56.7 / 48.8).
+    // From d = 96 on (int32 48) a step's sweep from memory is as fast (3000
+    // instances of up to 5000 points, ms with / without this criterion: d = 64 18.3
+    // / 23.8, 80 26.4 / 30.6, 90 34.7 / 34.6, 100 41.4 / 38.0, 128 56.7 / 48.8; int32
+    // 64 25.5 / 23.7, 100 44.1 / 35.4).
     const int L2_D = b.dtype == KC_F32 ? 96 : 48;
     const double part = b.lp ? 0.0 : (double)l2 / slots;   // a CTA's part of L2 (0: not a criterion)
     std::vector<int> size((size_t)b.count);

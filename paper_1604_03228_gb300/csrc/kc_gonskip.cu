@@ -19,9 +19,9 @@
 //   assign   every point's minimum over the centers so far and the center
 //            that gives it;
 //   skip     the remaining steps, one persistent cooperative launch.
-// 8M x 64, 100 Gaussian clusters, k = 1024 (GB300): 314 -> 41.5 ms per solve
-// (64 streaming steps 20.4 ms, probes 0.07, assignment 2.2, 960 skip steps and
-// two regroupings 17.7; 11.9 us a step once the clusters are covered, the
+// 8M x 64, 100 Gaussian clusters, k = 1024 (GB300): 314 -> 41.3 ms per solve
+// (32 streaming steps 9.8 ms, probes 0.04, assignment 1.2, 992 skip steps and
+// their regroupings 29; 11.9 us a step once the clusters are covered, the
 // 20 MB of one cluster's points per step being 2.9 us of it at the HBM rate);
 // with the bf16 sweep before the change-over 181 -> 34.4 ms.
 #include <algorithm>

@@ -374,7 +374,7 @@ int device_clock_khz(int dev);
 __host__ __device__ inline int64_t slot_stride(int G) { return (int64_t)G; }
 inline int64_t slot_words(int64_t k, int G, bool lp) { return k * slot_stride(G) * (lp ? 2 : 1); }
 // Words the first CTA of a large group publishes a step's result in
-// (group_exchange): the key's halves and the d coordinates.
+// (kc_gon.cuh): the key's halves and the d coordinates.
 inline int64_t bc_words(int d) { return (d + 2 + 15) / 16 * 16; }
 int gon_queue_warps();
 int gon_warps_per_cta();
