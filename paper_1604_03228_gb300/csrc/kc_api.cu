@@ -460,13 +460,7 @@ void attach_lp(GonInst &I, const LPBufs &L, int lp, float *cenT, int kcap, float
 }
 
 // Scratch of the skip kernel (kc_gonskip.cu) for n points.
-struct SkipBufs {
-    uint16_t *asg[2];
-    uint32_t *perm[2], *mind[2];
-    unsigned *hist;
-};
-
-void take_skip(Carve &cv, SkipBufs &B, int64_t n, int grid) {
+void take_skip(Carve &cv, GonSkip &B, int64_t n, int grid) {
     const size_t np = (size_t)skip_positions(n);
     for (int i = 0; i < 2; ++i) {
         B.asg[i] = cv.take<uint16_t>(np);
@@ -474,16 +468,6 @@ void take_skip(Carve &cv, SkipBufs &B, int64_t n, int grid) {
         B.mind[i] = cv.take<uint32_t>(np);
     }
     B.hist = cv.take<unsigned>((size_t)skip_hist_words(grid));
-}
-
-void attach_skip(GonInst &I, const SkipBufs &B) {
-    I.asg = B.asg[0];
-    I.skip_asg = B.asg[1];
-    for (int i = 0; i < 2; ++i) {
-        I.skip_perm[i] = B.perm[i];
-        I.skip_mind[i] = B.mind[i];
-    }
-    I.skip_hist = B.hist;
 }
 
 // A single instance: the streaming kernel to the end, or (nseg > 0) in
@@ -496,7 +480,7 @@ cudaError_t launch_gon_segments(GonArgs &g, const int *ends, int nseg, int *rout
         g.single.it1 = i < nseg ? ends[i] : 0;
         e = launch_gon(g, s);
         if (i < nseg && e == cudaSuccess)
-            e = launch_gon_probe(g.single, ends[i], i == nseg - 1, route, (unsigned *)route + 4, g.st, s);
+            e = launch_gon_probe(g, ends[i], i == nseg - 1, (unsigned *)route + 4, s);
     }
     if (nseg && e == cudaSuccess) e = launch_gon_skip(g, ends[nseg - 1], s);
     return e;
@@ -726,7 +710,7 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
     const size_t esz = 4;
     LPBufs LB;
     float *cenT = nullptr, *ecmax = nullptr;
-    SkipBufs SB;
+    GonSkip SB{};
     unsigned *route = nullptr;   // the route word and the probe's words
 
     auto layout = [&](Carve &cv, GonArgs &g, RadiusArgs &ra, void **staging, int64_t **cen_dev,
@@ -835,7 +819,7 @@ kc_status kc_gonzalez(const void *pts, int64_t n, int32_t d, int32_t k, int64_t 
     // exact rechecks read the FP32 rows where they are in device memory
     if ((lp && !pin_pts) || nseg) g.single.rm = (const float *)src;
     if (nseg) {
-        attach_skip(g.single, SB);
+        g.skip = SB;
         ra.pk = nullptr;   // the skip kernel packs the points anew, in its own order
         ra.rm = (const float *)src;
         g.single.cenT = cenT;
@@ -1452,7 +1436,7 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
     int *ctiles = nullptr, *cntile = nullptr;
     unsigned long long *cpairs = nullptr;
     bool assigned = false, no_cells = false;
-    SkipBufs SB{};
+    GonSkip SB{};
     bool skip_ok = !lp && gon_skip_possible(c.o.dtype, d, n, keff_max, grid);
     LPBufs LB;
     float *cenT = nullptr, *ecmax = nullptr;
@@ -1786,9 +1770,9 @@ kc_status kc_eim(const void *pts, int64_t n, int32_t d, int32_t k, double eps, i
         int seg_end[8];
         const int nseg = skip_ok ? gon_skip_segments(c.o.dtype, d, nC, kC, g.grid, seg_end, 8) : 0;
         if (nseg) {   // the rows of the sample are found through its index
-            attach_skip(g.single, SB);
+            g.skip = SB;
             g.single.rm = (const float *)src;
-            g.single.rmap = Lo.C;
+            g.skip.rmap = Lo.C;
             g.single.cenT = Lo.cenT;
             g.route = (int *)Lo.route;
         }

@@ -165,12 +165,13 @@ __global__ void __launch_bounds__(PROBE_NT) gon_probe_kernel(const float *__rest
 // Minimum over the first *route centers of every point of the packed array
 // (into mind) and the position of the center that gives it (asg).
 template <int DC>
-__global__ void __launch_bounds__(NEAREST_NT, 2) gon_assign_kernel(GonInst I, const int *route, const DevStatus *st) {
+__global__ void __launch_bounds__(NEAREST_NT, 2) gon_assign_kernel(GonInst I, uint16_t *asg, const int *route,
+                                                                   const DevStatus *st) {
     extern __shared__ __align__(16) float as_cen[];
     const int it0 = ld_volatile_i32(route);
     if (it0 == 0 || ld_volatile_i32(&st->code) != 0) return;
     nearest_centers<DC>((const float *)I.pk, I.n, I.d, it0, as_cen,
-                        [&](int c, int j) { return I.cenT[(int64_t)j * I.kcap + c]; }, I.mind, I.asg);
+                        [&](int c, int j) { return I.cenT[(int64_t)j * I.kcap + c]; }, I.mind, asg);
 }
 
 // The first *route centers' coordinates, transposed ([d][kcap]).
@@ -260,7 +261,7 @@ struct SkipMem {   // shared memory of a CTA
 __device__ __forceinline__ bool rep_shared(int ncen, int d) { return ncen * d <= SKIP_W * SKIP_TILE; }
 
 // One point's row number in rm.
-__device__ __forceinline__ int64_t row_of(const GonInst &I, uint32_t x) { return I.rmap ? I.rmap[x] : (int64_t)x; }
+__device__ __forceinline__ int64_t row_of(const GonSkip &K, uint32_t x) { return K.rmap ? K.rmap[x] : (int64_t)x; }
 
 // Counting sort of the positions by bin and repacking of the CTA's blocks.
 // from / to: the state (perm, mind, asg) before and after; from.perm null: the
@@ -272,12 +273,12 @@ struct SkipState {
 constexpr uint32_t NO_POINT = 0xFFFFFFFFu;
 
 template <int DC>
-__device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I, ShSkip &sh, const SkipMem &M, int r,
+__device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I, const GonSkip &SK, ShSkip &sh, const SkipMem &M, int r,
                                              int ncen, uint32_t far, int64_t npos, const SkipState &from,
                                              const SkipState &to, uint64_t *rows) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int d = DC > 0 ? DC : I.d, G = I.G, nbin = 2 * ncen;
-    const float g2 = a.skip_g2;
+    const float g2 = a.skip.g2;
     unsigned *cnt = M.bins, *off = M.bins + SKIP_BINS;
     for (int b = tid; b < nbin; b += SKIP_NT) cnt[b] = 0;
     __syncthreads();
@@ -290,7 +291,7 @@ __device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I,
             if (KC_IN_RANGE(a.st, b, nbin, KC_AT_SKIP_BIN)) atomicAdd(&cnt[b], 1u);
         }
     __syncthreads();
-    for (int b = tid; b < nbin; b += SKIP_NT) __stcg(I.skip_hist + (int64_t)r * SKIP_BINS + b, cnt[b]);
+    for (int b = tid; b < nbin; b += SKIP_NT) __stcg(SK.hist + (int64_t)r * SKIP_BINS + b, cnt[b]);
     __syncthreads();
     if (warp == 0) {
         bool ab = false;
@@ -305,7 +306,7 @@ __device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I,
         if (b < nbin) {
 #pragma unroll 8
             for (int q = 0; q < G; ++q) {
-                const unsigned v = __ldcg(I.skip_hist + (int64_t)q * SKIP_BINS + b);
+                const unsigned v = __ldcg(SK.hist + (int64_t)q * SKIP_BINS + b);
                 if (q < r) mine += v;
                 tot += v;
             }
@@ -378,7 +379,7 @@ __device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I,
     const int64_t nb = out / BLK;
     // the CTA's units: their centers (before the tiles overwrite the bins) ...
     const int nu = (int)((nb - r + G - 1) / G) * (BLK / UNIT);
-    if (!KC_IN_RANGE(a.st, nu, a.skip_units + 1, KC_AT_SKIP_UNIT) || !KC_IN_RANGE(a.st, out, extent + 1, KC_AT_SKIP_BIN)) return 0;
+    if (!KC_IN_RANGE(a.st, nu, a.skip.units + 1, KC_AT_SKIP_UNIT) || !KC_IN_RANGE(a.st, out, extent + 1, KC_AT_SKIP_BIN)) return 0;
     for (int u = tid; u < nu; u += SKIP_NT) {
         const unsigned gu = (unsigned)((int64_t)(u / (BLK / UNIT)) * G + r) * (BLK / UNIT) + u % (BLK / UNIT);
         int lo = 0, hi = nbin - 1;   // the last bin that starts at or before the unit
@@ -400,7 +401,7 @@ __device__ __noinline__ int64_t skip_regroup(const GonArgs &a, const GonInst &I,
         uint32_t x = __ldcg(to.perm + p);
         if (x != NO_POINT && !KC_IN_RANGE(a.st, x, I.n, KC_AT_SKIP_ROW)) x = NO_POINT;
         const uint32_t m = x != NO_POINT ? __ldcg(to.mind + p) : 0u;
-        const int64_t row = x != NO_POINT ? row_of(I, x) : -1;
+        const int64_t row = x != NO_POINT ? row_of(SK, x) : -1;
         const uint64_t key = warp_max_u64(x != NO_POINT ? make_key(m, x) : 0);
         if (lane == 0) {
             M.key[u] = key;
@@ -484,7 +485,7 @@ __device__ __forceinline__ void skip_units(const GonArgs &a, const GonInst &I, c
     const float *pk = (const float *)I.pk;
     for (int e = warp; e < n; e += SKIP_W) {
         const int u = (int)M.list[e];
-        if (!KC_IN_RANGE(a.st, u, a.skip_units, KC_AT_SKIP_UNIT)) continue;
+        if (!KC_IN_RANGE(a.st, u, a.skip.units, KC_AT_SKIP_UNIT)) continue;
         const int64_t b = (int64_t)(u / (BLK / UNIT)) * G + r;
         const int q = (u % (BLK / UNIT)) * UNIT + lane;
         const int64_t p = b * BLK + q;
@@ -530,19 +531,21 @@ template <int DC>
 __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ GonInst I;
+    __shared__ GonSkip SK;
     __shared__ ShSkip sh;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) SK = a.skip;
     copy_instance(I, &a.single);
     const int it0 = ld_volatile_i32(a.route);
     if (it0 == 0 || ld_volatile_i32(&a.st->code) != 0) return;
     const int r = (int)blockIdx.x, G = I.G, k = I.k;
     const int d = DC > 0 ? DC : I.d;
-    const float g2 = a.skip_g2;
+    const float g2 = a.skip.g2;
     SkipMem M;
     M.key = reinterpret_cast<unsigned long long *>(smem_raw);
-    M.rho = reinterpret_cast<float *>(M.key + a.skip_units);
-    M.list = reinterpret_cast<uint32_t *>(M.rho + a.skip_units);
-    M.cs = reinterpret_cast<float *>(M.list + a.skip_units);
+    M.rho = reinterpret_cast<float *>(M.key + a.skip.units);
+    M.list = reinterpret_cast<uint32_t *>(M.rho + a.skip.units);
+    M.cs = reinterpret_cast<float *>(M.list + a.skip.units);
     M.h = M.cs + ((d + 3) & ~3);
     M.bins = reinterpret_cast<unsigned *>(M.h + SKIP_BINS / 2);
     M.tile = reinterpret_cast<float *>(M.bins);
@@ -555,7 +558,7 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
         const int64_t c = key_idx(K);
         const bool ok = KC_IN_RANGE(a.st, c, I.n, KC_AT_CENTER_LOAD) && KC_IN_RANGE(a.st, it0, I.kcap, KC_AT_CENTER_COPY);
         if (ok) {
-            for (int j = lane; j < d; j += 32) M.cs[j] = I.rm[row_of(I, (uint32_t)c) * d + j];
+            for (int j = lane; j < d; j += 32) M.cs[j] = I.rm[row_of(SK, (uint32_t)c) * d + j];
             if (r == 0 && lane == 0) I.centers[it0] = out_index(I, c);
         }
         if (lane == 0) {
@@ -567,7 +570,7 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
     __syncthreads();
     if (sh.abort) return;
     // the state in point order, then the two regrouped ones in turn
-    SkipState S[2] = {{nullptr, I.mind, I.asg}, {I.skip_perm[0], I.skip_mind[0], I.skip_asg}};
+    SkipState S[2] = {{nullptr, I.mind, SK.asg[0]}, {SK.perm[0], SK.mind[0], SK.asg[1]}};
     // slot rows of the regroupings: behind the exchange rows of the k steps
     uint64_t *xrow = I.slots + (int64_t)k * slot_stride(G) * (I.lp_kind ? 2 : 1);
     uint64_t *const xrow0 = xrow;
@@ -599,11 +602,11 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
             }
             if (go) {
                 const uint32_t far = __float_as_uint(0.25f * __uint_as_float(key_val(K)));
-                const int64_t np = skip_regroup<DC>(a, I, sh, M, r, it, far, npos, S[cur], S[cur ^ 1], xrow);
+                const int64_t np = skip_regroup<DC>(a, I, SK, sh, M, r, it, far, npos, S[cur], S[cur ^ 1], xrow);
                 if (np == 0) break;
                 xrow += 2 * G;
                 npos = np;
-                if (rounds == 0) S[0] = {I.skip_perm[1], I.skip_mind[1], I.asg};
+                if (rounds == 0) S[0] = {SK.perm[1], SK.mind[1], SK.asg[0]};
                 cur ^= 1;
                 ncen = it;
                 nu = (int)((npos / BLK - r + G - 1) / G) * (BLK / UNIT);
@@ -623,7 +626,7 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
             ++rounds;
             next = 2 * it <= SKIP_BINS / 2 && rounds < SKIP_ROUNDS ? 2 * it : k;
         }
-        skip_bounds(I, M, d, ncen, a.skip_f);
+        skip_bounds(I, M, d, ncen, a.skip.f);
         for (int u0 = 0; u0 < nu; u0 += SKIP_NT) {
             const int u = u0 + tid;
             bool touch = false;
@@ -636,7 +639,7 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
             if (lane == 0 && bal) at = atomicAdd(&sh.ntouch, __popc(bal));
             at = __shfl_sync(0xFFFFFFFFu, at, 0);
             at += __popc(bal & ((1u << lane) - 1u));
-            if (touch && KC_IN_RANGE(a.st, at, a.skip_units, KC_AT_SKIP_UNIT)) M.list[at] = (uint32_t)u;
+            if (touch && KC_IN_RANGE(a.st, at, a.skip.units, KC_AT_SKIP_UNIT)) M.list[at] = (uint32_t)u;
         }
         __syncthreads();
         const int nt = sh.ntouch;
@@ -659,7 +662,7 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
             const bool more = it + 1 < k;
             // the CTA's candidate may be the next center: have its row on the way
             if (more && v != 0) {
-                const float *row = I.rm + row_of(I, key_idx(v)) * d;
+                const float *row = I.rm + row_of(SK, key_idx(v)) * d;
                 for (int j = lane * 8; j < d; j += 256) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + j));
             }
             const bool lead = G > LEADER_MIN;
@@ -683,7 +686,7 @@ __global__ void __launch_bounds__(SKIP_NT, 1) gon_skip_kernel(GonArgs a) {
             if (!ab && more && (!lead || r == 0)) {
                 const int64_t c = key_idx(g);
                 if (key_val(g) == 0 || KC_IN_RANGE(a.st, c, I.n, KC_AT_CENTER_LOAD)) {
-                    const float *src = key_val(g) != 0 ? I.rm + row_of(I, (uint32_t)c) * d : nullptr;
+                    const float *src = key_val(g) != 0 ? I.rm + row_of(SK, (uint32_t)c) * d : nullptr;
                     for (int j = lane; j < d; j += 32) {
                         const float x = src ? __ldg(src + j) : 0.f;
                         M.cs[j] = x;
@@ -773,8 +776,8 @@ bool gon_skip_possible(int dtype, int d, int64_t n, int k, int grid) {
     return gon_skip_segments(dtype, d, n, k, grid, ends, 8) > 0;
 }
 
-cudaError_t launch_gon_probe(const GonInst &I, int it0, bool last, int *route, unsigned *words, DevStatus *st,
-                             cudaStream_t s) {
+cudaError_t launch_gon_probe(const GonArgs &a, int it0, bool last, unsigned *words, cudaStream_t s) {
+    const GonInst &I = a.single;
     // microseconds: a whole sweep at the HBM rate, or the one of L2 where the
     // points stay there (half the bytes in mixed precision), the assignment at
     // the FP32 rate and two regroupings
@@ -793,9 +796,9 @@ cudaError_t launch_gon_probe(const GonInst &I, int it0, bool last, int *route, u
     // beyond a streaming step's exchange, with the tests of all units (10M x 10, a tenth
     // of the units touched: 36 us a step, 26 of them the units, 3.5 the exchange)
     const float fixed = (float)(3.0 + n / 2e6);
-    gon_probe_kernel<<<PROBE_CTAS, PROBE_NT, 0, s>>>(I.rm, I.rmap, I.n, I.d, I.centers, I.final_key, it0,
-                                                     force ? 1e9f : sweep, unit, fixed, once, I.k - it0, last, route,
-                                                     words, reinterpret_cast<uint2 *>(words + 4), st);
+    gon_probe_kernel<<<PROBE_CTAS, PROBE_NT, 0, s>>>(I.rm, a.skip.rmap, I.n, I.d, I.centers, I.final_key, it0,
+                                                     force ? 1e9f : sweep, unit, fixed, once, I.k - it0, last, a.route,
+                                                     words, reinterpret_cast<uint2 *>(words + 4), a.st);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -808,16 +811,16 @@ cudaError_t launch_gon_skip(GonArgs &a, int last, cudaStream_t s) {
     gon_center_rows_kernel<<<(int)std::min<int64_t>(sms, ((int64_t)last * I.d + 255) / 256), 256, 0, s>>>(I, a.route, a.st);
     const size_t smem_a = nearest_smem(I.d);
     const int ga = nearest_grid(I.n, sms);
-    if (I.d == 64) gon_assign_kernel<64><<<ga, NEAREST_NT, smem_a, s>>>(I, a.route, a.st);
-    else gon_assign_kernel<0><<<ga, NEAREST_NT, smem_a, s>>>(I, a.route, a.st);
+    if (I.d == 64) gon_assign_kernel<64><<<ga, NEAREST_NT, smem_a, s>>>(I, a.skip.asg[0], a.route, a.st);
+    else gon_assign_kernel<0><<<ga, NEAREST_NT, smem_a, s>>>(I, a.skip.asg[0], a.route, a.st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     void *fn = pick_skip(I.d);
-    a.skip_units = skip_units_max(I.n, a.grid);
+    a.skip.units = skip_units_max(I.n, a.grid);
     // FP64 is slow here: taken once, not by every thread
-    a.skip_g2 = (float)(2.0 * f32_gamma(I.d)) + 0x1p-22f;
-    a.skip_f = (float)(1.0 - 2.0 * f32_gamma(I.d) - 0x1p-18);
-    const size_t smem = skip_smem(I.d, a.skip_units);
+    a.skip.g2 = (float)(2.0 * f32_gamma(I.d)) + 0x1p-22f;
+    a.skip.f = (float)(1.0 - 2.0 * f32_gamma(I.d) - 0x1p-18);
+    const size_t smem = skip_smem(I.d, a.skip.units);
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
     note_launches(3);
     cudaLaunchConfig_t cfg = {};

@@ -272,17 +272,6 @@ struct GonInst {
     // low-precision pack), so a recheck evaluates only the newer centers
     uint32_t *m32;
     uint32_t *stamp;
-    // skip kernel (kc_gonskip.cu): per point of the packed array the center
-    // (its position in the selection) that gave the running minimum, and the
-    // row of rm that holds local point i (nullptr: row i); cenT as above
-    uint16_t *asg;
-    const int64_t *rmap;
-    // its regrouped states (two in turn), skip_positions(n) entries each (asg
-    // and pk have as many): the point of a position, minima, assignments (the
-    // second state's in asg); the regrouping's bin counts
-    uint32_t *skip_perm[2], *skip_mind[2];
-    uint16_t *skip_asg;
-    unsigned *skip_hist;
     // this launch runs steps [it0, it1) of the k (it1 = 0: to the end); from
     // it0 > 0 on, the state of the steps before it is in place and the first
     // center is the one *final_key names
@@ -297,6 +286,22 @@ struct GonInst {
     int32_t k;
     int32_t cta0;
     int32_t G;
+};
+
+// The skip kernel's part of a single instance (kc_gonskip.cu), beside the
+// instance: lists of instances, some of 100,000, do without it.  asg[0] holds,
+// per point of the packed array, the center (its position in the selection)
+// that gave the running minimum.
+struct GonSkip {
+    const int64_t *rmap;     // the row of rm that holds local point i (nullptr: row i)
+    // its regrouped states, two in turn, skip_positions(n) entries each (pk has as
+    // many): the point of a position, minima, assignments (the second state's in
+    // asg[0]); the regrouping's bin counts
+    uint32_t *perm[2], *mind[2];
+    uint16_t *asg[2];
+    unsigned *hist;
+    int units;               // units of 32 points a CTA has room for
+    float g2, f;             // slack factors for this d
 };
 
 struct GonArgs {
@@ -336,8 +341,7 @@ struct GonArgs {
     // 0 while the streaming kernels run, else the step at which it took over
     // (streaming launches then return at once); nullptr: never
     int *route;
-    int skip_units;          // skip kernel: units of 32 points a CTA has room for
-    float skip_g2, skip_f;   // its slack factors for this d (kc_gonskip.cu)
+    GonSkip skip;
 };
 cudaError_t launch_gon(GonArgs &a, cudaStream_t s);
 // Single large float instances with row-major rows in device memory: the
@@ -352,8 +356,7 @@ int64_t skip_route_words();          // the route word, the probe's counter and 
 int64_t skip_slot_rows();            // slot rows behind the k exchange rows
 bool gon_skip_possible(int dtype, int d, int64_t n, int k, int grid);   // for n points at most
 int gon_skip_segments(int dtype, int d, int64_t n, int k, int grid, int *ends, int cap);
-cudaError_t launch_gon_probe(const GonInst &I, int it0, bool last, int *route, unsigned *words, DevStatus *st,
-                             cudaStream_t s);
+cudaError_t launch_gon_probe(const GonArgs &a, int it0, bool last, unsigned *words, cudaStream_t s);
 cudaError_t launch_gon_skip(GonArgs &a, int last, cudaStream_t s);
 // Resident form for one instance of n points (row-major rows in device
 // memory): the grid (0 when the instance does not fit on chip or d has no
@@ -406,11 +409,6 @@ inline void gon_single(GonArgs &g, const void *pk, int dtype, int64_t n, int d, 
     I.ecmax_out = nullptr;
     I.m32 = nullptr;
     I.stamp = nullptr;
-    I.asg = nullptr;
-    I.rmap = nullptr;
-    I.skip_perm[0] = I.skip_perm[1] = I.skip_mind[0] = I.skip_mind[1] = nullptr;
-    I.skip_asg = nullptr;
-    I.skip_hist = nullptr;
     I.it0 = I.it1 = 0;
     I.lp_kind = 0;
     I.kcap = k;
