@@ -171,6 +171,7 @@ template <typename T, int DC, int NT, bool DYN = false, bool LEAD = false, int U
 __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, DevStatus *st,
                           long long timeout, int withhold = 0, bool bad_index = false) {
     constexpr int W = NT / 32;
+    constexpr int BATCH = NT != GROUP_NT ? 0 : DC < 0 ? 3 : DYN ? 2 : 1;   // the generic loop's form (dist4)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int d = DC > 0 ? DC : I.d;
     const T *pk = (const T *)I.pk;
@@ -193,14 +194,19 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
     const bool claim = DYN && NT == GROUP_NT && (I.lo + I.n - 1) / BLK - I.lo / BLK + 1 >= 4 * (int64_t)G * W;
     const bool tail = DYN && G > 1 && I.tail != nullptr;
     constexpr bool lead = LEAD;   // gon_lead
+    // the last step's number: in a register in the 1024-thread kernels (68,891 x 16
+    // 4.1 us a step, read from shared memory 4.2), from shared memory in the others
+    // (a batch of int32 1791 x 64 3.3 ms with it in a register, so 2.6)
+    const int it1 = I.it1;
+    auto end = [&] { return NT == GROUP_NT ? it1 : I.it1; };
     int it;
     uint64_t K = 0;
-    for (it = I.it0; it < I.it1; ++it) {
+    for (it = I.it0; it < end(); ++it) {
         // claimed blocks in the 1024-thread group CTAs when every warp has
         // several (measured: GON on 8M x 64, k = 1024, 313 -> 308 ms); the
         // fixed assignment in the 256-thread queue CTAs (MRG round 1 on
         // 10M x 16 was 5% slower with claims) and for small instances
-        uint64_t best = sweep<T, DC, NT, UNR, NT == GROUP_NT ? (DYN ? 2 : 1) : 0>(pk, I.mind, I.lo, I.n, d, cs, it == 0, r, G,
+        uint64_t best = sweep<T, DC, NT, UNR, BATCH>(pk, I.mind, I.lo, I.n, d, cs, it == 0, r, G,
                                          claim ? &sh.ctr[it & 1] : nullptr, tail ? I.tail + it : nullptr);
         best = warp_max_u64(best);
         if (lane == 0) sh.red[warp] = best;
@@ -211,7 +217,7 @@ __device__ void gon_solve(const GonInst &I, int r, int G, T *cs, Shared &sh, Dev
             v = warp_max_u64(v);
             uint64_t g = v;
             bool ab = false;
-            const bool more = it + 1 < I.it1;
+            const bool more = it + 1 < end();
             const uint64_t tagw = (uint64_t)(it + 1) << 32;
             if (G > 1) {
                 uint64_t *row = I.slots + (int64_t)it * slot_stride(G);
@@ -1330,7 +1336,10 @@ template <bool DYN, bool LEAD> void *pick_group_f32(int dc) {
         case 10: return group_fn<float, 10, DYN, LEAD>();
         case 16: return group_fn<float, 16, DYN, LEAD>();
         case 32: return group_fn<float, 32, DYN, LEAD>();
-        default: return group_fn<float, 0, DYN, LEAD>();
+        default:   // -1: the generic loop for few coordinates
+            if constexpr (!DYN)
+                if (dc < 12) return group_fn<float, -1, DYN, LEAD>();
+            return group_fn<float, 0, DYN, LEAD>();
     }
 }
 template <bool LEAD> void *pick_group_i32(int dc) {

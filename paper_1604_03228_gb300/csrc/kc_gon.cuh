@@ -27,16 +27,18 @@ __device__ __forceinline__ void st_relaxed_u64(uint64_t *p, uint64_t v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// UNR: coordinates in flight in the generic loop (DC = 0).  BATCH: their loads
-// written out ahead of the terms, with one more batch for the remainder (1) or a
-// load at a time (2), or (0) left to the compiler.  In the 1024-thread kernels it
-// mixed loads and terms of a plain unrolled loop differently from build to build
-// (us a step: 800k x 256 on 98 CTAs 147 or 160, written out 129; 1.5M x 24 30.5
-// or 32, 27.8; 4M x 40 111, 98), and the loop written out beats the full unrolling
+// UNR: coordinates in flight in the generic loop (DC <= 0).  BATCH, its form: the
+// loads written out ahead of the terms, with one more batch for the remainder
+// (1) or a load at a time (2); groups of UNR, then by fours (0); a plain unrolled
+// loop (3).  In the 1024-thread kernels the compiler mixed loads and terms of
+// the plain loop differently from build to build (us a step: 800k x 256 on 98
+// CTAs 147 or 160, written out 129; 1.5M x 24 30.5 or 32, 27.8; 4M x 40 111, 98;
+// int32 2M x 64 87 to 100, 88), and the loop written out beats the full unrolling
 // of d = 64 too (1.5M x 64 70.2 / 65.2, 8M x 64 309 / 297).  The remainder as a
 // batch made the claimed-block instantiation a third slower (5M x 37 128 -> 173,
-// one by one 116).  In the 256-thread kernels the plain loop is the better one
-// (MRG on 2M x 64 18.4 ms, written out 22.2).
+// one by one 116), and below twelve coordinates on up to 64 CTAs the plain loop
+// is the better one (80k x 9 3.0 / 2.8).  In the 256-thread kernels the groups are
+// (MRG on 2M x 64 18.2 ms, written out 22.2).
 template <typename T, int DC, int UNR, int BATCH>
 __device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T *cs, int lane,
                                       typename AccOf<T>::type acc[4]) {
@@ -54,7 +56,7 @@ __device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T 
             a2 = sq_step(a2, v.z, c);
             a3 = sq_step(a3, v.w, c);
         }
-    } else if constexpr (BATCH != 0) {
+    } else if constexpr (BATCH == 1 || BATCH == 2) {
         int j = 0;
 #pragma unroll 1
         for (; j + UNR <= d; j += UNR) {
@@ -94,6 +96,16 @@ __device__ __forceinline__ void dist4(const T *__restrict__ blk, int d, const T 
                     a2 = sq_step(a2, v[t].z, c);
                     a3 = sq_step(a3, v[t].w, c);
                 }
+        }
+    } else if constexpr (BATCH == 3) {
+#pragma unroll UNR
+        for (int j = 0; j < d; ++j) {
+            const V4 v = __ldg(src + j * (BLK / 4));
+            const T c = cs[j];
+            a0 = sq_step(a0, v.x, c);
+            a1 = sq_step(a1, v.y, c);
+            a2 = sq_step(a2, v.z, c);
+            a3 = sq_step(a3, v.w, c);
         }
     } else {
         // whole groups of UNR coordinates, then by fours: a loop unrolled by eight
