@@ -1480,13 +1480,13 @@ int gon_resident_plan(int dtype, int d, int64_t n, int *cap, int *slot_words) {
 // other's polling, and the leader's second hop and the code it adds to the sweep
 // are what shows (not between queue CTAs either, which share their SM with other
 // groups: MRG round 1 on 10M x 16 20.2 -> 20.7 ms).  All polling / leader, us a
-// step, float: 200k x 2 (49 CTAs) 2.65 / 3.2, x 10 3.4 / 4.0, x 16 5.4 / 4.6; 600k x
-// 2 4.7 / 3.4, 1M x 10 7.2 / 5.7, 600k x 37 (89 MB) 11.3 / 8.8, 2.4M x 16 30.0 /
-// 28.4; beyond L2 1.5M x 64 68.6 / 72.4, 800k x 128 83 / 87; 200k x 100 14.6 / 15.3.
-// int32: 1.5M x 64 76 / 66, 1M x 100 74 / 66.
-static bool gon_lead(int dtype, int d, int64_t n, int G) {
+// step: 200k (49 CTAs) x 2 2.6 / 3.2, x 10 3.4 / 4.0, x 16 5.4 / 4.6; 600k x 2 4.4 /
+// 3.2, 1M x 10 7.3 / 5.0, 600k x 37 (89 MB) 10.8 / 9.1, 2.4M x 16 28.8 / 27.6, int32
+// 600k x 31 10.2 / 8.0; beyond L2 1.5M x 64 68.6 / 72.4, int32 66.6 / 68.3, 800k x
+// 128 83 / 87, int32 1M x 100 64.1 / 65.5; 200k x 100 14.6 / 15.3.
+static bool gon_lead(int d, int64_t n, int G) {
     if (G <= (d <= 10 ? 64 : LEADER_MIN) || nblocks(n) >= 4 * (int64_t)G * (GROUP_NT / 32)) return false;
-    return dtype == KC_I32 || d <= 16 || (d <= 64 && 4.0 * (double)n * d <= 100e6);
+    return d <= 16 || (d <= 64 && 4.0 * (double)n * d <= 100e6);
 }
 
 cudaError_t launch_gon(GonArgs &a, cudaStream_t s) {
@@ -1511,7 +1511,7 @@ cudaError_t launch_gon(GonArgs &a, cudaStream_t s) {
         return cudaLaunchKernelExC(&cfg, fn, args);
     }
     const size_t smem = smem_for(a.dtype, a.lp_kind, a.dmax, a.queue != 0);
-    const bool lead = !a.insts && !a.lp_kind && a.single.bc && gon_lead(a.dtype, a.dc, a.single.n, a.grid);
+    const bool lead = !a.insts && !a.lp_kind && a.single.bc && gon_lead(a.dc, a.single.n, a.grid);
     void *fn = pick_fn(a.dtype, a.lp_kind, a.dc, a.queue != 0, a.dyn != 0, lead);
     if (const cudaError_t e = opt_in_smem(fn, smem)) return e;
     note_launches(1);
